@@ -303,8 +303,12 @@ template <class R> struct Coef {
     R ir_a;    // 1 / (1/2 + 3 nu_p)
     R ir_b;    // 1 / (1 + 6 nu_p)
     R six_nu;  // 6 nu_p
+    R s2y2;    // 2 sigma_y^2, the square of the IR yield threshold
+    R ir_as;   // s2y ir_a
+    R ir_bn;   // six_nu ir_b
+    R ir_bs;   // s2y ir_b
     int newton;  // PR: Newton iterations of the implicit tau update
-    R cg[13];   // c_i . g of direction i = 2p + 1 (PR force terms), per pair p
+    R cg[13];   // c_i . g of direction i = 2p + 1 (PR force terms of the class form), per pair p
     R cgg[13];  // (c_i . g)^2
 };
 
@@ -451,6 +455,21 @@ __device__ __forceinline__ void gather(const KParams& kp, const Src& P, uint32_t
 template <class R> struct Mom {
     R d, jx, jy, jz, xx, yy, zz, xy, xz, yz;
 };
+// symmetric second-order tensor
+template <class R> struct Tens {
+    R xx, yy, zz, xy, xz, yz;
+};
+
+// Which form of the collision a storage form runs.  Pair form (below): FP64,
+// whose step is bound by the FP64 pipe (D3Q27 IR, duct 1 x 64 x 64: 24.5 ->
+// 19.0 us a step; D2Q9 PR, 80 x 80: 15.6 -> 13.5), and the 16-bit forms, whose
+// step is bound by instruction issue (D3Q27 PR FP16: 703 -> 607 instructions a
+// warp; BF16 IR, duct 256 x 128 x 128: 96.1 -> 90.7 us; D3Q19 PR FP16, compact
+// porous 256^3: 326 -> 311).  Errors against FP64 did not grow.  FP32 storage
+// keeps the class sums, which are bit for bit the results it has always had:
+// the pair form gained it 0.4-3 % (its large steps are bound by HBM), and near
+// a steady state the residual shows any change of rounding.
+template <class S> __host__ __device__ constexpr bool pair_form() { return sizeof(S) != 4; }
 
 // Grouped sums: populations are added once per velocity class (c_x = +1, -1,
 // 0; c_y = +-1; c_z = +-1; sign of c_x c_y, c_x c_z, c_y c_z) and the moments
@@ -474,8 +493,8 @@ template <class L> __host__ __device__ constexpr int first_in_class(int k) {
     return -1;
 }
 
-template <class L, class S, class R = typename Store<S>::R>
-__device__ __forceinline__ Mom<R> moments(const R (&f)[L::Q]) {
+template <class L, class S, class R>
+__device__ __forceinline__ Mom<R> class_moments(const R (&f)[L::Q]) {
     R acc[kNumClasses];
     static_for<0, L::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -515,23 +534,179 @@ __device__ __forceinline__ Mom<R> moments(const R (&f)[L::Q]) {
     return m;
 }
 
-// Non-equilibrium second moment T = Pi - rho c_s^2 I - rho u u written with
-// offsets: Pi = c_s^2 I + p, rho = 1 + d.
-template <class R> struct Tens {
-    R xx, yy, zz, xy, xz, yz;
+// Direction families.  In the pair order of lattice.cuh the axis pairs come
+// first, then the face diagonals (xy+, xy-, xz+, xz-, yz+, yz-), then the
+// corners (+++), (++-), (+-+), (-++); first() is the index i of a family's
+// first member, 0 where the lattice has none.  All members of a family share
+// their weight.
+template <class L> struct Fam {
+    static constexpr int axis = 1;
+    static constexpr int face = L::Q == 9 ? 5 : L::Q == 15 ? 0 : 7;
+    static constexpr int corner = L::Q == 15 ? 7 : L::Q == 27 ? 19 : 0;
 };
+template <class L> constexpr bool fam_order() {
+    auto is = [](int i, int x, int y, int z) { return L::cx(i) == x && L::cy(i) == y && L::cz(i) == z; };
+    bool ok = is(1, 1, 0, 0) && is(3, 0, 1, 0) && (L::D == 2 || is(5, 0, 0, 1));
+    constexpr int f = Fam<L>::face, c = Fam<L>::corner;
+    if (f) ok = ok && is(f, 1, 1, 0) && is(f + 2, 1, -1, 0);
+    if (f && L::D == 3)
+        ok = ok && is(f + 4, 1, 0, 1) && is(f + 6, 1, 0, -1) && is(f + 8, 0, 1, 1) && is(f + 10, 0, 1, -1);
+    if (c) ok = ok && is(c, 1, 1, 1) && is(c + 2, 1, 1, -1) && is(c + 4, 1, -1, 1) && is(c + 6, -1, 1, 1);
+    return ok;
+}
+static_assert(fam_order<D2Q9>() && fam_order<D3Q15>() && fam_order<D3Q19>() && fam_order<D3Q27>(),
+              "direction families");
 
+// b x and y + b x for a compile-time factor b (a plain x, y + x where it is 1)
+template <class R, class B> __device__ __forceinline__ R scale(B b, R x) {
+    if (b == B(1)) return x;
+    return x * R(b);
+}
+template <class R, class B> __device__ __forceinline__ R axpy(B b, R x, R y) {
+    if (b == B(1)) return y + x;
+    return y + x * R(b);
+}
+
+// Pair form: f[i] = f_i + f_o and f[o] = f_i - f_o for every opposite pair
+// (i, o = i + 1).  Even moments need the sums only, odd ones the differences
+// only, and so do the two halves of the TRT collision.
+template <class L, class R> __device__ __forceinline__ void to_pairs(R (&f)[L::Q]) {
+    static_for<0, (L::Q - 1) / 2>([&](auto P) {
+        constexpr int i = 2 * decltype(P)::value + 1;
+        const R a = f[i], b = f[i + 1];
+        f[i] = a + b;
+        f[i + 1] = a - b;
+    });
+}
+
+// Moments from the pair form.  Per family the members are first combined by
+// sums and differences (xx + yy against xy of a face plane; the four corners
+// by one 4-point butterfly), then scaled once by the family's beta (memory
+// units to offsets) and added to the axis terms.  On D3Q27 this takes 82 adds
+// where adding every population to its velocity classes took 96, and 26 of
+// them are the pair sums that the TRT collision needs anyway; in the 16-bit
+// forms the classes' 96 multiply-adds by beta become 20.
+template <class L, class S, class R>
+__device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
+    constexpr int F = Fam<L>::face, C = Fam<L>::corner;
+    constexpr auto b0 = Store<S>::template beta<L, 0>();
+    constexpr auto bA = Store<S>::template beta<L, 1>();
+    constexpr auto bF = Store<S>::template beta<L, (F ? F : 1)>();
+    constexpr auto bC = Store<S>::template beta<L, (C ? C : 1)>();
+    Mom<R> m;
+    if constexpr (L::D == 2) {
+        const R XY = scale(bF, R(f[F] + f[F + 2]));
+        m.xx = axpy(bA, f[1], XY);
+        m.yy = axpy(bA, f[3], XY);
+        m.d = m.xx + axpy(b0, f[0], scale(bA, f[3]));
+        m.xy = scale(bF, R(f[F] - f[F + 2]));
+        m.jx = axpy(bA, f[2], scale(bF, R(f[F + 1] + f[F + 3])));
+        m.jy = axpy(bA, f[4], scale(bF, R(f[F + 1] - f[F + 3])));
+        m.zz = R(0);
+        m.jz = R(0);
+        m.xz = R(0);
+        m.yz = R(0);
+    } else {
+        R X, Y, Z, rest = scale(bA, R(f[3] + f[5]));   // X: diagonal sums beyond the axis pairs
+        R jx, jy, jz;
+        if constexpr (C != 0) {
+            const R ab = f[C] + f[C + 2], amb = f[C] - f[C + 2];
+            const R ce = f[C + 4] + f[C + 6], cme = f[C + 4] - f[C + 6];
+            X = scale(bC, R(ab + ce));
+            m.xy = scale(bC, R(ab - ce));
+            m.xz = scale(bC, R(amb + cme));
+            m.yz = scale(bC, R(amb - cme));
+            const R dp = f[C + 1] + f[C + 3], dq = f[C + 5] - f[C + 7];
+            jx = scale(bC, R(dp + dq));
+            jy = scale(bC, R(dp - dq));
+            jz = scale(bC, R((f[C + 1] - f[C + 3]) + (f[C + 5] + f[C + 7])));
+            Y = X;
+            Z = X;
+        }
+        if constexpr (F != 0) {
+            const R sxy = f[F] + f[F + 2], sxz = f[F + 4] + f[F + 6], syz = f[F + 8] + f[F + 10];
+            const R oxy = f[F] - f[F + 2], oxz = f[F + 4] - f[F + 6], oyz = f[F + 8] - f[F + 10];
+            const R fx = (f[F + 1] + f[F + 3]) + (f[F + 5] + f[F + 7]);
+            const R fy = (f[F + 1] - f[F + 3]) + (f[F + 9] + f[F + 11]);
+            const R fz = (f[F + 5] - f[F + 7]) + (f[F + 9] - f[F + 11]);
+            const R xs = sxy + sxz, ys = sxy + syz, zs = sxz + syz;
+            rest = axpy(bF, syz, rest);
+            if constexpr (C != 0) {
+                X = axpy(bF, xs, X);
+                Y = axpy(bF, ys, Y);
+                Z = axpy(bF, zs, Z);
+                m.xy = axpy(bF, oxy, m.xy);
+                m.xz = axpy(bF, oxz, m.xz);
+                m.yz = axpy(bF, oyz, m.yz);
+                jx = axpy(bF, fx, jx);
+                jy = axpy(bF, fy, jy);
+                jz = axpy(bF, fz, jz);
+            } else {
+                X = scale(bF, xs);
+                Y = scale(bF, ys);
+                Z = scale(bF, zs);
+                m.xy = scale(bF, oxy);
+                m.xz = scale(bF, oxz);
+                m.yz = scale(bF, oyz);
+                jx = scale(bF, fx);
+                jy = scale(bF, fy);
+                jz = scale(bF, fz);
+            }
+        }
+        m.xx = axpy(bA, f[1], X);
+        m.yy = axpy(bA, f[3], Y);
+        m.zz = axpy(bA, f[5], Z);
+        m.d = m.xx + axpy(b0, f[0], rest);
+        m.jx = axpy(bA, f[2], jx);
+        m.jy = axpy(bA, f[4], jy);
+        m.jz = axpy(bA, f[6], jz);
+    }
+    return m;
+}
+
+// moments of populations in memory units (f may be overwritten)
+template <class L, class S, class R = typename Store<S>::R>
+__device__ __forceinline__ Mom<R> moments(R (&f)[L::Q]) {
+    if constexpr (pair_form<S>()) {
+        to_pairs<L>(f);
+        return pair_moments<L, S, R>(f);
+    } else {
+        return class_moments<L, S, R>(f);
+    }
+}
+
+// a_i b_j of two parallel vectors (symmetric)
 template <class L, class R>
-__device__ __forceinline__ Tens<R> noneq(const Mom<R>& m, R rho, R ux, R uy, R uz, uint32_t flags) {
+__device__ __forceinline__ Tens<R> outer(R ax, R ay, R az, R bx, R by, R bz) {
+    Tens<R> t;
+    t.xx = ax * bx;
+    t.yy = ay * by;
+    t.xy = ax * by;
+    if constexpr (L::D == 3) {
+        t.zz = az * bz;
+        t.xz = ax * bz;
+        t.yz = ay * bz;
+    } else {
+        t.zz = R(0);
+        t.xz = R(0);
+        t.yz = R(0);
+    }
+    return t;
+}
+
+// Non-equilibrium second moment T = Pi - rho c_s^2 I - rho u u written with
+// offsets: Pi = c_s^2 I + p, rho = 1 + d.  ruu = rho u u.
+template <class L, class R>
+__device__ __forceinline__ Tens<R> noneq(const Mom<R>& m, const Tens<R>& ruu, uint32_t flags) {
     const R d3 = m.d * R(1.0 / 3.0);
     Tens<R> t;
-    t.xx = m.xx - d3 - rho * ux * ux;
-    t.yy = m.yy - d3 - rho * uy * uy;
-    t.xy = m.xy - rho * ux * uy;
+    t.xx = m.xx - d3 - ruu.xx;
+    t.yy = m.yy - d3 - ruu.yy;
+    t.xy = m.xy - ruu.xy;
     if constexpr (L::D == 3) {
-        t.zz = m.zz - d3 - rho * uz * uz;
-        t.xz = m.xz - rho * ux * uz;
-        t.yz = m.yz - rho * uy * uz;
+        t.zz = m.zz - d3 - ruu.zz;
+        t.xz = m.xz - ruu.xz;
+        t.yz = m.yz - ruu.yz;
     } else {
         t.zz = R(0);
         t.xz = R(0);
@@ -547,16 +722,81 @@ template <class L, class R> __device__ __forceinline__ R tnorm2(const Tens<R>& T
     return s;
 }
 
-// c.T.c for a lattice velocity, from T and the doubled off-diagonals
-template <int cx, int cy, int cz, class R>
-__device__ __forceinline__ R ctc(const Tens<R>& T, R t2xy, R t2xz, R t2yz) {
-    return cdot6<cx * cx, cy * cy, cz * cz, cx * cy, cx * cz, cy * cz>(T.xx, T.yy, T.zz, t2xy,
-                                                                        t2xz, t2yz);
+template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t) {
+    if constexpr (L::D == 3) return t.xx + t.yy + t.zz;
+    return t.xx + t.yy;
+}
+
+// The post-collision populations of both models have the form
+//   f_i = [kept part] + w_i (e0 + 9/2 c.N.c) + 3 w_i c.q
+// (memory units).  The even bracket takes six numbers per cell, and the
+// members of a family differ only by the signs of the off-diagonal terms: one
+// sum per axis pair, two per face plane, one 4-point butterfly for the
+// corners, instead of c.u, its square and c.T.c per pair (D3Q27: 23 adds
+// against 150 operations).  put(i, even, odd) stores pair i: even and odd
+// carry their weights.  Where w_i in memory units is the same for every
+// direction (the 16-bit forms) it goes into the six numbers and q once.
+template <class L, class S, class R, class Put>
+__device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R qz, Put&& put) {
+    constexpr int F = Fam<L>::face, C = Fam<L>::corner;
+    constexpr bool same = sizeof(S) == 2;   // gam, god do not depend on the direction
+    constexpr auto g0 = Store<S>::template gam<L, 1>();
+    constexpr auto o0 = Store<S>::template god<L, 1>();
+    if constexpr (same) {
+        e0 = scale(g0, e0);
+        qx = scale(o0, qx);
+        qy = scale(o0, qy);
+        if constexpr (L::D == 3) qz = scale(o0, qz);
+    }
+    const R k = R(same ? decltype(g0)(4.5) * g0 : decltype(g0)(4.5));
+    const R k2 = R(same ? decltype(g0)(9) * g0 : decltype(g0)(9));
+    auto pair = [&](auto I, R e, R cq) {
+        constexpr int i = decltype(I)::value;
+        if constexpr (same)
+            put(I, e, cq);
+        else
+            put(I, R(e * R(Store<S>::template gam<L, i>())), R(cq * R(Store<S>::template god<L, i>())));
+    };
+#define BLBM_I(n) std::integral_constant<int, (n)>{}
+    const R ex = e0 + k * N.xx;
+    pair(BLBM_I(1), ex, qx);
+    const R ay = k * N.yy;
+    pair(BLBM_I(3), R(e0 + ay), qy);
+    const R exy = ex + ay;
+    const R bxy = k2 * N.xy;
+    const R qxpy = qx + qy, qxmy = qx - qy;
+    if constexpr (L::D == 2) {
+        pair(BLBM_I(F), R(exy + bxy), qxpy);
+        pair(BLBM_I(F + 2), R(exy - bxy), qxmy);
+    } else {
+        const R az = k * N.zz;
+        const R bxz = k2 * N.xz, byz = k2 * N.yz;
+        pair(BLBM_I(5), R(e0 + az), qz);
+        if constexpr (F != 0) {
+            pair(BLBM_I(F), R(exy + bxy), qxpy);
+            pair(BLBM_I(F + 2), R(exy - bxy), qxmy);
+            const R exz = ex + az, eyz = e0 + ay + az;
+            pair(BLBM_I(F + 4), R(exz + bxz), R(qx + qz));
+            pair(BLBM_I(F + 6), R(exz - bxz), R(qx - qz));
+            pair(BLBM_I(F + 8), R(eyz + byz), R(qy + qz));
+            pair(BLBM_I(F + 10), R(eyz - byz), R(qy - qz));
+        }
+        if constexpr (C != 0) {
+            const R e = exy + az;
+            const R ep = e + byz, em = e - byz, bp = bxy + bxz, bm = bxy - bxz;
+            pair(BLBM_I(C), R(ep + bp), R(qxpy + qz));
+            pair(BLBM_I(C + 2), R(em + bm), R(qxpy - qz));
+            pair(BLBM_I(C + 4), R(em - bm), R(qxmy + qz));
+            pair(BLBM_I(C + 6), R(ep - bp), R(qz - qxmy));
+        }
+    }
+#undef BLBM_I
 }
 
 // ---------------------------------------------------------------------------
 // IR yield solve, per cell: s = as T, sigma = asg T (eq. Vikh_sigmaS_tensor)
-// from |T|^2.
+// from |T|^2.  Both factors are linear in 1 / |T|: -(|T| - sqrt2 sigma_y) a / |T|
+// = sqrt2 sigma_y a / |T| - a, so one reciprocal square root is all it takes.
 template <class R>
 __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R tn2, R& as_out,
                                          R& asg_out) {
@@ -564,13 +804,13 @@ __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R
     Sc as[Lanes<R>::n], asg[Lanes<R>::n];
 #pragma unroll
     for (int k = 0; k < Lanes<R>::n; ++k) {
-        const Sc tn = sqrt(Lanes<R>::get(tn2, k));
+        const Sc t2 = Lanes<R>::get(tn2, k);
         as[k] = Sc(0);
         asg[k] = Sc(-1);
-        if (tn > Sc(0) && tn >= c.s2y) {
-            const Sc it = Sc(1) / tn;
-            as[k] = -(tn - c.s2y) * c.ir_a * it;
-            asg[k] = -(c.six_nu * tn + c.s2y) * c.ir_b * it;
+        if (t2 > Sc(0) && t2 >= c.s2y2) {
+            const Sc it = rsqrt(t2);
+            as[k] = c.ir_as * it - c.ir_a;
+            asg[k] = -(c.ir_bs * it + c.ir_bn);
         }
     }
     as_out = Lanes<R>::make(as);
@@ -580,8 +820,8 @@ __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R
 // ---------------------------------------------------------------------------
 // IR collision (Secs. 2.3, 3.2).  f: memory units in, memory units out.  R is
 // the arithmetic type: one cell (float, double) or two cells (F2).
-template <class L, class S, class R = typename Store<S>::R>
-__device__ __forceinline__ void collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+template <class L, class S, class R>
+__device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
                                            R (&f)[L::Q], R& drho, R (&ur)[3]) {
     const Mom<R> m = moments<L, S, R>(f);
     const R rho = R(1) + m.d;
@@ -589,42 +829,40 @@ __device__ __forceinline__ void collide_ir(const Coef<typename Lanes<R>::Sc>& c,
     const R Fx = rho * R(c.g[0]), Fy = rho * R(c.g[1]);
     R Fz = R(0);
     if constexpr (L::D == 3) Fz = rho * R(c.g[2]);
-    const R ux = (m.jx + R(0.5) * Fx) * inv;
-    const R uy = (m.jy + R(0.5) * Fy) * inv;
+    const R px = m.jx + R(0.5) * Fx, py = m.jy + R(0.5) * Fy;   // rho u
+    R pz = R(0);
+    if constexpr (L::D == 3) pz = m.jz + R(0.5) * Fz;
+    const R ux = px * inv, uy = py * inv;
     R uz = R(0);
-    if constexpr (L::D == 3) uz = (m.jz + R(0.5) * Fz) * inv;
-    const Tens<R> T = noneq<L, R>(m, rho, ux, uy, uz, flags);
+    if constexpr (L::D == 3) uz = pz * inv;
+    const Tens<R> U = outer<L, R>(px, py, pz, ux, uy, uz);
+    const Tens<R> T = noneq<L, R>(m, U, flags);
     R as, asg;
     ir_yield<R>(c, tnorm2<L, R>(T), as, asg);
-    // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I
-    const R trT = T.xx + T.yy + T.zz;
+    // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I;
+    // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i
     const R k1 = R(0.5) * as - asg;
-    const R k2 = asg * trT * R(1.0 / L::D);
-    // (c c - c_s^2 I):A = k1 (cTc - trT/3) + k2 (|c|^2 - D/3) = h0 + k1 cTc + k2 |c|^2
-    const R h0 = -(k1 * trT + k2 * R(L::D)) * R(1.0 / 3.0);
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R base = m.d - R(1.5) * rho * uu;
-    const R r45 = R(4.5) * rho;
-    const R k145 = R(4.5) * k1;
-    const R t2xy = R(2) * T.xy, t2xz = R(2) * T.xz, t2yz = R(2) * T.yz;
+    const R k2 = asg * trace<L, R>(T) * R(1.0 / L::D);
+    Tens<R> N;
+    N.xx = U.xx + (k1 * T.xx + k2);
+    N.yy = U.yy + (k1 * T.yy + k2);
+    N.xy = U.xy + k1 * T.xy;
+    N.zz = R(0);
+    N.xz = R(0);
+    N.yz = R(0);
+    if constexpr (L::D == 3) {
+        N.zz = U.zz + (k1 * T.zz + k2);
+        N.xz = U.xz + k1 * T.xz;
+        N.yz = U.yz + k1 * T.yz;
+    }
+    const R e0 = m.d - R(1.5) * trace<L, R>(N);
     // odd part: w_i (3 rho c.u + 3/2 c.F) = 3 w_i c.(j + F), since rho u = j + F/2
     const R qx = m.jx + Fx, qy = m.jy + Fy, qz = m.jz + Fz;
-    f[0] = R(Store<S>::template gam<L, 0>()) * (base + R(4.5) * h0);
-    static_for<0, (L::Q - 1) / 2>([&](auto P) {
-        constexpr int i = 2 * decltype(P)::value + 1;
-        constexpr int o = i + 1;
-        constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-        constexpr int c2 = cx * cx + cy * cy + cz * cz;
-        const R w = R(Store<S>::template gam<L, i>());   // w_i in memory units
-        // even part e = w (base + 4.5 rho cu^2 + 4.5 h) = A + B cu^2 + C cTc (per class A, B, C)
-        const R A = w * (base + R(4.5) * (h0 + k2 * R(c2)));
-        const R B = w * r45;
-        const R C = w * k145;
-        const R cu = cdot<cx, cy, cz>(ux, uy, uz);
-        const R e = A + B * (cu * cu) + C * ctc<cx, cy, cz>(T, t2xy, t2xz, t2yz);
-        const R od = R(Store<S>::template god<L, i>()) * cdot<cx, cy, cz>(qx, qy, qz);
+    f[0] = R(Store<S>::template gam<L, 0>()) * e0;
+    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, R od) {
+        constexpr int i = decltype(I)::value;
         f[i] = e + od;
-        f[o] = e - od;
+        f[i + 1] = e - od;
     });
     drho = m.d;
     ur[0] = ux;
@@ -701,8 +939,8 @@ __device__ __forceinline__ void pr_rates(const Coef<typename Lanes<R>::Sc>& c, R
 // PR collision (Sec. 3.1 + TRT + EDM).  tau: previous step's relaxation time
 // in, this step's out.  f: memory units in, memory units out (the TRT update is
 // linear and opposite populations share their unit).  R as for collide_ir.
-template <class L, class S, bool IMPLICIT, class R = typename Store<S>::R>
-__device__ __forceinline__ void collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+template <class L, class S, bool IMPLICIT, class R>
+__device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
                                            R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
     const Mom<R> m = moments<L, S, R>(f);
     const R rho = R(1) + m.d;
@@ -710,7 +948,170 @@ __device__ __forceinline__ void collide_pr(const Coef<typename Lanes<R>::Sc>& c,
     const R ux = m.jx * inv, uy = m.jy * inv;
     R uz = R(0);
     if constexpr (L::D == 3) uz = m.jz * inv;
-    const Tens<R> T = noneq<L, R>(m, rho, ux, uy, uz, flags);
+    R wp, wm;
+    {
+        const Tens<R> T = noneq<L, R>(m, outer<L, R>(m.jx, m.jy, m.jz, ux, uy, uz), flags);
+        pr_rates<IMPLICIT, R>(c, tnorm2<L, R>(T), inv, tau, wp, wm);
+    }
+    const R gx = R(c.g[0]), gy = R(c.g[1]);
+    R gz = R(0);
+    if constexpr (L::D == 3) gz = R(c.g[2]);
+    const R Fx = rho * gx, Fy = rho * gy, Fz = rho * gz;
+    // Per pair (i, o = opposite), with f^+- = (f_i +- f_o) / 2:
+    //   E = f^+ - wp (f^+ - f_eq^+) + F^+ = (1 - wp)/2 (f_i + f_o) + w_i (K0 + 9/2 c.N.c),
+    //       N = rho (wp u u + u g + g u + g g) = j (wp u + g) + F (u + g),
+    //       K0 = wp d - 3/2 tr N;
+    //   O = f^- - wm (f^- - f_eq^-) + F^- = (1 - wm)/2 (f_i - f_o) + 3 w_i c.(wm j + F),
+    // the odd equilibrium and force parts from j and F directly (3 w_i rho c.u
+    // = 3 w_i c.j exactly).  f holds the pair sums and differences.
+    Tens<R> N;
+    {
+        const R vx = wp * ux + gx, vy = wp * uy + gy, zx = ux + gx, zy = uy + gy;
+        N.xx = m.jx * vx + Fx * zx;
+        N.yy = m.jy * vy + Fy * zy;
+        N.xy = m.jx * vy + Fx * zy;
+        N.zz = R(0);
+        N.xz = R(0);
+        N.yz = R(0);
+        if constexpr (L::D == 3) {
+            const R vz = wp * uz + gz, zz = uz + gz;
+            N.zz = m.jz * vz + Fz * zz;
+            N.xz = m.jx * vz + Fx * zz;
+            N.yz = m.jy * vz + Fy * zz;
+        }
+    }
+    const R omp = R(0.5) - R(0.5) * wp;
+    const R omm = R(0.5) - R(0.5) * wm;
+    const R K0 = wp * m.d - R(1.5) * trace<L, R>(N);
+    const R qx = wm * m.jx + Fx, qy = wm * m.jy + Fy, qz = wm * m.jz + Fz;
+    {
+        const R w0 = R(Store<S>::template gam<L, 0>());
+        f[0] = (R(1) - wp) * f[0] + w0 * K0;
+    }
+    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, R od) {
+        constexpr int i = decltype(I)::value;
+        const R E = omp * f[i] + e;
+        const R O = omm * f[i + 1] + od;
+        f[i] = E + O;
+        f[i + 1] = E - O;
+    });
+    drho = m.d;
+    ur[0] = ux + R(0.5) * gx;
+    ur[1] = uy + R(0.5) * gy;
+    ur[2] = uz + R(0.5) * gz;
+}
+
+// ---------------------------------------------------------------------------
+// The same two collisions on class sums, for FP32 storage (see pair_form).
+template <class L, class R>
+__device__ __forceinline__ Tens<R> class_noneq(const Mom<R>& m, R rho, R ux, R uy, R uz, uint32_t flags) {
+    const R d3 = m.d * R(1.0 / 3.0);
+    Tens<R> t;
+    t.xx = m.xx - d3 - rho * ux * ux;
+    t.yy = m.yy - d3 - rho * uy * uy;
+    t.xy = m.xy - rho * ux * uy;
+    if constexpr (L::D == 3) {
+        t.zz = m.zz - d3 - rho * uz * uz;
+        t.xz = m.xz - rho * ux * uz;
+        t.yz = m.yz - rho * uy * uz;
+    } else {
+        t.zz = R(0);
+        t.xz = R(0);
+        t.yz = R(0);
+    }
+    if (flags & LBM_FLAG_BURNETT_X) t.xx = R(0);
+    return t;
+}
+
+// c.T.c for a lattice velocity, from T and the doubled off-diagonals
+template <int cx, int cy, int cz, class R>
+__device__ __forceinline__ R ctc(const Tens<R>& T, R t2xy, R t2xz, R t2yz) {
+    return cdot6<cx * cx, cy * cy, cz * cz, cx * cy, cx * cz, cy * cz>(T.xx, T.yy, T.zz, t2xy,
+                                                                        t2xz, t2yz);
+}
+
+template <class R>
+__device__ __forceinline__ void class_ir_yield(const Coef<typename Lanes<R>::Sc>& c, R tn2, R& as_out,
+                                         R& asg_out) {
+    using Sc = typename Lanes<R>::Sc;
+    Sc as[Lanes<R>::n], asg[Lanes<R>::n];
+#pragma unroll
+    for (int k = 0; k < Lanes<R>::n; ++k) {
+        const Sc tn = sqrt(Lanes<R>::get(tn2, k));
+        as[k] = Sc(0);
+        asg[k] = Sc(-1);
+        if (tn > Sc(0) && tn >= c.s2y) {
+            const Sc it = Sc(1) / tn;
+            as[k] = -(tn - c.s2y) * c.ir_a * it;
+            asg[k] = -(c.six_nu * tn + c.s2y) * c.ir_b * it;
+        }
+    }
+    as_out = Lanes<R>::make(as);
+    asg_out = Lanes<R>::make(asg);
+}
+
+template <class L, class S, class R>
+__device__ __forceinline__ void class_collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                           R (&f)[L::Q], R& drho, R (&ur)[3]) {
+    const Mom<R> m = class_moments<L, S, R>(f);
+    const R rho = R(1) + m.d;
+    const R inv = recip(rho);
+    const R Fx = rho * R(c.g[0]), Fy = rho * R(c.g[1]);
+    R Fz = R(0);
+    if constexpr (L::D == 3) Fz = rho * R(c.g[2]);
+    const R ux = (m.jx + R(0.5) * Fx) * inv;
+    const R uy = (m.jy + R(0.5) * Fy) * inv;
+    R uz = R(0);
+    if constexpr (L::D == 3) uz = (m.jz + R(0.5) * Fz) * inv;
+    const Tens<R> T = class_noneq<L, R>(m, rho, ux, uy, uz, flags);
+    R as, asg;
+    class_ir_yield<R>(c, tnorm2<L, R>(T), as, asg);
+    // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I
+    const R trT = T.xx + T.yy + T.zz;
+    const R k1 = R(0.5) * as - asg;
+    const R k2 = asg * trT * R(1.0 / L::D);
+    // (c c - c_s^2 I):A = k1 (cTc - trT/3) + k2 (|c|^2 - D/3) = h0 + k1 cTc + k2 |c|^2
+    const R h0 = -(k1 * trT + k2 * R(L::D)) * R(1.0 / 3.0);
+    const R uu = ux * ux + uy * uy + uz * uz;
+    const R base = m.d - R(1.5) * rho * uu;
+    const R r45 = R(4.5) * rho;
+    const R k145 = R(4.5) * k1;
+    const R t2xy = R(2) * T.xy, t2xz = R(2) * T.xz, t2yz = R(2) * T.yz;
+    // odd part: w_i (3 rho c.u + 3/2 c.F) = 3 w_i c.(j + F), since rho u = j + F/2
+    const R qx = m.jx + Fx, qy = m.jy + Fy, qz = m.jz + Fz;
+    f[0] = R(Store<S>::template gam<L, 0>()) * (base + R(4.5) * h0);
+    static_for<0, (L::Q - 1) / 2>([&](auto P) {
+        constexpr int i = 2 * decltype(P)::value + 1;
+        constexpr int o = i + 1;
+        constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+        constexpr int c2 = cx * cx + cy * cy + cz * cz;
+        const R w = R(Store<S>::template gam<L, i>());   // w_i in memory units
+        // even part e = w (base + 4.5 rho cu^2 + 4.5 h) = A + B cu^2 + C cTc (per class A, B, C)
+        const R A = w * (base + R(4.5) * (h0 + k2 * R(c2)));
+        const R B = w * r45;
+        const R C = w * k145;
+        const R cu = cdot<cx, cy, cz>(ux, uy, uz);
+        const R e = A + B * (cu * cu) + C * ctc<cx, cy, cz>(T, t2xy, t2xz, t2yz);
+        const R od = R(Store<S>::template god<L, i>()) * cdot<cx, cy, cz>(qx, qy, qz);
+        f[i] = e + od;
+        f[o] = e - od;
+    });
+    drho = m.d;
+    ur[0] = ux;
+    ur[1] = uy;
+    ur[2] = uz;
+}
+
+template <class L, class S, bool IMPLICIT, class R>
+__device__ __forceinline__ void class_collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                           R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
+    const Mom<R> m = class_moments<L, S, R>(f);
+    const R rho = R(1) + m.d;
+    const R inv = recip(rho);
+    const R ux = m.jx * inv, uy = m.jy * inv;
+    R uz = R(0);
+    if constexpr (L::D == 3) uz = m.jz * inv;
+    const Tens<R> T = class_noneq<L, R>(m, rho, ux, uy, uz, flags);
     R wp, wm;
     pr_rates<IMPLICIT, R>(c, tnorm2<L, R>(T), inv, tau, wp, wm);
     const R gx = R(c.g[0]), gy = R(c.g[1]);
@@ -756,6 +1157,20 @@ __device__ __forceinline__ void collide_pr(const Coef<typename Lanes<R>::Sc>& c,
     ur[0] = ux + R(0.5) * gx;
     ur[1] = uy + R(0.5) * gy;
     ur[2] = uz + R(0.5) * gz;
+}
+
+template <class L, class S, class R = typename Store<S>::R>
+__device__ __forceinline__ void collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                           R (&f)[L::Q], R& drho, R (&ur)[3]) {
+    if constexpr (pair_form<S>()) pair_collide_ir<L, S, R>(c, flags, f, drho, ur);
+    else class_collide_ir<L, S, R>(c, flags, f, drho, ur);
+}
+
+template <class L, class S, bool IMPLICIT, class R = typename Store<S>::R>
+__device__ __forceinline__ void collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                           R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
+    if constexpr (pair_form<S>()) pair_collide_pr<L, S, IMPLICIT, R>(c, flags, f, tau, drho, ur);
+    else class_collide_pr<L, S, IMPLICIT, R>(c, flags, f, tau, drho, ur);
 }
 
 // ---------------------------------------------------------------------------
@@ -1428,7 +1843,7 @@ k_step_batch(const BatchDesc* __restrict__ descs, const int* __restrict__ tile_d
 
 // density and velocity u = (j + F/2) / rho of gathered populations
 template <class L, class S>
-__device__ __forceinline__ void fields_of(const KArgs& a, const typename Store<S>::R (&v)[L::Q],
+__device__ __forceinline__ void fields_of(const KArgs& a, typename Store<S>::R (&v)[L::Q],
                                           double& r, double (&u)[3]) {
     using R = typename Store<S>::R;
     const Mom<R> m = moments<L, S>(v);
@@ -1670,10 +2085,15 @@ template <class R> inline Coef<R> make_coef(const KParams& kp) {
     c.e_c = (R)(kp.m * kp.gdot_c > 0.0 ? -expm1(-kp.m * kp.gdot_c) / kp.gdot_c : 0.0);
     c.magic = (R)kp.magic;
     for (int d = 0; d < 3; ++d) c.g[d] = (R)kp.g[d];
-    c.s2y = (R)(1.4142135623730951 * kp.sigma_y);
+    const double s2y = 1.4142135623730951 * kp.sigma_y;
+    c.s2y = (R)s2y;
     c.ir_a = (R)(1.0 / (0.5 + 3.0 * nu));
     c.ir_b = (R)(1.0 / (1.0 + 6.0 * nu));
     c.six_nu = (R)(6.0 * nu);
+    c.s2y2 = (R)(2.0 * kp.sigma_y * kp.sigma_y);
+    c.ir_as = (R)(s2y / (0.5 + 3.0 * nu));
+    c.ir_bn = (R)(6.0 * nu / (1.0 + 6.0 * nu));
+    c.ir_bs = (R)(s2y / (1.0 + 6.0 * nu));
     c.newton = kp.newton;
     return c;
 }
