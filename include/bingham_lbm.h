@@ -350,7 +350,8 @@ void lbm_destroy(lbm_solver *s);
 /* ------------------------------------------------------------------------
  * Tuning table (no counterpart in the paper): threads per block (128, 256 or
  * 512) of the plain step kernel for a (lattice, model, storage, size class),
- * size class = floor(log2(cells)).  Process-wide; entries default to 256.
+ * size class = floor(log2(cells)).  Process-wide.  Without an entry a solver
+ * picks its block by storage form and domain size, and lbm_tuning_get reports 256.
  * Solvers adopt a changed entry at their next lbm_step (re-capturing their
  * graphs).  Check steps always use 256 threads, so flow rates and residuals
  * do not depend on the tuning.  The project's autotuner

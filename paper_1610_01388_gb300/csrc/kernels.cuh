@@ -1245,6 +1245,7 @@ __device__ __forceinline__ void step_begin(int& n) {
 #define BLBM_IR_MINB 0
 #endif
 template <class L, int MODEL, class S, bool CHECK, int BLOCK> constexpr int step_min_blocks() {
+    if (BLOCK < 128) return 0;   // small grids, and FP64: left to the allocator
     if (MODEL == LBM_MODEL_IR) return BLBM_IR_MINB;
     if (std::is_same<typename Store<S>::R, double>::value) return 0;
     if (BLBM_PR_MINB >= 0) return BLBM_PR_MINB;
@@ -2182,7 +2183,9 @@ cudaError_t launch_step_c(bool check, const KParams& kp, const StepArgs& s, cuda
     const int ncell = kp.cell_end - kp.cell_begin;   // the cells this launch covers
     const SrcPlanes<S> src = src_planes<L, S>(s.fsrc, kp.plane);
     const DstPlanes<S> dst = dst_planes<L, S>(s.fdst, kp.plane);
-    const int block = (check || MODEL == kModelPRImplicit) ? kBlock : s.block;   // implicit: untuned
+    constexpr bool f64 = std::is_same<typename Store<S>::R, double>::value;
+    // the implicit step is not in the tuning table (FP64: 64 threads, as untuned_block())
+    const int block = check ? kBlock : MODEL == kModelPRImplicit ? (f64 ? 64 : kBlock) : s.block;
     if constexpr (MODEL != kModelPRImplicit && std::is_same<typename Store<S>::R, float>::value) {
         if (!check && s.cpt == 2) {   // two cells per thread
             if (block == 128)
@@ -2200,6 +2203,9 @@ cudaError_t launch_step_c(bool check, const KParams& kp, const StepArgs& s, cuda
     // one part of a step taken in parts (256 threads)
     if (kp.cell_begin != 0 || kp.cell_end != kp.ncells)
         return go(k_step<L, MODEL, S, false, kBlock, COPY, true>, kBlock);
+    if constexpr (MODEL != kModelPRImplicit || f64) {
+        if (block == 64) return go(k_step<L, MODEL, S, false, 64, COPY>, 64);
+    }
     if constexpr (MODEL != kModelPRImplicit) {
         if (block == 128) return go(k_step<L, MODEL, S, false, 128, COPY>, 128);
         if (block == 512) return go(k_step<L, MODEL, S, false, 512, COPY>, 512);

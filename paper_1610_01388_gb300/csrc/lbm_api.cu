@@ -632,6 +632,7 @@ namespace {
 
 struct Shape {
     int block = kBlock, cpt = 1;
+    bool set = false;   // an entry of the table
 };
 
 std::mutex g_tune_mu;
@@ -654,11 +655,33 @@ Shape tune_lookup(int lat, int model, int storage, int64_t cells) {
     return it == g_tune.end() ? Shape{} : it->second;
 }
 
+// Threads per block of the plain steps of a dense solver the table has no
+// entry for (the compact layout and the Newton-implicit step have their own).
+// Measured on GB300, us per step at 64 / 128 / 256 threads:
+//  - FP64: one FP64 warp instruction holds its SM sub-partition's FP64 pipe for
+//    64 cycles, so warps must be spread over sub-partitions, 64-thread blocks
+//    the finest that fills them: D2Q9 IR 4 x 64: 3.9 / 4.3 / 7.5; D3Q27 IR 1 x
+//    64 x 64: 8.9 / 10.2 / 18.6; D3Q19 PR 40 x 64 x 64: 75.1 / 78.3 / 86.8.
+//  - FP32 arithmetic up to 8 blocks of 256 per SM (152 SMs): smaller blocks
+//    spread the last wave: D3Q15 PR F32 91k cells 2.85 / 2.89 / 3.07, D3Q27 IR F32
+//    80k 3.66 / 3.80 / 4.01, D3Q27 PR F32 262k 8.02 / 8.15 / 8.49.
+//  - larger 16-bit domains, bound by issue: 128 (D3Q27 PR F16 duct 256 x 128 x
+//    128: 113 / 102 / 109, porous 160^3: 117 / 116 / 123; D3Q19 IR F16: 68 / 65 / 67).
+//  - larger FP32 domains, bound by HBM: 256 (D3Q27 IR, porous 160^3: 157 / 156 /
+//    134), where a wider block's reads meet in L1, but for the PR step of
+//    domains whose walls fill whole warps: 64 (duct: 138.7 / 139.8 / 141.2).
+int untuned_block(const lbm_solver* s) {
+    if (s->p.storage == LBM_F64 || s->ncells <= 8 * 152 * kBlock) return 64;
+    if (storage_bytes(s->p.storage) == 2) return 128;
+    return s->p.model == LBM_MODEL_PR && !s->copy ? 64 : kBlock;
+}
+
 // Adopt the current table; a changed launch shape invalidates captured graphs.
 void apply_tuning(lbm_solver* s) {
     const uint64_t ver = g_tune_version.load();
     if (s->tune_version == ver) return;
-    const Shape sh = tune_lookup(s->lat, s->p.model, s->p.storage, s->ncells);
+    Shape sh = tune_lookup(s->lat, s->p.model, s->p.storage, s->ncells);
+    if (!sh.set) sh.block = untuned_block(s);
     if (sh.block != s->block || sh.cpt != s->cpt) {
         for (int k = 0; k < 2; ++k)
             if (s->graph[k]) {
@@ -683,7 +706,7 @@ lbm_status set_shape(int lat, int32_t model, int32_t storage, int32_t cls, int32
     if (cpt == 2 && storage == LBM_F64) return fail(LBM_EINVAL, "two cells per thread need FP32 arithmetic (not LBM_F64)");
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[tune_key(lat, model, storage, cls)] = Shape{block, cpt};
+        g_tune[tune_key(lat, model, storage, cls)] = Shape{block, cpt, true};
     }
     g_tune_version.fetch_add(1);
     return LBM_OK;
