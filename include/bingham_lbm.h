@@ -381,8 +381,10 @@ lbm_status lbm_tuning_clear(void);   /* also resets the batch schedule below */
  *   ctas_per_sm -- per (lattice, model, storage) group: 0 (default) launches
  *     one CTA per tile; n > 0 launches a persistent grid of min(tiles,
  *     n x SMs) CTAs that walk the tiles.  0..32.
- *   concurrency -- 1: the captured 16-step graphs run the groups as parallel
- *     branches (they touch disjoint memory); 0 (default): one after another.
+ *   concurrency -- 1: captured graphs run the groups as parallel branches
+ *     (they touch disjoint memory); 0: one after another.  Until it is set, a
+ *     batch of several groups runs them as branches, and
+ *     lbm_tuning_get_batch_concurrency reports 0.
  * Results do not depend on either: the per-cell arithmetic and the order of
  * every reduction are the same (check-step partials are kept per tile).
  * The project's autotuner (paper_1610_01388_gb300.autotune.tune_batch) times

@@ -32,6 +32,9 @@ constexpr int kFlowChangeSlot = kStatFlowChange;
 static_assert(kFlowChangeSlot == kNumStats - 1 && kStatNonFinite < kFlowChangeSlot,
               "the flow change takes the stats row's last entry, which check steps leave at 0");
 constexpr int kGraphLen = 16;       // steps per captured graph (even)
+// What a captured graph holds: kGraphLen plain steps, one plain step, or one
+// check step.  The last two exist for concurrent groups only.
+enum { kGraphRun = 0, kGraphOne, kGraphCheck, kGraphKinds };
 
 // Per domain: the fixed-order sum of its tiles' partials into its stats row,
 // and in the row's last entry the relative change of the flow-rate vector
@@ -40,7 +43,9 @@ constexpr int kGraphLen = 16;       // steps per captured graph (even)
 // the row held no previous check (lbm_batch_add clears it).
 __global__ void k_finalize_domains(const BatchDesc* __restrict__ descs,
                                    const double* __restrict__ partials, double* __restrict__ slots) {
-    const BatchDesc& D = descs[blockIdx.x];
+    int dom = blockIdx.x;
+    step_begin(dom);
+    const BatchDesc& D = descs[dom];
     double* row = slots + (int64_t)D.slot * kNumStats;
     double prev[3] = {0.0, 0.0, 0.0};
     if (threadIdx.x == 0)
@@ -123,7 +128,7 @@ double now_s() {
 std::mutex g_sched_mu;
 std::map<int, int> g_sched_ctas;
 std::map<int, std::map<int, std::pair<int, int>>> g_sched_tile;   // key -> size class -> shape
-std::atomic<int> g_sched_concurrent{0};
+std::atomic<int> g_sched_concurrent{-1};   // -1: not set, the library chooses
 std::atomic<uint64_t> g_sched_version{1};
 
 int sched_key(int lat, int model, int storage) { return (lat * 4 + model) * 8 + storage; }
@@ -172,7 +177,7 @@ void blbm::clear_batch_schedule() {
         g_sched_ctas.clear();
         g_sched_tile.clear();
     }
-    g_sched_concurrent.store(0);
+    g_sched_concurrent.store(-1);
     g_sched_version.fetch_add(1);
 }
 
@@ -191,7 +196,8 @@ struct lbm_batch {
     double* d_slots = nullptr;      // [kMaxSlots][kNumStats]
     double* h_slots = nullptr;      // pinned mirror
     bool dirty = true;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t graph[kGraphKinds][2] = {};   // by kind and phase
+    int rows = 0;                         // stats rows in use: [0, rows)
     bool poisoned = false;
     int sms = 1;                          // multiprocessors of the device
     uint64_t sched_version = 0;           // schedule the groups were built with
@@ -233,11 +239,12 @@ lbm_status benter(const lbm_batch* b) {
 }
 
 void drop_graphs(lbm_batch* b) {
-    for (int p = 0; p < 2; ++p)
-        if (b->graph[p]) {
-            cudaGraphExecDestroy(b->graph[p]);
-            b->graph[p] = nullptr;
-        }
+    for (auto& kind : b->graph)
+        for (auto& g : kind)
+            if (g) {
+                cudaGraphExecDestroy(g);
+                g = nullptr;
+            }
 }
 
 // (Re)build the per-group device tables after the set of domains or the
@@ -245,7 +252,12 @@ void drop_graphs(lbm_batch* b) {
 lbm_status rebuild(lbm_batch* b) {
     drop_graphs(b);
     b->sched_version = g_sched_version.load();
+    // Concurrent unless it was switched off: most groups of a mix are too small
+    // to fill the GPU (48 domains of the serving mix in 10 groups, us per step:
+    // 90 one after another, 61 as branches).
     b->concurrent = g_sched_concurrent.load() != 0;
+    b->rows = 0;
+    for (const auto& kv : b->doms) b->rows = std::max(b->rows, kv.second.slot + 1);
     std::vector<Group> old;
     old.swap(b->groups);
     for (auto& kv : b->doms) {
@@ -360,8 +372,8 @@ cudaError_t launch_group(lbm_batch* b, const Group& g, bool check, int phase, cu
                                          g.d_pblock_dom, g.pnblocks, g.pgrid, phase, nullptr,
                                          g.tile_threads, g.tile_cpt, st);
     if (e != cudaSuccess || !check) return e;
-    k_finalize_domains<<<(int)g.ids.size(), kBlock, 0, st>>>(g.d_desc, g.d_partials, b->d_slots);
-    return cudaGetLastError();
+    return launch_overlapped(k_finalize_domains, (int)g.ids.size(), kBlock, st, g.d_desc, g.d_partials,
+                             b->d_slots);
 }
 
 cudaError_t launch_all(lbm_batch* b, bool check, cudaStream_t st) {
@@ -377,7 +389,7 @@ cudaError_t launch_all(lbm_batch* b, bool check, cudaStream_t st) {
 // their step chains need no order between them.  Every forked branch is
 // joined back into the origin stream, also after an error, so the capture
 // can always be ended.
-cudaError_t capture_branches(lbm_batch* b, int par, int active) {
+cudaError_t capture_branches(lbm_batch* b, int kind, int par, int active) {
     cudaError_t e = cudaSuccess;
     if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     while (e == cudaSuccess && (int)b->branch.size() < active) {
@@ -396,8 +408,9 @@ cudaError_t capture_branches(lbm_batch* b, int par, int active) {
         if (g.ids.empty()) continue;
         cudaStream_t st = b->branch[k];
         cudaError_t eb = cudaStreamWaitEvent(st, b->fork, 0);
-        for (int t = 0; t < kGraphLen && eb == cudaSuccess; ++t)
-            eb = launch_group(b, g, false, par ^ (t & 1), st);
+        const int steps = kind == kGraphRun ? kGraphLen : 1;
+        for (int t = 0; t < steps && eb == cudaSuccess; ++t)
+            eb = launch_group(b, g, kind == kGraphCheck, par ^ (t & 1), st);
         cudaError_t ej = cudaEventRecord(b->join[k], st);
         if (ej == cudaSuccess) ej = cudaStreamWaitEvent(b->cap, b->join[k], 0);
         if (e == cudaSuccess) e = eb != cudaSuccess ? eb : ej;
@@ -406,7 +419,7 @@ cudaError_t capture_branches(lbm_batch* b, int par, int active) {
     return e;
 }
 
-cudaError_t capture(lbm_batch* b, int par) {
+cudaError_t capture(lbm_batch* b, int kind, int par) {
     if (!b->cap) {
         cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
         if (e != cudaSuccess) return e;
@@ -421,8 +434,8 @@ cudaError_t capture(lbm_batch* b, int par) {
     int active = 0;
     for (const auto& g : b->groups) active += !g.ids.empty();
     if (b->concurrent && active > 1) {
-        e = capture_branches(b, par, active);
-    } else {
+        e = capture_branches(b, kind, par, active);
+    } else {   // kGraphRun
         for (int t = 0; t < kGraphLen && e == cudaSuccess; ++t) {
             e = launch_all(b, false, b->cap);
             b->phase ^= 1;
@@ -436,7 +449,7 @@ cudaError_t capture(lbm_batch* b, int par) {
         return e;
     }
     if (e2 != cudaSuccess) return e2;
-    e = cudaGraphInstantiate(&b->graph[par], g, 0);
+    e = cudaGraphInstantiate(&b->graph[kind][par], g, 0);
     cudaGraphDestroy(g);
     return e;
 }
@@ -552,30 +565,47 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     }
     if (b->sched_version != g_sched_version.load()) b->dirty = true;
     if (b->dirty && (v = rebuild(b)) != LBM_OK) return v;
+    int active = 0;
+    for (const auto& g : b->groups) active += !g.ids.empty();
+    const bool branches = b->concurrent && active > 1;
+    // one launch of a graph of this kind, at the current phase
+    auto replay = [&](int kind) {
+        cudaGraphExec_t& g = b->graph[kind][b->phase];
+        if (!g) BCK(b, capture(b, kind, b->phase), "batch graph capture");
+        BCK(b, cudaGraphLaunch(g, b->stream), "batch graph launch");
+        return LBM_OK;
+    };
     int64_t left = nsteps;
     while (left > 0) {
         const int64_t to_check = b->k - (b->gstep % b->k);
         int64_t plain = std::min(to_check - 1, left);
         while (plain >= kGraphLen) {
-            if (!b->graph[b->phase]) BCK(b, capture(b, b->phase), "batch graph capture");
-            BCK(b, cudaGraphLaunch(b->graph[b->phase], b->stream), "batch graph launch");
+            if ((v = replay(kGraphRun)) != LBM_OK) return v;
             b->gstep += kGraphLen;          // even: the phase is unchanged
             plain -= kGraphLen;
             left -= kGraphLen;
         }
         while (plain > 0) {
-            BCK(b, launch_all(b, false, b->stream), "batch step");
+            if (branches) {
+                if ((v = replay(kGraphOne)) != LBM_OK) return v;
+            } else {
+                BCK(b, launch_all(b, false, b->stream), "batch step");
+            }
             b->phase ^= 1;
             b->gstep += 1;
             --plain;
             --left;
         }
         if (left > 0) {
-            BCK(b, launch_all(b, true, b->stream), "batch check step");
+            if (branches) {
+                if ((v = replay(kGraphCheck)) != LBM_OK) return v;
+            } else {
+                BCK(b, launch_all(b, true, b->stream), "batch check step");
+            }
             b->phase ^= 1;
             b->gstep += 1;
             --left;
-            BCK(b, cudaMemcpyAsync(b->h_slots, b->d_slots, sizeof(double) * kNumStats * kMaxSlots,
+            BCK(b, cudaMemcpyAsync(b->h_slots, b->d_slots, sizeof(double) * kNumStats * b->rows,
                                    cudaMemcpyDeviceToHost, b->stream), "batch stats copy");
             for (auto& kv : b->doms) kv.second.checks += 1;
         }
@@ -690,7 +720,7 @@ lbm_status lbm_tuning_set_batch_concurrency(int32_t concurrent) {
 
 lbm_status lbm_tuning_get_batch_concurrency(int32_t* concurrent) {
     if (!concurrent) return fail(LBM_EINVAL, "concurrent is NULL");
-    *concurrent = g_sched_concurrent.load();
+    *concurrent = g_sched_concurrent.load() == 1;
     return LBM_OK;
 }
 
