@@ -205,6 +205,22 @@ __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ F2 recip(F2 x) { return F2(1.0f / x.lo(), 1.0f / x.hi()); }
 
+// Arithmetic with every rounding spelled out (mad: one, fused).  The compiler
+// may neither fuse these nor take a fused one apart, so a collision written in
+// them gives the same bits in every kernel it is compiled into.
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ F2 add(F2 a, F2 b) { return f2_add(a, b); }
+__device__ __forceinline__ F2 sub(F2 a, F2 b) { return f2_sub(a, b); }
+__device__ __forceinline__ F2 mul(F2 a, F2 b) { return f2_mul(a, b); }
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return f2_fma(a, b, c); }
+
 // ---------------------------------------------------------------------------
 // storage.  R is the arithmetic type.  ld / st move population i between
 // memory and registers; enc / dec convert full FP64 populations at the ABI
@@ -560,11 +576,11 @@ static_assert(fam_order<D2Q9>() && fam_order<D3Q15>() && fam_order<D3Q19>() && f
 // b x and y + b x for a compile-time factor b (a plain x, y + x where it is 1)
 template <class R, class B> __device__ __forceinline__ R scale(B b, R x) {
     if (b == B(1)) return x;
-    return x * R(b);
+    return mul(x, R(b));
 }
 template <class R, class B> __device__ __forceinline__ R axpy(B b, R x, R y) {
-    if (b == B(1)) return y + x;
-    return y + x * R(b);
+    if (b == B(1)) return add(y, x);
+    return mad(x, R(b), y);
 }
 
 // Pair form: f[i] = f_i + f_o and f[o] = f_i - f_o for every opposite pair
@@ -574,8 +590,8 @@ template <class L, class R> __device__ __forceinline__ void to_pairs(R (&f)[L::Q
     static_for<0, (L::Q - 1) / 2>([&](auto P) {
         constexpr int i = 2 * decltype(P)::value + 1;
         const R a = f[i], b = f[i + 1];
-        f[i] = a + b;
-        f[i + 1] = a - b;
+        f[i] = add(a, b);
+        f[i + 1] = sub(a, b);
     });
 }
 
@@ -595,41 +611,41 @@ __device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
     constexpr auto bC = Store<S>::template beta<L, (C ? C : 1)>();
     Mom<R> m;
     if constexpr (L::D == 2) {
-        const R XY = scale(bF, R(f[F] + f[F + 2]));
+        const R XY = scale(bF, add(f[F], f[F + 2]));
         m.xx = axpy(bA, f[1], XY);
         m.yy = axpy(bA, f[3], XY);
-        m.d = m.xx + axpy(b0, f[0], scale(bA, f[3]));
-        m.xy = scale(bF, R(f[F] - f[F + 2]));
-        m.jx = axpy(bA, f[2], scale(bF, R(f[F + 1] + f[F + 3])));
-        m.jy = axpy(bA, f[4], scale(bF, R(f[F + 1] - f[F + 3])));
+        m.d = add(m.xx, axpy(b0, f[0], scale(bA, f[3])));
+        m.xy = scale(bF, sub(f[F], f[F + 2]));
+        m.jx = axpy(bA, f[2], scale(bF, add(f[F + 1], f[F + 3])));
+        m.jy = axpy(bA, f[4], scale(bF, sub(f[F + 1], f[F + 3])));
         m.zz = R(0);
         m.jz = R(0);
         m.xz = R(0);
         m.yz = R(0);
     } else {
-        R X, Y, Z, rest = scale(bA, R(f[3] + f[5]));   // X: diagonal sums beyond the axis pairs
+        R X, Y, Z, rest = scale(bA, add(f[3], f[5]));   // X: diagonal sums beyond the axis pairs
         R jx, jy, jz;
         if constexpr (C != 0) {
-            const R ab = f[C] + f[C + 2], amb = f[C] - f[C + 2];
-            const R ce = f[C + 4] + f[C + 6], cme = f[C + 4] - f[C + 6];
-            X = scale(bC, R(ab + ce));
-            m.xy = scale(bC, R(ab - ce));
-            m.xz = scale(bC, R(amb + cme));
-            m.yz = scale(bC, R(amb - cme));
-            const R dp = f[C + 1] + f[C + 3], dq = f[C + 5] - f[C + 7];
-            jx = scale(bC, R(dp + dq));
-            jy = scale(bC, R(dp - dq));
-            jz = scale(bC, R((f[C + 1] - f[C + 3]) + (f[C + 5] + f[C + 7])));
+            const R ab = add(f[C], f[C + 2]), amb = sub(f[C], f[C + 2]);
+            const R ce = add(f[C + 4], f[C + 6]), cme = sub(f[C + 4], f[C + 6]);
+            X = scale(bC, add(ab, ce));
+            m.xy = scale(bC, sub(ab, ce));
+            m.xz = scale(bC, add(amb, cme));
+            m.yz = scale(bC, sub(amb, cme));
+            const R dp = add(f[C + 1], f[C + 3]), dq = sub(f[C + 5], f[C + 7]);
+            jx = scale(bC, add(dp, dq));
+            jy = scale(bC, sub(dp, dq));
+            jz = scale(bC, add(sub(f[C + 1], f[C + 3]), add(f[C + 5], f[C + 7])));
             Y = X;
             Z = X;
         }
         if constexpr (F != 0) {
-            const R sxy = f[F] + f[F + 2], sxz = f[F + 4] + f[F + 6], syz = f[F + 8] + f[F + 10];
-            const R oxy = f[F] - f[F + 2], oxz = f[F + 4] - f[F + 6], oyz = f[F + 8] - f[F + 10];
-            const R fx = (f[F + 1] + f[F + 3]) + (f[F + 5] + f[F + 7]);
-            const R fy = (f[F + 1] - f[F + 3]) + (f[F + 9] + f[F + 11]);
-            const R fz = (f[F + 5] - f[F + 7]) + (f[F + 9] - f[F + 11]);
-            const R xs = sxy + sxz, ys = sxy + syz, zs = sxz + syz;
+            const R sxy = add(f[F], f[F + 2]), sxz = add(f[F + 4], f[F + 6]), syz = add(f[F + 8], f[F + 10]);
+            const R oxy = sub(f[F], f[F + 2]), oxz = sub(f[F + 4], f[F + 6]), oyz = sub(f[F + 8], f[F + 10]);
+            const R fx = add(add(f[F + 1], f[F + 3]), add(f[F + 5], f[F + 7]));
+            const R fy = add(sub(f[F + 1], f[F + 3]), add(f[F + 9], f[F + 11]));
+            const R fz = add(sub(f[F + 5], f[F + 7]), sub(f[F + 9], f[F + 11]));
+            const R xs = add(sxy, sxz), ys = add(sxy, syz), zs = add(sxz, syz);
             rest = axpy(bF, syz, rest);
             if constexpr (C != 0) {
                 X = axpy(bF, xs, X);
@@ -656,7 +672,7 @@ __device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
         m.xx = axpy(bA, f[1], X);
         m.yy = axpy(bA, f[3], Y);
         m.zz = axpy(bA, f[5], Z);
-        m.d = m.xx + axpy(b0, f[0], rest);
+        m.d = add(m.xx, axpy(b0, f[0], rest));
         m.jx = axpy(bA, f[2], jx);
         m.jy = axpy(bA, f[4], jy);
         m.jz = axpy(bA, f[6], jz);
@@ -679,13 +695,13 @@ __device__ __forceinline__ Mom<R> moments(R (&f)[L::Q]) {
 template <class L, class R>
 __device__ __forceinline__ Tens<R> outer(R ax, R ay, R az, R bx, R by, R bz) {
     Tens<R> t;
-    t.xx = ax * bx;
-    t.yy = ay * by;
-    t.xy = ax * by;
+    t.xx = mul(ax, bx);
+    t.yy = mul(ay, by);
+    t.xy = mul(ax, by);
     if constexpr (L::D == 3) {
-        t.zz = az * bz;
-        t.xz = ax * bz;
-        t.yz = ay * bz;
+        t.zz = mul(az, bz);
+        t.xz = mul(ax, bz);
+        t.yz = mul(ay, bz);
     } else {
         t.zz = R(0);
         t.xz = R(0);
@@ -698,15 +714,15 @@ __device__ __forceinline__ Tens<R> outer(R ax, R ay, R az, R bx, R by, R bz) {
 // offsets: Pi = c_s^2 I + p, rho = 1 + d.  ruu = rho u u.
 template <class L, class R>
 __device__ __forceinline__ Tens<R> noneq(const Mom<R>& m, const Tens<R>& ruu, uint32_t flags) {
-    const R d3 = m.d * R(1.0 / 3.0);
+    const R third = R(-1.0 / 3.0);
     Tens<R> t;
-    t.xx = m.xx - d3 - ruu.xx;
-    t.yy = m.yy - d3 - ruu.yy;
-    t.xy = m.xy - ruu.xy;
+    t.xx = sub(mad(m.d, third, m.xx), ruu.xx);
+    t.yy = sub(mad(m.d, third, m.yy), ruu.yy);
+    t.xy = sub(m.xy, ruu.xy);
     if constexpr (L::D == 3) {
-        t.zz = m.zz - d3 - ruu.zz;
-        t.xz = m.xz - ruu.xz;
-        t.yz = m.yz - ruu.yz;
+        t.zz = sub(mad(m.d, third, m.zz), ruu.zz);
+        t.xz = sub(m.xz, ruu.xz);
+        t.yz = sub(m.yz, ruu.yz);
     } else {
         t.zz = R(0);
         t.xz = R(0);
@@ -716,15 +732,19 @@ __device__ __forceinline__ Tens<R> noneq(const Mom<R>& m, const Tens<R>& ruu, ui
     return t;
 }
 
-template <class L, class R> __device__ __forceinline__ R tnorm2(const Tens<R>& T) {
-    R s = T.xx * T.xx + T.yy * T.yy + R(2) * T.xy * T.xy;
-    if constexpr (L::D == 3) s += T.zz * T.zz + R(2) * (T.xz * T.xz + T.yz * T.yz);
-    return s;
+// T:T
+template <class L, class R> __device__ __forceinline__ R square(const Tens<R>& T) {
+    R off = mul(T.xy, T.xy), diag = mad(T.yy, T.yy, mul(T.xx, T.xx));
+    if constexpr (L::D == 3) {
+        off = mad(T.yz, T.yz, mad(T.xz, T.xz, off));
+        diag = mad(T.zz, T.zz, diag);
+    }
+    return mad(R(2), off, diag);
 }
 
 template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t) {
-    if constexpr (L::D == 3) return t.xx + t.yy + t.zz;
-    return t.xx + t.yy;
+    if constexpr (L::D == 3) return add(add(t.xx, t.yy), t.zz);
+    return add(t.xx, t.yy);
 }
 
 // The post-collision populations of both models have the form
@@ -733,61 +753,60 @@ template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t)
 // members of a family differ only by the signs of the off-diagonal terms: one
 // sum per axis pair, two per face plane, one 4-point butterfly for the
 // corners, instead of c.u, its square and c.T.c per pair (D3Q27: 23 adds
-// against 150 operations).  put(i, even, odd) stores pair i: even and odd
-// carry their weights.  Where w_i in memory units is the same for every
-// direction (the 16-bit forms) it goes into the six numbers and q once.
+// against 150 operations).  put(i, e, we, cq, wo) stores pair i, its even part
+// we e and its odd part wo cq.  Where w_i in memory units is the same for
+// every direction (the 16-bit forms) it goes into the six numbers and q once,
+// and we = wo = 1.
 template <class L, class S, class R, class Put>
 __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R qz, Put&& put) {
     constexpr int F = Fam<L>::face, C = Fam<L>::corner;
     constexpr bool same = sizeof(S) == 2;   // gam, god do not depend on the direction
     constexpr auto g0 = Store<S>::template gam<L, 1>();
     constexpr auto o0 = Store<S>::template god<L, 1>();
+    using B = std::remove_const_t<decltype(g0)>;
     if constexpr (same) {
         e0 = scale(g0, e0);
         qx = scale(o0, qx);
         qy = scale(o0, qy);
         if constexpr (L::D == 3) qz = scale(o0, qz);
     }
-    const R k = R(same ? decltype(g0)(4.5) * g0 : decltype(g0)(4.5));
-    const R k2 = R(same ? decltype(g0)(9) * g0 : decltype(g0)(9));
+    const R k = R(same ? B(4.5) * g0 : B(4.5));
+    const R k2 = R(same ? B(9) * g0 : B(9));
     auto pair = [&](auto I, R e, R cq) {
         constexpr int i = decltype(I)::value;
-        if constexpr (same)
-            put(I, e, cq);
-        else
-            put(I, R(e * R(Store<S>::template gam<L, i>())), R(cq * R(Store<S>::template god<L, i>())));
+        if constexpr (same) put(I, e, B(1), cq, B(1));
+        else put(I, e, Store<S>::template gam<L, i>(), cq, Store<S>::template god<L, i>());
     };
 #define BLBM_I(n) std::integral_constant<int, (n)>{}
-    const R ex = e0 + k * N.xx;
+    const R ex = mad(k, N.xx, e0);
     pair(BLBM_I(1), ex, qx);
-    const R ay = k * N.yy;
-    pair(BLBM_I(3), R(e0 + ay), qy);
-    const R exy = ex + ay;
-    const R bxy = k2 * N.xy;
-    const R qxpy = qx + qy, qxmy = qx - qy;
+    pair(BLBM_I(3), mad(k, N.yy, e0), qy);
+    const R exy = mad(k, N.yy, ex);
+    const R bxy = mul(k2, N.xy);
+    const R qxpy = add(qx, qy), qxmy = sub(qx, qy);
     if constexpr (L::D == 2) {
-        pair(BLBM_I(F), R(exy + bxy), qxpy);
-        pair(BLBM_I(F + 2), R(exy - bxy), qxmy);
+        pair(BLBM_I(F), add(exy, bxy), qxpy);
+        pair(BLBM_I(F + 2), sub(exy, bxy), qxmy);
     } else {
-        const R az = k * N.zz;
-        const R bxz = k2 * N.xz, byz = k2 * N.yz;
-        pair(BLBM_I(5), R(e0 + az), qz);
+        const R bxz = mul(k2, N.xz), byz = mul(k2, N.yz);
+        const R ez = mad(k, N.zz, e0);
+        pair(BLBM_I(5), ez, qz);
         if constexpr (F != 0) {
-            pair(BLBM_I(F), R(exy + bxy), qxpy);
-            pair(BLBM_I(F + 2), R(exy - bxy), qxmy);
-            const R exz = ex + az, eyz = e0 + ay + az;
-            pair(BLBM_I(F + 4), R(exz + bxz), R(qx + qz));
-            pair(BLBM_I(F + 6), R(exz - bxz), R(qx - qz));
-            pair(BLBM_I(F + 8), R(eyz + byz), R(qy + qz));
-            pair(BLBM_I(F + 10), R(eyz - byz), R(qy - qz));
+            pair(BLBM_I(F), add(exy, bxy), qxpy);
+            pair(BLBM_I(F + 2), sub(exy, bxy), qxmy);
+            const R exz = mad(k, N.zz, ex), eyz = mad(k, N.yy, ez);
+            pair(BLBM_I(F + 4), add(exz, bxz), add(qx, qz));
+            pair(BLBM_I(F + 6), sub(exz, bxz), sub(qx, qz));
+            pair(BLBM_I(F + 8), add(eyz, byz), add(qy, qz));
+            pair(BLBM_I(F + 10), sub(eyz, byz), sub(qy, qz));
         }
         if constexpr (C != 0) {
-            const R e = exy + az;
-            const R ep = e + byz, em = e - byz, bp = bxy + bxz, bm = bxy - bxz;
-            pair(BLBM_I(C), R(ep + bp), R(qxpy + qz));
-            pair(BLBM_I(C + 2), R(em + bm), R(qxpy - qz));
-            pair(BLBM_I(C + 4), R(em - bm), R(qxmy + qz));
-            pair(BLBM_I(C + 6), R(ep - bp), R(qz - qxmy));
+            const R e = mad(k, N.zz, exy);
+            const R ep = add(e, byz), em = sub(e, byz), bp = add(bxy, bxz), bm = sub(bxy, bxz);
+            pair(BLBM_I(C), add(ep, bp), add(qxpy, qz));
+            pair(BLBM_I(C + 2), add(em, bm), sub(qxpy, qz));
+            pair(BLBM_I(C + 4), sub(em, bm), add(qxmy, qz));
+            pair(BLBM_I(C + 6), sub(ep, bp), sub(qz, qxmy));
         }
     }
 #undef BLBM_I
@@ -809,8 +828,8 @@ __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R
         asg[k] = Sc(-1);
         if (t2 > Sc(0) && t2 >= c.s2y2) {
             const Sc it = rsqrt(t2);
-            as[k] = c.ir_as * it - c.ir_a;
-            asg[k] = -(c.ir_bs * it + c.ir_bn);
+            as[k] = mad(c.ir_as, it, -c.ir_a);
+            asg[k] = mad(-c.ir_bs, it, -c.ir_bn);
         }
     }
     as_out = Lanes<R>::make(as);
@@ -824,45 +843,49 @@ template <class L, class S, class R>
 __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
                                            R (&f)[L::Q], R& drho, R (&ur)[3]) {
     const Mom<R> m = moments<L, S, R>(f);
-    const R rho = R(1) + m.d;
+    const R rho = add(R(1), m.d);
     const R inv = recip(rho);
-    const R Fx = rho * R(c.g[0]), Fy = rho * R(c.g[1]);
-    R Fz = R(0);
-    if constexpr (L::D == 3) Fz = rho * R(c.g[2]);
-    const R px = m.jx + R(0.5) * Fx, py = m.jy + R(0.5) * Fy;   // rho u
+    const R gx = R(c.g[0]), gy = R(c.g[1]);
+    R gz = R(0);
+    if constexpr (L::D == 3) gz = R(c.g[2]);
+    const R half = mul(R(0.5), rho);
+    const R px = mad(half, gx, m.jx), py = mad(half, gy, m.jy);   // rho u
     R pz = R(0);
-    if constexpr (L::D == 3) pz = m.jz + R(0.5) * Fz;
-    const R ux = px * inv, uy = py * inv;
+    if constexpr (L::D == 3) pz = mad(half, gz, m.jz);
+    const R ux = mul(px, inv), uy = mul(py, inv);
     R uz = R(0);
-    if constexpr (L::D == 3) uz = pz * inv;
+    if constexpr (L::D == 3) uz = mul(pz, inv);
     const Tens<R> U = outer<L, R>(px, py, pz, ux, uy, uz);
     const Tens<R> T = noneq<L, R>(m, U, flags);
     R as, asg;
-    ir_yield<R>(c, tnorm2<L, R>(T), as, asg);
+    ir_yield<R>(c, square<L, R>(T), as, asg);
     // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I;
     // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i
-    const R k1 = R(0.5) * as - asg;
-    const R k2 = asg * trace<L, R>(T) * R(1.0 / L::D);
+    const R k1 = mad(R(0.5), as, -asg);
+    const R k2 = mul(asg, mul(trace<L, R>(T), R(1.0 / L::D)));
     Tens<R> N;
-    N.xx = U.xx + (k1 * T.xx + k2);
-    N.yy = U.yy + (k1 * T.yy + k2);
-    N.xy = U.xy + k1 * T.xy;
+    N.xx = add(U.xx, mad(k1, T.xx, k2));
+    N.yy = add(U.yy, mad(k1, T.yy, k2));
+    N.xy = mad(k1, T.xy, U.xy);
     N.zz = R(0);
     N.xz = R(0);
     N.yz = R(0);
     if constexpr (L::D == 3) {
-        N.zz = U.zz + (k1 * T.zz + k2);
-        N.xz = U.xz + k1 * T.xz;
-        N.yz = U.yz + k1 * T.yz;
+        N.zz = add(U.zz, mad(k1, T.zz, k2));
+        N.xz = mad(k1, T.xz, U.xz);
+        N.yz = mad(k1, T.yz, U.yz);
     }
-    const R e0 = m.d - R(1.5) * trace<L, R>(N);
+    const R e0 = mad(R(-1.5), trace<L, R>(N), m.d);
     // odd part: w_i (3 rho c.u + 3/2 c.F) = 3 w_i c.(j + F), since rho u = j + F/2
-    const R qx = m.jx + Fx, qy = m.jy + Fy, qz = m.jz + Fz;
-    f[0] = R(Store<S>::template gam<L, 0>()) * e0;
-    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, R od) {
+    const R qx = mad(rho, gx, m.jx), qy = mad(rho, gy, m.jy);
+    R qz = R(0);
+    if constexpr (L::D == 3) qz = mad(rho, gz, m.jz);
+    f[0] = scale(Store<S>::template gam<L, 0>(), e0);
+    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, auto we, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
-        f[i] = e + od;
-        f[i + 1] = e - od;
+        e = scale(we, e);
+        f[i] = axpy(wo, cq, e);
+        f[i + 1] = axpy(-wo, cq, e);
     });
     drho = m.d;
     ur[0] = ux;
@@ -935,6 +958,48 @@ __device__ __forceinline__ void pr_rates(const Coef<typename Lanes<R>::Sc>& c, R
     wm_out = Lanes<R>::make(wm_);
 }
 
+// The same for the pair form.  itau: 1 / (previous step's tau).  FP64 takes
+// both rates from one division (a product of two moderate numbers; beyond that
+// range, which only an extreme m reaches, from two).
+template <bool IMPLICIT, class R>
+__device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>& c, R tn2, R inv,
+                                              R itau, R& tau, R& wp_out, R& wm_out) {
+    using Sc = typename Lanes<R>::Sc;
+    Sc tau_[Lanes<R>::n], wp_[Lanes<R>::n], wm_[Lanes<R>::n];
+#pragma unroll
+    for (int k = 0; k < Lanes<R>::n; ++k) {
+        const Sc tt = mul(Sc(1.5), sqrt(mul(Sc(2), Lanes<R>::get(tn2, k))));
+        Sc gd = mul(Lanes<R>::get(itau, k), tt);
+        const Sc sy_rho = mul(c.sigma_y, Lanes<R>::get(inv, k));
+        if constexpr (IMPLICIT) gd = pr_newton(c, tt, gd, sy_rho);
+        Sc nu;
+        if (gd >= c.gdot_c) {
+            nu = add(c.nu_p, mul(sy_rho, -expm1(mul(-c.m, gd))) / gd);
+        } else {
+            const Sc nu0 = mad(c.m, sy_rho, c.nu_p);
+            const Sc nuc = mad(sy_rho, c.e_c, c.nu_p);
+            const Sc s = mul(gd, c.inv_gc);
+            nu = mad(mul(sub(c.gdot_c, gd), c.inv_gc), nu0, mul(s, nuc));
+        }
+        const Sc tn = mad(Sc(3), nu, Sc(0.5));
+        // 1 / tau_odd with tau_odd = 1/2 + Lambda / (tau - 1/2) is tm / odd
+        const Sc tm = sub(tn, Sc(0.5));
+        const Sc odd = mad(Sc(0.5), tm, c.magic);
+        if (sizeof(Sc) == 8 && tn < Sc(1e30)) {
+            const Sc r = recip(mul(tn, odd));
+            wp_[k] = mul(r, odd);
+            wm_[k] = mul(tm, mul(r, tn));
+        } else {
+            wp_[k] = recip(tn);
+            wm_[k] = tm / odd;
+        }
+        tau_[k] = tn;
+    }
+    tau = Lanes<R>::make(tau_);
+    wp_out = Lanes<R>::make(wp_);
+    wm_out = Lanes<R>::make(wm_);
+}
+
 // ---------------------------------------------------------------------------
 // PR collision (Sec. 3.1 + TRT + EDM).  tau: previous step's relaxation time
 // in, this step's out.  f: memory units in, memory units out (the TRT update is
@@ -943,20 +1008,30 @@ template <class L, class S, bool IMPLICIT, class R>
 __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
                                            R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
     const Mom<R> m = moments<L, S, R>(f);
-    const R rho = R(1) + m.d;
-    const R inv = recip(rho);
-    const R ux = m.jx * inv, uy = m.jy * inv;
+    const R rho = add(R(1), m.d);
+    R inv, itau;   // 1 / rho, 1 / tau_old
+    if constexpr (sizeof(typename Lanes<R>::Sc) == 8) {
+        const R q = recip(mul(rho, tau));   // one FP64 division for both
+        inv = mul(q, tau);
+        itau = mul(q, rho);
+    } else {
+        inv = recip(rho);
+        itau = recip(tau);
+    }
+    const R ux = mul(m.jx, inv), uy = mul(m.jy, inv);
     R uz = R(0);
-    if constexpr (L::D == 3) uz = m.jz * inv;
+    if constexpr (L::D == 3) uz = mul(m.jz, inv);
     R wp, wm;
     {
         const Tens<R> T = noneq<L, R>(m, outer<L, R>(m.jx, m.jy, m.jz, ux, uy, uz), flags);
-        pr_rates<IMPLICIT, R>(c, tnorm2<L, R>(T), inv, tau, wp, wm);
+        pair_pr_rates<IMPLICIT, R>(c, square<L, R>(T), inv, itau, tau, wp, wm);
     }
     const R gx = R(c.g[0]), gy = R(c.g[1]);
     R gz = R(0);
     if constexpr (L::D == 3) gz = R(c.g[2]);
-    const R Fx = rho * gx, Fy = rho * gy, Fz = rho * gz;
+    const R Fx = mul(rho, gx), Fy = mul(rho, gy);
+    R Fz = R(0);
+    if constexpr (L::D == 3) Fz = mul(rho, gz);
     // Per pair (i, o = opposite), with f^+- = (f_i +- f_o) / 2:
     //   E = f^+ - wp (f^+ - f_eq^+) + F^+ = (1 - wp)/2 (f_i + f_o) + w_i (K0 + 9/2 c.N.c),
     //       N = rho (wp u u + u g + g u + g g) = j (wp u + g) + F (u + g),
@@ -966,43 +1041,48 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     // = 3 w_i c.j exactly).  f holds the pair sums and differences.
     Tens<R> N;
     {
-        const R vx = wp * ux + gx, vy = wp * uy + gy, zx = ux + gx, zy = uy + gy;
-        N.xx = m.jx * vx + Fx * zx;
-        N.yy = m.jy * vy + Fy * zy;
-        N.xy = m.jx * vy + Fx * zy;
+        const R vx = mad(wp, ux, gx), vy = mad(wp, uy, gy), zx = add(ux, gx), zy = add(uy, gy);
+        N.xx = mad(m.jx, vx, mul(Fx, zx));
+        N.yy = mad(m.jy, vy, mul(Fy, zy));
+        N.xy = mad(m.jx, vy, mul(Fx, zy));
         N.zz = R(0);
         N.xz = R(0);
         N.yz = R(0);
         if constexpr (L::D == 3) {
-            const R vz = wp * uz + gz, zz = uz + gz;
-            N.zz = m.jz * vz + Fz * zz;
-            N.xz = m.jx * vz + Fx * zz;
-            N.yz = m.jy * vz + Fy * zz;
+            const R vz = mad(wp, uz, gz), zz = add(uz, gz);
+            N.zz = mad(m.jz, vz, mul(Fz, zz));
+            N.xz = mad(m.jx, vz, mul(Fx, zz));
+            N.yz = mad(m.jy, vz, mul(Fy, zz));
         }
     }
-    const R omp = R(0.5) - R(0.5) * wp;
-    const R omm = R(0.5) - R(0.5) * wm;
-    const R K0 = wp * m.d - R(1.5) * trace<L, R>(N);
-    const R qx = wm * m.jx + Fx, qy = wm * m.jy + Fy, qz = wm * m.jz + Fz;
-    {
-        const R w0 = R(Store<S>::template gam<L, 0>());
-        f[0] = (R(1) - wp) * f[0] + w0 * K0;
-    }
-    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, R od) {
+    const R omp = mad(R(-0.5), wp, R(0.5));
+    const R omm = mad(R(-0.5), wm, R(0.5));
+    const R K0 = mad(R(-1.5), trace<L, R>(N), mul(wp, m.d));
+    const R qx = mad(wm, m.jx, Fx), qy = mad(wm, m.jy, Fy);
+    R qz = R(0);
+    if constexpr (L::D == 3) qz = mad(wm, m.jz, Fz);
+    f[0] = axpy(Store<S>::template gam<L, 0>(), K0, mul(sub(R(1), wp), f[0]));
+    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, auto we, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
-        const R E = omp * f[i] + e;
-        const R O = omm * f[i + 1] + od;
-        f[i] = E + O;
-        f[i + 1] = E - O;
+        const R E = mad(omp, f[i], scale(we, e));
+        const R O = mad(omm, f[i + 1], scale(wo, cq));
+        f[i] = add(E, O);
+        f[i + 1] = sub(E, O);
     });
     drho = m.d;
-    ur[0] = ux + R(0.5) * gx;
-    ur[1] = uy + R(0.5) * gy;
-    ur[2] = uz + R(0.5) * gz;
+    ur[0] = mad(R(0.5), gx, ux);
+    ur[1] = mad(R(0.5), gy, uy);
+    ur[2] = mad(R(0.5), gz, uz);
 }
 
 // ---------------------------------------------------------------------------
 // The same two collisions on class sums, for FP32 storage (see pair_form).
+template <class L, class R> __device__ __forceinline__ R tnorm2(const Tens<R>& T) {
+    R s = T.xx * T.xx + T.yy * T.yy + R(2) * T.xy * T.xy;
+    if constexpr (L::D == 3) s += T.zz * T.zz + R(2) * (T.xz * T.xz + T.yz * T.yz);
+    return s;
+}
+
 template <class L, class R>
 __device__ __forceinline__ Tens<R> class_noneq(const Mom<R>& m, R rho, R ux, R uy, R uz, uint32_t flags) {
     const R d3 = m.d * R(1.0 / 3.0);
@@ -1496,6 +1576,128 @@ k_step2(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
         rnd[1] = pcg_hash(((uint32_t)idx[1] + kp.hash_offset) ^ (seed * 0x9e3779b9u));
     }
     cell_step2<L, MODEL, S>(kp, a.cf, src, dst, lk, idx, act, tau, rnd);
+}
+
+// ---------------------------------------------------------------------------
+// Resident steps: a run of plain steps of a small domain in one launch, its
+// populations held in the shared memory of one cluster.  A step of such a
+// domain is almost only launch and memory latency (256 cells: 1.6 us of which
+// the arithmetic is a quarter); here a step is a gather from the cluster's
+// shared memory, the collision and one cluster barrier.  Thread t of block b
+// owns cell b T + t for the whole run (T = blockDim.x), so where each of its
+// populations comes from (a neighbour's slot, in this block or another one of
+// the cluster, or at a wall its own opposite population) is worked out once.
+// Arithmetic, rounding bits and results are k_step's.
+//
+// Most threads per block: the registers hold the source addresses and the
+// populations of one cell.  FP64 is kept to one warp per SM sub-partition
+// (see untuned_block).
+template <class L, class S> __host__ __device__ constexpr int resident_threads() {
+    return sizeof(typename Store<S>::R) == 8 ? 128 : L::Q == 9 ? 640 : 512;
+}
+constexpr int kResidentCluster = 16;    // blocks per cluster (non-portable above 8)
+
+template <class S> __device__ __forceinline__ typename Store<S>::R ld_cluster(uint32_t a) {
+    if constexpr (sizeof(S) == 8) {
+        double v;
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+        return v;
+    } else if constexpr (sizeof(S) == 4) {
+        float v;
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+        return v;
+    } else {
+        unsigned short v;
+        asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a));
+        if constexpr (std::is_same<S, __half>::value) return __half2float(__ushort_as_half(v));
+        else return __bfloat162float(__ushort_as_bfloat16(v));
+    }
+}
+// one barrier of the cluster's threads; the writes before it are visible after it
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" : : : "memory");
+}
+
+template <class L, int MODEL, class S>
+__global__ void __launch_bounds__(resident_threads<L, S>())
+k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ links,
+           typename Store<S>::R* __restrict__ tau, uint32_t* __restrict__ rng_ctr, int parity,
+           int nsteps) {
+    using R = typename Store<S>::R;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const KParams& kp = a.kp;
+    const int T = (int)blockDim.x, t = (int)threadIdx.x;
+    int idx = (int)blockIdx.x * T + t;
+    const bool inside = idx < kp.ncells;
+    const uint32_t lk = inside ? __ldg(links + idx) : kSolidBit;
+    const bool active = !(lk & kSolidBit);
+    step_begin(idx);
+    // element (i, n) of a block's buffer, as in a population buffer of T cells
+    auto elem = [&](int i, int n) { return (int)pop_base<S>(i, T) + pop_step<S>(i) * n; };
+    S* const buf = reinterpret_cast<S*>(smem);
+    const int half = L::Q * T;               // elements of one of the two buffers
+    if (inside) {
+        // both buffers: a solid or ghost cell is never stepped, but may be read
+        static_for<0, L::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            const S v = src[pop_base<S>(i, kp.plane) + (int64_t)pop_step<S>(i) * idx];
+            buf[elem(i, t)] = v;
+            buf[half + elem(i, t)] = v;
+        });
+    }
+    uint32_t from[L::Q];                     // shared::cluster address of each population's source
+    {
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        PullOffsets o{0, 0, 0, 0, 0, 0};
+        if (active) o = pull_offsets(kp, idx);
+        static_for<0, L::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            const bool wall = (lk >> i) & 1u;
+            const int n = active && !wall ? idx + o.template of<L, i>() : inside ? idx : 0;
+            const int b = n / T;
+            const uint32_t own = base + (uint32_t)(elem(wall ? L::opp(i) : i, n - b * T) * (int)sizeof(S));
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(from[i]) : "r"(own), "r"(b));
+        });
+    }
+    uint32_t seed = 0u;
+    if constexpr (Store<S>::kStochastic) seed = rng_ctr[parity];
+    R tc = R(0);
+    if constexpr (MODEL != LBM_MODEL_IR)
+        if (active) tc = tau[idx];
+    cluster_barrier();
+    uint32_t rd = 0u;                        // byte offset of the buffer this step reads
+    const uint32_t bytes = (uint32_t)half * (uint32_t)sizeof(S);
+    for (int k = 0; k < nsteps; ++k) {
+        if (active) {
+            R f[L::Q];
+            static_for<0, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                f[i] = ld_cluster<S>(from[i] + rd);
+            });
+            R drho, ur[3];
+            if constexpr (MODEL != LBM_MODEL_IR)
+                collide_pr<L, S, false>(coef<R>(a), kp.flags, f, tc, drho, ur);
+            else
+                collide_ir<L, S>(coef<R>(a), kp.flags, f, drho, ur);
+            uint32_t rnd = 0u;
+            if constexpr (Store<S>::kStochastic)
+                rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ ((seed + (uint32_t)k) * 0x9e3779b9u));
+            store_cell<L, S>(DstStride<S>{reinterpret_cast<S*>(smem + (bytes - rd)), T}, t, f, rnd);
+        }
+        rd = bytes - rd;
+        cluster_barrier();
+    }
+    if (active) {
+        const S* last = reinterpret_cast<const S*>(smem + rd);
+        static_for<0, L::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            dst[pop_base<S>(i, kp.plane) + (int64_t)pop_step<S>(i) * idx] = last[elem(i, t)];
+        });
+        if constexpr (MODEL != LBM_MODEL_IR) tau[idx] = tc;
+    }
+    if constexpr (Store<S>::kStochastic)
+        // as after nsteps launches: the counter of the buffer now current
+        if (blockIdx.x == 0 && t == 0) rng_ctr[parity ^ (nsteps & 1)] = seed + (uint32_t)nsteps;
 }
 
 // ---------------------------------------------------------------------------
@@ -2207,6 +2409,117 @@ inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, 
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// Threads per block and blocks of a resident run of ncells cells, and whether
+// the domain takes it (fits one cluster): small domains of FP32 arithmetic
+// share one block, larger ones spread over the cluster's 16 (D2Q9 F32 IR, us a
+// step: 256 cells in one block 0.55, 512 cells in one block 0.74, 640 cells in
+// 10 blocks 0.58).  Steps launched one by one take 1.35-1.55.
+template <class L, class S> inline bool resident_shape(int ncells, int& threads, int& blocks) {
+    constexpr int most = resident_threads<L, S>();
+    const int one = sizeof(typename Store<S>::R) == 8 ? 32 : L::Q == 9 ? 256 : 64;
+    const int per = ncells <= one ? ncells : (ncells + kResidentCluster - 1) / kResidentCluster;
+    threads = std::max((per + 31) / 32 * 32, sizeof(typename Store<S>::R) == 8 ? 32 : 64);
+    blocks = (ncells + threads - 1) / threads;
+    return threads <= most;
+}
+
+// Raises the kernel's limits (shared memory and blocks per cluster above the
+// defaults) and asks whether the device can hold its largest cluster; once per
+// instantiation.
+template <class L, int MODEL, class S> bool resident_ready() {
+    static const bool ready = [] {
+        auto kernel = k_resident<L, MODEL, S>;
+        constexpr int threads = resident_threads<L, S>();
+        constexpr int bytes = (int)sizeof(S) * 2 * L::Q * threads;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = kResidentCluster;
+        attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(kResidentCluster);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = bytes;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && clusters > 0;
+    }();
+    return ready;
+}
+
+template <class L, int MODEL, class S>
+cudaError_t launch_resident_t(const KParams& kp, const StepArgs& s, int nsteps, cudaStream_t st) {
+    using R = typename Store<S>::R;
+    auto kernel = k_resident<L, MODEL, S>;
+    int threads = 0, blocks = 0;
+    if (!resident_shape<L, S>(kp.ncells, threads, blocks)) return cudaErrorNotSupported;
+    const KArgs a = make_args<L>(kp);
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)blocks;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = sizeof(S) * 2 * L::Q * (size_t)threads;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, a, (const S*)s.fsrc, (S*)s.fdst, s.links, (R*)s.tau,
+                              s.rng_ctr, s.parity, nsteps);
+}
+
+template <class L, class S>
+cudaError_t launch_resident_model(int model, const KParams& kp, const StepArgs& s, int nsteps,
+                                  cudaStream_t st) {
+    if (model == LBM_MODEL_PR) return launch_resident_t<L, LBM_MODEL_PR, S>(kp, s, nsteps, st);
+    if constexpr (pair_form<S>()) return launch_resident_t<L, LBM_MODEL_IR, S>(kp, s, nsteps, st);
+    return cudaErrorNotSupported;
+}
+
+template <class L>
+cudaError_t launch_resident_lat(int model, int storage, const KParams& kp, const StepArgs& s,
+                                int nsteps, cudaStream_t st) {
+    switch (storage) {
+    case LBM_F32: return launch_resident_model<L, float>(model, kp, s, nsteps, st);
+    case LBM_F64: return launch_resident_model<L, double>(model, kp, s, nsteps, st);
+    case LBM_F16_OFS: return launch_resident_model<L, __half>(model, kp, s, nsteps, st);
+    case LBM_BF16_OFS: return launch_resident_model<L, __nv_bfloat16>(model, kp, s, nsteps, st);
+    default: return cudaErrorNotSupported;
+    }
+}
+
+// Left out: FP32 IR, whose class-sum collision the compiler contracts
+// differently here than in k_step (the other forms give the same bits), and the
+// Newton-implicit step.
+template <class L, class S> bool resident_fits_model(int model, int ncells) {
+    int threads = 0, blocks = 0;
+    if (!resident_shape<L, S>(ncells, threads, blocks)) return false;
+    if (model == kModelPRImplicit || (!pair_form<S>() && model == LBM_MODEL_IR)) return false;
+    if (model == LBM_MODEL_PR) return resident_ready<L, LBM_MODEL_PR, S>();
+    if constexpr (pair_form<S>()) return resident_ready<L, LBM_MODEL_IR, S>();
+    return false;
+}
+
+template <class L> bool resident_fits_lat(int model, int storage, int ncells) {
+    switch (storage) {
+    case LBM_F32: return resident_fits_model<L, float>(model, ncells);
+    case LBM_F64: return resident_fits_model<L, double>(model, ncells);
+    case LBM_F16_OFS: return resident_fits_model<L, __half>(model, ncells);
+    case LBM_BF16_OFS: return resident_fits_model<L, __nv_bfloat16>(model, ncells);
+    default: return false;
+    }
+}
+
 template <class L, int MODEL, class S, bool COPY>
 cudaError_t launch_step_c(bool check, const KParams& kp, const StepArgs& s, cudaStream_t st) {
     using R = typename Store<S>::R;
@@ -2536,5 +2849,17 @@ template <class L> void lattice_table(int* c, double* w) {
                                       double* partials, int threads, int cpt, cudaStream_t st) {\
         return launch_batch_lat<L>(model, storage, check, descs, block_dom, nblocks, grid,      \
                                    phase, partials, threads, cpt, st);                          \
+    }                                                                                           \
+    }
+
+// The resident runs of a lattice, in a translation unit of their own.
+#define BLBM_DEFINE_RESIDENT_LAUNCHERS(L)                                                      \
+    namespace blbm {                                                                            \
+    cudaError_t launch_resident_##L(int model, int storage, const KParams& kp,                 \
+                                    const StepArgs& a, int nsteps, cudaStream_t st) {           \
+        return launch_resident_lat<L>(model, storage, kp, a, nsteps, st);                       \
+    }                                                                                           \
+    bool resident_fits_##L(int model, int storage, int ncells) {                                \
+        return resident_fits_lat<L>(model, storage, ncells);                                           \
     }                                                                                           \
     }

@@ -181,10 +181,11 @@ lbm_status enter(const lbm_solver* s) {
     return LBM_OK;
 }
 
-cudaError_t launch_step(lbm_solver* s, bool check, cudaStream_t st) {
+// arguments of a launch that leaves the state in buffer cur ^ flip
+StepArgs step_args(const lbm_solver* s, int flip) {
     StepArgs a;
     a.fsrc = s->f[s->cur];
-    a.fdst = s->f[s->cur ^ 1];
+    a.fdst = s->f[s->cur ^ flip];
     a.links = s->links;
     a.tau = s->tau;
     a.usnap = s->usnap;
@@ -196,12 +197,39 @@ cudaError_t launch_step(lbm_solver* s, bool check, cudaStream_t st) {
     a.copy = s->copy;
     a.cellidx = s->cellidx;
     a.rank = s->rank;
+    return a;
+}
+
+cudaError_t launch_step(lbm_solver* s, bool check, cudaStream_t st) {
+    const StepArgs a = step_args(s, 1);
     const int km = kernel_model(s->p.model, s->kp.newton);
     switch (s->lat) {
     case LBM_D2Q9: return launch_step_D2Q9(km, s->p.storage, check, s->kp, a, st);
     case LBM_D3Q15: return launch_step_D3Q15(km, s->p.storage, check, s->kp, a, st);
     case LBM_D3Q19: return launch_step_D3Q19(km, s->p.storage, check, s->kp, a, st);
     default: return launch_step_D3Q27(km, s->p.storage, check, s->kp, a, st);
+    }
+}
+
+// nsteps plain steps in one launch (see k_resident)
+cudaError_t launch_resident(lbm_solver* s, int nsteps, cudaStream_t st) {
+    const StepArgs a = step_args(s, nsteps & 1);
+    const int km = kernel_model(s->p.model, s->kp.newton);
+    switch (s->lat) {
+    case LBM_D2Q9: return launch_resident_D2Q9(km, s->p.storage, s->kp, a, nsteps, st);
+    case LBM_D3Q15: return launch_resident_D3Q15(km, s->p.storage, s->kp, a, nsteps, st);
+    case LBM_D3Q19: return launch_resident_D3Q19(km, s->p.storage, s->kp, a, nsteps, st);
+    default: return launch_resident_D3Q27(km, s->p.storage, s->kp, a, nsteps, st);
+    }
+}
+
+bool resident_fits(const lbm_solver* s) {
+    const int km = kernel_model(s->p.model, s->kp.newton);
+    switch (s->lat) {
+    case LBM_D2Q9: return resident_fits_D2Q9(km, s->p.storage, s->ncells);
+    case LBM_D3Q15: return resident_fits_D3Q15(km, s->p.storage, s->ncells);
+    case LBM_D3Q19: return resident_fits_D3Q19(km, s->p.storage, s->ncells);
+    default: return resident_fits_D3Q27(km, s->p.storage, s->ncells);
     }
 }
 
@@ -682,6 +710,8 @@ void apply_tuning(lbm_solver* s) {
     if (s->tune_version == ver) return;
     Shape sh = tune_lookup(s->lat, s->p.model, s->p.storage, s->ncells);
     if (!sh.set) sh.block = untuned_block(s);
+    // an entry of the table keeps its launch shape
+    s->resident = !sh.set && !s->rank && resident_fits(s);
     if (sh.block != s->block || sh.cpt != s->cpt) {
         for (int k = 0; k < 2; ++k)
             if (s->graph[k]) {
@@ -751,6 +781,10 @@ lbm_status lbm_tuning_clear(void) {
     return LBM_OK;
 }
 
+// Steps of one resident run: fewer cost more in loading and storing the state
+// than they save; more only make one launch long (2048 steps: 1-8 ms).
+static constexpr int kResidentMin = 4, kResidentMax = 2048;
+
 lbm_status lbm_step(lbm_solver* s, int64_t nsteps) {
     lbm_status v = enter(s);
     if (v != LBM_OK) return v;
@@ -764,6 +798,14 @@ lbm_status lbm_step(lbm_solver* s, int64_t nsteps) {
         if (k > 0) {
             const int64_t to_check = k - (s->steps % k);   // the to_check-th step from now is a check step
             plain = (to_check - 1 < left) ? to_check - 1 : left;
+        }
+        while (s->resident && plain >= kResidentMin) {
+            const int n = (int)std::min<int64_t>(plain, kResidentMax);
+            CK(s, launch_resident(s, n, s->stream), "resident run launch");
+            s->cur ^= n & 1;
+            s->steps += n;
+            plain -= n;
+            left -= n;
         }
         while (plain >= s->graph_len) {
             if (!s->graph[s->cur]) CK(s, build_graph(s, s->cur), "CUDA graph capture");

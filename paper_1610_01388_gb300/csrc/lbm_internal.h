@@ -87,6 +87,9 @@ struct BatchDesc;   // per-domain descriptor of a batched launch (kernels.cuh)
     cudaError_t launch_halo_##L(int storage, const KParams& kp, void* f, void* buf, int side,   \
                                 bool pack, cudaStream_t st);                                    \
     int face_count_##L();                                                                       \
+    cudaError_t launch_resident_##L(int model, int storage, const KParams& kp,                  \
+                                    const StepArgs& a, int nsteps, cudaStream_t st);            \
+    bool resident_fits_##L(int model, int storage, int ncells);                                 \
     cudaError_t launch_step_batch_##L(int model, int storage, bool check,                       \
                                       const struct BatchDesc* descs, const int* block_dom,      \
                                       int nblocks, int grid, int phase, double* partials,       \
