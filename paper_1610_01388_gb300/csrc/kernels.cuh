@@ -1704,7 +1704,7 @@ k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ lin
 // Compact layout (LBM_FLAG_COMPACT).  The population planes, the link words,
 // tau and the check-step snapshot hold the stepped fluid cells only: slot k is
 // the k-th fluid cell in cell-index order, cellidx[k] its cell index, and
-// rank[n] the slot of cell n (-1 for a solid cell).  One thread per slot, so
+// rank[n] the slot of cell n (negative for a solid cell).  One thread per slot, so
 // every lane of a warp is a fluid cell and every store fills whole sectors,
 // whereas on a porous medium the dense layout also moves the solid cells that
 // share a DRAM access with fluid ones.  The pull reads population i of the
@@ -1714,6 +1714,19 @@ k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ lin
 // dense step's (the same collision code, the same stochastic-rounding hash of
 // the cell index); compiled into another kernel, it may differ from it by the
 // compiler's multiply-add contraction, i.e. to round-off.
+//
+// rank[] is a running count: a fluid cell holds its slot, a solid cell ~n with
+// n the number of fluid cells before it.  Slots are in cell order, so along a
+// row the slots of the neighbours x - 1 and x + 1 follow from the word of the
+// cell between them (one less; one more if that cell is fluid), and a gather
+// reads one word per neighbouring row, 8 (D3Q15, D3Q19, D3Q27) instead of 14,
+// 18 and 26.  The wrap in x is the exception: a warp that holds a cell at
+// either end of a row looks every neighbour up.
+template <class L> __host__ __device__ constexpr int dir_index(int cx, int cy, int cz) {
+    for (int i = 0; i < L::Q; ++i)
+        if (L::cx(i) == cx && L::cy(i) == cy && L::cz(i) == cz) return i;
+    return -1;
+}
 template <class L, class S, class Src>
 __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, uint32_t lk,
                                                int idx, int slot, const int* __restrict__ rank,
@@ -1724,11 +1737,47 @@ __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, 
     // faster steps on 256^3 porous boxes)
     const int* __restrict__ rk = rank + idx;
     v[0] = Store<S>::template ld<L, 0>(P.template at<0>(slot));
-    if (__all_sync(__activemask(), lk == 0u)) {
-        static_for<1, L::Q>([&](auto I) {
+    const bool edge = o.dxm != -1 || o.dxp != 1;   // the x neighbours wrap
+    const unsigned warp = __activemask();
+    // by rows (cy, cz): f(direction, slot of its source if that is fluid)
+    auto rows = [&](bool solid_free, auto&& f) {
+        static_for<0, 9>([&](auto J) {
+            constexpr int cy = decltype(J)::value % 3 - 1, cz = decltype(J)::value / 3 - 1;
+            constexpr int im = dir_index<L>(1, cy, cz), i0 = dir_index<L>(0, cy, cz),
+                          ip = dir_index<L>(-1, cy, cz);
+            if constexpr (im >= 0 || i0 >= 0 || ip >= 0) {
+                int c = slot, after = slot + 1;
+                if constexpr (cy != 0 || cz != 0) {
+                    int off = 0;
+                    if constexpr (cy > 0) off += o.dym;
+                    if constexpr (cy < 0) off += o.dyp;
+                    if constexpr (cz > 0) off += o.dzm;
+                    if constexpr (cz < 0) off += o.dzp;
+                    c = __ldg(rk + off);
+                    if (i0 >= 0 && solid_free) {     // the row's own cell is a source, hence fluid
+                        after = c + 1;
+                    } else {
+                        const int s = c >> 31;       // -1 for a solid cell
+                        c ^= s;
+                        after = c + 1 + s;
+                    }
+                }
+                if constexpr (im >= 0) f(std::integral_constant<int, im>{}, c - 1);
+                if constexpr (i0 > 0) f(std::integral_constant<int, i0>{}, c);
+                if constexpr (ip >= 0) f(std::integral_constant<int, ip>{}, after);
+            }
+        });
+    };
+    if (__all_sync(warp, lk == 0u && !edge)) {
+        rows(true, [&](auto I, int k) {
             constexpr int i = decltype(I)::value;
-            const int k = __ldg(rk + o.template of<L, i>());
             v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
+        });
+    } else if (__all_sync(warp, !edge)) {
+        rows(false, [&](auto I, int k) {
+            constexpr int i = decltype(I)::value;
+            const S* p = ((lk >> i) & 1u) ? P.template at<L::opp(i)>(slot) : P.template at<i>(k);
+            v[i] = Store<S>::template ld<L, i>(p);   // opposite planes share w_i
         });
     } else {
         static_for<1, L::Q>([&](auto I) {
@@ -1738,7 +1787,7 @@ __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, 
                 p = P.template at<L::opp(i)>(slot);
             else
                 p = P.template at<i>(__ldg(rk + o.template of<L, i>()));
-            v[i] = Store<S>::template ld<L, i>(p);   // opposite planes share w_i
+            v[i] = Store<S>::template ld<L, i>(p);
         });
     }
 }

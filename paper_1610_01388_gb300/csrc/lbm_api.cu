@@ -9,7 +9,7 @@
 // (one slot each, in cell-index order; plane >= the fluid count), and two
 // more regions map between slots and cells:
 //   cellidx   cell index of each slot
-//   rank      slot of each cell, -1 for a solid cell
+//   rank      slot of each cell; for a solid cell ~n, n the fluid cells before it
 //   tau       PR relaxation time per cell, updated in place
 //   usnap     check-step velocity snapshot [3][plane]
 //   partials  per-block FP64 reduction partials
@@ -595,12 +595,12 @@ static lbm_status create_impl(lbm_solver** out, lbm_lattice lat, int nx, int ny,
         s->cellidx = (int*)(s->base + s->lay.off_cellidx);
         s->rank = (int*)(s->base + s->lay.off_rank);
         h_cellidx.reserve((size_t)s->nfluid);
-        h_rank.assign((size_t)s->ncells, -1);
-        for (int i = 0; i < s->ncells; ++i)
-            if (stepped(i)) {
-                h_rank[i] = (int)h_cellidx.size();
-                h_cellidx.push_back(i);
-            }
+        h_rank.resize((size_t)s->ncells);
+        for (int i = 0; i < s->ncells; ++i) {
+            h_rank[i] = (int)h_cellidx.size();
+            if (stepped(i)) h_cellidx.push_back(i);
+            else h_rank[i] = ~h_rank[i];
+        }
     }
 
     lbm_status rc = LBM_OK;

@@ -59,7 +59,7 @@ struct StepArgs {
     int cpt;             // cells per thread of plain steps (1, or 2 with block 128 / 256)
     int copy;            // 16-bit PR: solid cells of mixed groups copy through (geometry choice)
     const int* cellidx;  // compact layout: cell index of each slot (nullptr: dense layout)
-    const int* rank;     // compact layout: slot of each cell, -1 for solid cells
+    const int* rank;     // compact layout: slot of each cell, negative for solid cells
 };
 
 enum ReduceMode { kReduceFlow = 0, kReduceTotals = 1 };

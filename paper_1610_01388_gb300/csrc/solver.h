@@ -49,7 +49,7 @@ struct lbm_solver {
     void* f[2] = {nullptr, nullptr};   // population buffers; f[cur] is the state
     uint32_t* links = nullptr;         // per cell, or per slot in the compact layout
     int* cellidx = nullptr;            // compact layout: cell index of each slot
-    int* rank = nullptr;               // compact layout: slot of each cell (-1: solid)
+    int* rank = nullptr;               // compact layout: slot of each cell (negative: solid)
     void* tau = nullptr;
     void* usnap = nullptr;
     double* partials = nullptr;
