@@ -32,9 +32,9 @@ constexpr int kFlowChangeSlot = kStatFlowChange;
 static_assert(kFlowChangeSlot == kNumStats - 1 && kStatNonFinite < kFlowChangeSlot,
               "the flow change takes the stats row's last entry, which check steps leave at 0");
 constexpr int kGraphLen = 16;       // steps per captured graph (even)
-// What a captured graph holds: kGraphLen plain steps, one plain step, or one
-// check step.  The last two exist for concurrent groups only.
-enum { kGraphRun = 0, kGraphOne, kGraphCheck, kGraphKinds };
+// Captured graphs, by the plain steps they hold (1..kGraphLen); 0 is a check
+// step.  Only concurrent groups have the ones below kGraphLen.
+constexpr int kGraphCheck = 0;
 
 // Per domain: the fixed-order sum of its tiles' partials into its stats row,
 // and in the row's last entry the relative change of the flow-rate vector
@@ -133,10 +133,24 @@ std::atomic<uint64_t> g_sched_version{1};
 
 int sched_key(int lat, int model, int storage) { return (lat * 4 + model) * 8 + storage; }
 
-int sched_ctas(int lat, int model, int storage) {
+// unset: what to return where the schedule has no entry
+int sched_ctas(int lat, int model, int storage, int unset = 0) {
     std::lock_guard<std::mutex> lk(g_sched_mu);
     auto it = g_sched_ctas.find(sched_key(lat, model, storage));
-    return it == g_sched_ctas.end() ? 0 : it->second;
+    return it == g_sched_ctas.end() ? unset : it->second;
+}
+
+// Resident CTAs per SM that concurrent groups without a schedule entry share
+// out by the bytes of their steps, at least one each.  With one CTA per tile a
+// large group's blocks, and those of its next step that already wait for it,
+// keep the other groups off the SMs (48 domains of the serving mix, us per step:
+// 52 with a CTA per tile, 42 shared out).
+constexpr int kSharedCtas = 8;
+
+// bytes a group's plain step moves at least
+double step_bytes(const lbm_solver* s) {
+    return (double)s->nfluid * (2.0 * s->Q * storage_bytes(s->p.storage) +
+                                (s->p.model == LBM_MODEL_PR ? 2.0 * arith_bytes(s->p.storage) : 0.0));
 }
 
 // size class of a group: floor(log2) of its domains' mean cell count
@@ -196,7 +210,7 @@ struct lbm_batch {
     double* d_slots = nullptr;      // [kMaxSlots][kNumStats]
     double* h_slots = nullptr;      // pinned mirror
     bool dirty = true;
-    cudaGraphExec_t graph[kGraphKinds][2] = {};   // by kind and phase
+    cudaGraphExec_t graph[kGraphLen + 1][2] = {};   // by content and phase
     int rows = 0;                         // stats rows in use: [0, rows)
     bool poisoned = false;
     int sms = 1;                          // multiprocessors of the device
@@ -239,8 +253,8 @@ lbm_status benter(const lbm_batch* b) {
 }
 
 void drop_graphs(lbm_batch* b) {
-    for (auto& kind : b->graph)
-        for (auto& g : kind)
+    for (auto& content : b->graph)
+        for (auto& g : content)
             if (g) {
                 cudaGraphExecDestroy(g);
                 g = nullptr;
@@ -294,6 +308,9 @@ lbm_status rebuild(lbm_batch* b) {
             if (o.d_pblock_dom) cudaFreeAsync(o.d_pblock_dom, b->stream);
             cudaFreeAsync(o.d_partials, b->stream);
         }
+    double all_bytes = 0.0;
+    for (const auto& kv : b->doms) all_bytes += step_bytes(kv.second.s);
+    const bool share = b->concurrent && b->groups.size() > 1;
     for (auto& g : b->groups) {
         std::vector<BatchDesc> desc(g.ids.size());
         std::vector<int> bd, pbd;
@@ -335,7 +352,10 @@ lbm_status rebuild(lbm_batch* b) {
         }
         g.nblocks = blocks;
         g.pnblocks = pblocks;
-        const int ctas = sched_ctas(g.lat, g.user_model, g.storage);
+        double bytes = 0.0;
+        for (int64_t id : g.ids) bytes += step_bytes(b->doms[id].s);
+        const int part = share ? std::max(1, (int)std::lround(kSharedCtas * bytes / all_bytes)) : 0;
+        const int ctas = sched_ctas(g.lat, g.user_model, g.storage, part);
         g.grid = ctas > 0 ? std::min(blocks, ctas * b->sms) : blocks;
         g.pgrid = ctas > 0 ? std::min(pblocks, ctas * b->sms) : pblocks;
         if ((int)desc.size() > g.cap_desc) {
@@ -389,7 +409,7 @@ cudaError_t launch_all(lbm_batch* b, bool check, cudaStream_t st) {
 // their step chains need no order between them.  Every forked branch is
 // joined back into the origin stream, also after an error, so the capture
 // can always be ended.
-cudaError_t capture_branches(lbm_batch* b, int kind, int par, int active) {
+cudaError_t capture_branches(lbm_batch* b, int content, int par, int active) {
     cudaError_t e = cudaSuccess;
     if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     while (e == cudaSuccess && (int)b->branch.size() < active) {
@@ -408,9 +428,9 @@ cudaError_t capture_branches(lbm_batch* b, int kind, int par, int active) {
         if (g.ids.empty()) continue;
         cudaStream_t st = b->branch[k];
         cudaError_t eb = cudaStreamWaitEvent(st, b->fork, 0);
-        const int steps = kind == kGraphRun ? kGraphLen : 1;
+        const int steps = content == kGraphCheck ? 1 : content;
         for (int t = 0; t < steps && eb == cudaSuccess; ++t)
-            eb = launch_group(b, g, kind == kGraphCheck, par ^ (t & 1), st);
+            eb = launch_group(b, g, content == kGraphCheck, par ^ (t & 1), st);
         cudaError_t ej = cudaEventRecord(b->join[k], st);
         if (ej == cudaSuccess) ej = cudaStreamWaitEvent(b->cap, b->join[k], 0);
         if (e == cudaSuccess) e = eb != cudaSuccess ? eb : ej;
@@ -419,7 +439,7 @@ cudaError_t capture_branches(lbm_batch* b, int kind, int par, int active) {
     return e;
 }
 
-cudaError_t capture(lbm_batch* b, int kind, int par) {
+cudaError_t capture(lbm_batch* b, int content, int par) {
     if (!b->cap) {
         cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
         if (e != cudaSuccess) return e;
@@ -434,8 +454,8 @@ cudaError_t capture(lbm_batch* b, int kind, int par) {
     int active = 0;
     for (const auto& g : b->groups) active += !g.ids.empty();
     if (b->concurrent && active > 1) {
-        e = capture_branches(b, kind, par, active);
-    } else {   // kGraphRun
+        e = capture_branches(b, content, par, active);
+    } else {   // kGraphLen plain steps
         for (int t = 0; t < kGraphLen && e == cudaSuccess; ++t) {
             e = launch_all(b, false, b->cap);
             b->phase ^= 1;
@@ -449,7 +469,7 @@ cudaError_t capture(lbm_batch* b, int kind, int par) {
         return e;
     }
     if (e2 != cudaSuccess) return e2;
-    e = cudaGraphInstantiate(&b->graph[kind][par], g, 0);
+    e = cudaGraphInstantiate(&b->graph[content][par], g, 0);
     cudaGraphDestroy(g);
     return e;
 }
@@ -568,10 +588,10 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     int active = 0;
     for (const auto& g : b->groups) active += !g.ids.empty();
     const bool branches = b->concurrent && active > 1;
-    // one launch of a graph of this kind, at the current phase
-    auto replay = [&](int kind) {
-        cudaGraphExec_t& g = b->graph[kind][b->phase];
-        if (!g) BCK(b, capture(b, kind, b->phase), "batch graph capture");
+    // one launch of the graph with this content, at the current phase
+    auto replay = [&](int content) {
+        cudaGraphExec_t& g = b->graph[content][b->phase];
+        if (!g) BCK(b, capture(b, content, b->phase), "batch graph capture");
         BCK(b, cudaGraphLaunch(g, b->stream), "batch graph launch");
         return LBM_OK;
     };
@@ -580,17 +600,21 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
         const int64_t to_check = b->k - (b->gstep % b->k);
         int64_t plain = std::min(to_check - 1, left);
         while (plain >= kGraphLen) {
-            if ((v = replay(kGraphRun)) != LBM_OK) return v;
+            if ((v = replay(kGraphLen)) != LBM_OK) return v;
             b->gstep += kGraphLen;          // even: the phase is unchanged
             plain -= kGraphLen;
             left -= kGraphLen;
         }
+        if (branches && plain > 0) {
+            const int rest = (int)plain;
+            if ((v = replay(rest)) != LBM_OK) return v;
+            b->phase ^= rest & 1;
+            b->gstep += rest;
+            left -= rest;
+            plain = 0;
+        }
         while (plain > 0) {
-            if (branches) {
-                if ((v = replay(kGraphOne)) != LBM_OK) return v;
-            } else {
-                BCK(b, launch_all(b, false, b->stream), "batch step");
-            }
+            BCK(b, launch_all(b, false, b->stream), "batch step");
             b->phase ^= 1;
             b->gstep += 1;
             --plain;
