@@ -221,6 +221,45 @@ __device__ __forceinline__ F2 sub(F2 a, F2 b) { return f2_sub(a, b); }
 __device__ __forceinline__ F2 mul(F2 a, F2 b) { return f2_mul(a, b); }
 __device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return f2_fma(a, b, c); }
 
+// Reciprocal and (reciprocal) square root of the pair-form collision: the
+// hardware's approximation refined by the residual of its defining equation.
+// With e = 1 - x r, 1 / x = r (1 + e + e^2 + ...); with e = 1 - x r^2, 1 / sqrt(x)
+// = r (1 + e/2 + 3/8 e^2 + ...).  FP32 starts within 2^-23 (one term of the
+// first series makes it correct to an ulp; the roots are used as they are);
+// FP64 starts within 2^-19 and takes two terms, 3 and 5 operations on the FP64
+// pipe where the division and the root take 9 to 10.  Arguments are normal
+// numbers (callers guard the rest).
+__device__ __forceinline__ float rcp(float x) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return mad(r, mad(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = mad(-x, r, 1.0);
+    return mad(r, mad(e, e, e), r);
+}
+__device__ __forceinline__ F2 rcp(F2 x) { return F2(rcp(x.lo()), rcp(x.hi())); }
+__device__ __forceinline__ float rcp_root(float x) {
+    float r;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ double rcp_root(double x) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = mad(-mul(x, r), r, 1.0);
+    return mad(mul(r, e), mad(0.375, e, 0.5), r);
+}
+__device__ __forceinline__ float root(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// (below 1e-290 the root counts as 0: the flush to zero of its start)
+__device__ __forceinline__ double root(double x) { return x > 1e-290 ? mul(x, rcp_root(x)) : 0.0 * x; }
+
 // ---------------------------------------------------------------------------
 // storage.  R is the arithmetic type.  ld / st move population i between
 // memory and registers; enc / dec convert full FP64 populations at the ABI
@@ -691,38 +730,37 @@ __device__ __forceinline__ Mom<R> moments(R (&f)[L::Q]) {
     }
 }
 
-// a_i b_j of two parallel vectors (symmetric)
-template <class L, class R>
-__device__ __forceinline__ Tens<R> outer(R ax, R ay, R az, R bx, R by, R bz) {
+// Pi - c_s^2 rho I written with offsets: Pi = c_s^2 I + p, rho = 1 + d.
+template <class L, class R> __device__ __forceinline__ Tens<R> dynamic(const Mom<R>& m) {
+    const R third = R(-1.0 / 3.0);
     Tens<R> t;
-    t.xx = mul(ax, bx);
-    t.yy = mul(ay, by);
-    t.xy = mul(ax, by);
+    t.xx = mad(m.d, third, m.xx);
+    t.yy = mad(m.d, third, m.yy);
+    t.xy = m.xy;
+    t.zz = R(0);
+    t.xz = R(0);
+    t.yz = R(0);
     if constexpr (L::D == 3) {
-        t.zz = mul(az, bz);
-        t.xz = mul(ax, bz);
-        t.yz = mul(ay, bz);
-    } else {
-        t.zz = R(0);
-        t.xz = R(0);
-        t.yz = R(0);
+        t.zz = mad(m.d, third, m.zz);
+        t.xz = m.xz;
+        t.yz = m.yz;
     }
     return t;
 }
 
-// Non-equilibrium second moment T = Pi - rho c_s^2 I - rho u u written with
-// offsets: Pi = c_s^2 I + p, rho = 1 + d.  ruu = rho u u.
+// Non-equilibrium second moment T = Pi - rho c_s^2 I - rho u u, from the first
+// two terms P, p = -rho u and u.
 template <class L, class R>
-__device__ __forceinline__ Tens<R> noneq(const Mom<R>& m, const Tens<R>& ruu, uint32_t flags) {
-    const R third = R(-1.0 / 3.0);
+__device__ __forceinline__ Tens<R> noneq(const Tens<R>& P, R px, R py, R pz, R ux, R uy, R uz,
+                                         uint32_t flags) {
     Tens<R> t;
-    t.xx = sub(mad(m.d, third, m.xx), ruu.xx);
-    t.yy = sub(mad(m.d, third, m.yy), ruu.yy);
-    t.xy = sub(m.xy, ruu.xy);
+    t.xx = mad(px, ux, P.xx);
+    t.yy = mad(py, uy, P.yy);
+    t.xy = mad(px, uy, P.xy);
     if constexpr (L::D == 3) {
-        t.zz = sub(mad(m.d, third, m.zz), ruu.zz);
-        t.xz = sub(m.xz, ruu.xz);
-        t.yz = sub(m.yz, ruu.yz);
+        t.zz = mad(pz, uz, P.zz);
+        t.xz = mad(px, uz, P.xz);
+        t.yz = mad(py, uz, P.yz);
     } else {
         t.zz = R(0);
         t.xz = R(0);
@@ -753,10 +791,10 @@ template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t)
 // members of a family differ only by the signs of the off-diagonal terms: one
 // sum per axis pair, two per face plane, one 4-point butterfly for the
 // corners, instead of c.u, its square and c.T.c per pair (D3Q27: 23 adds
-// against 150 operations).  put(i, e, we, cq, wo) stores pair i, its even part
-// we e and its odd part wo cq.  Where w_i in memory units is the same for
+// against 150 operations).  put(i, e, cq, wo) stores pair i, its even part e
+// (weighted) and its odd part wo cq.  Where w_i in memory units is the same for
 // every direction (the 16-bit forms) it goes into the six numbers and q once,
-// and we = wo = 1.
+// and wo = 1.
 template <class L, class S, class R, class Put>
 __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R qz, Put&& put) {
     constexpr int F = Fam<L>::face, C = Fam<L>::corner;
@@ -770,38 +808,47 @@ __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R
         qy = scale(o0, qy);
         if constexpr (L::D == 3) qz = scale(o0, qz);
     }
-    const R k = R(same ? B(4.5) * g0 : B(4.5));
-    const R k2 = R(same ? B(9) * g0 : B(9));
+#define BLBM_I(n) std::integral_constant<int, (n)>{}
+    // Even parts carry their weights: per family gam enters e0's sums once (the
+    // axis family through its constants) and the off-diagonal terms' constant.
+    constexpr B gA = same ? B(1) : Store<S>::template gam<L, 1>();
+    constexpr B gF = same ? B(1) : Store<S>::template gam<L, (F ? F : 1)>();
+    constexpr B gC = same ? B(1) : Store<S>::template gam<L, (C ? C : 1)>();
+    constexpr B unit = same ? g0 : B(1);
+    const R k = R(B(4.5) * unit), kA = R(B(4.5) * gA * unit);
+    const R kF = R(B(9) * gF * unit), kC = R(B(9) * gC * unit);
     auto pair = [&](auto I, R e, R cq) {
         constexpr int i = decltype(I)::value;
-        if constexpr (same) put(I, e, B(1), cq, B(1));
-        else put(I, e, Store<S>::template gam<L, i>(), cq, Store<S>::template god<L, i>());
+        if constexpr (same) put(I, e, cq, B(1));
+        else put(I, e, cq, Store<S>::template god<L, i>());
     };
-#define BLBM_I(n) std::integral_constant<int, (n)>{}
+    const R eA = scale(gA, e0);
+    pair(BLBM_I(1), mad(kA, N.xx, eA), qx);
+    pair(BLBM_I(3), mad(kA, N.yy, eA), qy);
     const R ex = mad(k, N.xx, e0);
-    pair(BLBM_I(1), ex, qx);
-    pair(BLBM_I(3), mad(k, N.yy, e0), qy);
     const R exy = mad(k, N.yy, ex);
-    const R bxy = mul(k2, N.xy);
     const R qxpy = add(qx, qy), qxmy = sub(qx, qy);
     if constexpr (L::D == 2) {
-        pair(BLBM_I(F), add(exy, bxy), qxpy);
-        pair(BLBM_I(F + 2), sub(exy, bxy), qxmy);
+        const R s = scale(gF, exy), b = mul(kF, N.xy);
+        pair(BLBM_I(F), add(s, b), qxpy);
+        pair(BLBM_I(F + 2), sub(s, b), qxmy);
     } else {
-        const R bxz = mul(k2, N.xz), byz = mul(k2, N.yz);
+        pair(BLBM_I(5), mad(kA, N.zz, eA), qz);
         const R ez = mad(k, N.zz, e0);
-        pair(BLBM_I(5), ez, qz);
         if constexpr (F != 0) {
-            pair(BLBM_I(F), add(exy, bxy), qxpy);
-            pair(BLBM_I(F + 2), sub(exy, bxy), qxmy);
-            const R exz = mad(k, N.zz, ex), eyz = mad(k, N.yy, ez);
-            pair(BLBM_I(F + 4), add(exz, bxz), add(qx, qz));
-            pair(BLBM_I(F + 6), sub(exz, bxz), sub(qx, qz));
-            pair(BLBM_I(F + 8), add(eyz, byz), add(qy, qz));
-            pair(BLBM_I(F + 10), sub(eyz, byz), sub(qy, qz));
+            const R sxy = scale(gF, exy), bxy = mul(kF, N.xy);
+            pair(BLBM_I(F), add(sxy, bxy), qxpy);
+            pair(BLBM_I(F + 2), sub(sxy, bxy), qxmy);
+            const R sxz = scale(gF, mad(k, N.zz, ex)), bxz = mul(kF, N.xz);
+            pair(BLBM_I(F + 4), add(sxz, bxz), add(qx, qz));
+            pair(BLBM_I(F + 6), sub(sxz, bxz), sub(qx, qz));
+            const R syz = scale(gF, mad(k, N.yy, ez)), byz = mul(kF, N.yz);
+            pair(BLBM_I(F + 8), add(syz, byz), add(qy, qz));
+            pair(BLBM_I(F + 10), sub(syz, byz), sub(qy, qz));
         }
         if constexpr (C != 0) {
-            const R e = mad(k, N.zz, exy);
+            const R e = scale(gC, mad(k, N.zz, exy));
+            const R bxy = mul(kC, N.xy), bxz = mul(kC, N.xz), byz = mul(kC, N.yz);
             const R ep = add(e, byz), em = sub(e, byz), bp = add(bxy, bxz), bm = sub(bxy, bxz);
             pair(BLBM_I(C), add(ep, bp), add(qxpy, qz));
             pair(BLBM_I(C + 2), add(em, bm), sub(qxpy, qz));
@@ -826,8 +873,9 @@ __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R
         const Sc t2 = Lanes<R>::get(tn2, k);
         as[k] = Sc(0);
         asg[k] = Sc(-1);
-        if (t2 > Sc(0) && t2 >= c.s2y2) {
-            const Sc it = rsqrt(t2);
+        // (an FP64 |T| below 1e-145 counts as not yielded: see rcp_root)
+        if (t2 > Sc(sizeof(Sc) == 8 ? 1e-290 : 0.0) && t2 >= c.s2y2) {
+            const Sc it = rcp_root(t2);
             as[k] = mad(c.ir_as, it, -c.ir_a);
             asg[k] = mad(-c.ir_bs, it, -c.ir_bn);
         }
@@ -844,7 +892,7 @@ __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc
                                            R (&f)[L::Q], R& drho, R (&ur)[3]) {
     const Mom<R> m = moments<L, S, R>(f);
     const R rho = add(R(1), m.d);
-    const R inv = recip(rho);
+    const R inv = rcp(rho);
     const R gx = R(c.g[0]), gy = R(c.g[1]);
     R gz = R(0);
     if constexpr (L::D == 3) gz = R(c.g[2]);
@@ -855,35 +903,36 @@ __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc
     const R ux = mul(px, inv), uy = mul(py, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(pz, inv);
-    const Tens<R> U = outer<L, R>(px, py, pz, ux, uy, uz);
-    const Tens<R> T = noneq<L, R>(m, U, flags);
+    const Tens<R> P = dynamic<L, R>(m);
+    const Tens<R> T = noneq<L, R>(P, -px, -py, -pz, ux, uy, uz, flags);
     R as, asg;
     ir_yield<R>(c, square<L, R>(T), as, asg);
     // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I;
-    // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i
-    const R k1 = mad(R(0.5), as, -asg);
+    // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i,
+    // and rho u u = P - T
+    const R k1 = sub(mad(R(0.5), as, -asg), R(1));
     const R k2 = mul(asg, mul(trace<L, R>(T), R(1.0 / L::D)));
     Tens<R> N;
-    N.xx = add(U.xx, mad(k1, T.xx, k2));
-    N.yy = add(U.yy, mad(k1, T.yy, k2));
-    N.xy = mad(k1, T.xy, U.xy);
+    N.xx = mad(k1, T.xx, add(P.xx, k2));
+    N.yy = mad(k1, T.yy, add(P.yy, k2));
+    N.xy = mad(k1, T.xy, P.xy);
     N.zz = R(0);
     N.xz = R(0);
     N.yz = R(0);
     if constexpr (L::D == 3) {
-        N.zz = add(U.zz, mad(k1, T.zz, k2));
-        N.xz = mad(k1, T.xz, U.xz);
-        N.yz = mad(k1, T.yz, U.yz);
+        N.zz = mad(k1, T.zz, add(P.zz, k2));
+        N.xz = mad(k1, T.xz, P.xz);
+        N.yz = mad(k1, T.yz, P.yz);
     }
+    if (flags & LBM_FLAG_BURNETT_X) N.xx = add(mul(px, ux), k2);   // T.xx was dropped
     const R e0 = mad(R(-1.5), trace<L, R>(N), m.d);
     // odd part: w_i (3 rho c.u + 3/2 c.F) = 3 w_i c.(j + F), since rho u = j + F/2
     const R qx = mad(rho, gx, m.jx), qy = mad(rho, gy, m.jy);
     R qz = R(0);
     if constexpr (L::D == 3) qz = mad(rho, gz, m.jz);
     f[0] = scale(Store<S>::template gam<L, 0>(), e0);
-    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, auto we, R cq, auto wo) {
+    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
-        e = scale(we, e);
         f[i] = axpy(wo, cq, e);
         f[i + 1] = axpy(-wo, cq, e);
     });
@@ -968,13 +1017,15 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>&
     Sc tau_[Lanes<R>::n], wp_[Lanes<R>::n], wm_[Lanes<R>::n];
 #pragma unroll
     for (int k = 0; k < Lanes<R>::n; ++k) {
-        const Sc tt = mul(Sc(1.5), sqrt(mul(Sc(2), Lanes<R>::get(tn2, k))));
+        const Sc tt = mul(Sc(1.5), root(mul(Sc(2), Lanes<R>::get(tn2, k))));
         Sc gd = mul(Lanes<R>::get(itau, k), tt);
         const Sc sy_rho = mul(c.sigma_y, Lanes<R>::get(inv, k));
         if constexpr (IMPLICIT) gd = pr_newton(c, tt, gd, sy_rho);
         Sc nu;
         if (gd >= c.gdot_c) {
-            nu = add(c.nu_p, mul(sy_rho, -expm1(mul(-c.m, gd))) / gd);
+            const Sc y = mul(sy_rho, -expm1(mul(-c.m, gd)));
+            if (sizeof(Sc) == 4 || gd > Sc(1e-290)) nu = mad(y, rcp(gd), c.nu_p);
+            else nu = add(c.nu_p, y / gd);
         } else {
             const Sc nu0 = mad(c.m, sy_rho, c.nu_p);
             const Sc nuc = mad(sy_rho, c.e_c, c.nu_p);
@@ -986,12 +1037,12 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>&
         const Sc tm = sub(tn, Sc(0.5));
         const Sc odd = mad(Sc(0.5), tm, c.magic);
         if (sizeof(Sc) == 8 && tn < Sc(1e30)) {
-            const Sc r = recip(mul(tn, odd));
+            const Sc r = rcp(mul(tn, odd));
             wp_[k] = mul(r, odd);
             wm_[k] = mul(tm, mul(r, tn));
         } else {
-            wp_[k] = recip(tn);
-            wm_[k] = tm / odd;
+            wp_[k] = rcp(tn);
+            wm_[k] = mul(tm, rcp(odd));
         }
         tau_[k] = tn;
     }
@@ -1011,19 +1062,19 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     const R rho = add(R(1), m.d);
     R inv, itau;   // 1 / rho, 1 / tau_old
     if constexpr (sizeof(typename Lanes<R>::Sc) == 8) {
-        const R q = recip(mul(rho, tau));   // one FP64 division for both
+        const R q = rcp(mul(rho, tau));   // one FP64 reciprocal for both
         inv = mul(q, tau);
         itau = mul(q, rho);
     } else {
-        inv = recip(rho);
-        itau = recip(tau);
+        inv = rcp(rho);
+        itau = rcp(tau);
     }
     const R ux = mul(m.jx, inv), uy = mul(m.jy, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(m.jz, inv);
     R wp, wm;
     {
-        const Tens<R> T = noneq<L, R>(m, outer<L, R>(m.jx, m.jy, m.jz, ux, uy, uz), flags);
+        const Tens<R> T = noneq<L, R>(dynamic<L, R>(m), -m.jx, -m.jy, -m.jz, ux, uy, uz, flags);
         pair_pr_rates<IMPLICIT, R>(c, square<L, R>(T), inv, itau, tau, wp, wm);
     }
     const R gx = R(c.g[0]), gy = R(c.g[1]);
@@ -1062,9 +1113,9 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     R qz = R(0);
     if constexpr (L::D == 3) qz = mad(wm, m.jz, Fz);
     f[0] = axpy(Store<S>::template gam<L, 0>(), K0, mul(sub(R(1), wp), f[0]));
-    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, auto we, R cq, auto wo) {
+    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
-        const R E = mad(omp, f[i], scale(we, e));
+        const R E = mad(omp, f[i], e);
         const R O = mad(omm, f[i + 1], scale(wo, cq));
         f[i] = add(E, O);
         f[i + 1] = sub(E, O);
