@@ -291,10 +291,8 @@ cudaError_t do_step(lbm_solver* s, bool check, cudaStream_t st) {
     s->cur ^= 1;
     s->steps += 1;
     if (check) {
-        e = launch_finalize(s->partials, step_grid(held_cells(s)), s->stats, st);
-        if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(s->host_stats, s->stats, kNumStats * sizeof(double),
-                            cudaMemcpyDeviceToHost, st);
+        // straight into the pinned host copy
+        e = launch_finalize(s->partials, step_grid(held_cells(s)), s->host_stats, st);
         if (e != cudaSuccess) return e;
         s->checks += 1;
         s->last_check = s->steps;
@@ -332,43 +330,46 @@ cudaError_t build_graph(lbm_solver* s, int par) {
 
 namespace blbm {
 
-// Grid stage of the FP64 sums: one block of kFinThreads threads adds the
-// per-block partials in a fixed order (thread t takes partials t, t + kFinThreads,
-// ...; then a fixed shuffle tree).  1024 threads keep each thread's chain of
-// FP64 adds short, which matters at GB300's FP64 rate.
+// Grid stage of the FP64 sums: block k adds the per-block partials of stat k in
+// a fixed order (thread t takes partials t, t + kFinThreads, ...; then a fixed
+// shuffle tree).  1024 threads keep each thread's chain of FP64 adds short, and
+// a block per stat keeps the adds off one SM's FP64 pipe, where a warp's add
+// takes 64 cycles of its sub-partition: one block for all eight stats took 50
+// us on 16,384 partials and 15 us on one.
 constexpr int kFinThreads = 1024;
 
 __global__ void __launch_bounds__(kFinThreads)
-k_finalize(const double* __restrict__ partials, int nparts, double* __restrict__ out) {
-    double v[kNumStats];
-#pragma unroll
-    for (int k = 0; k < kNumStats; ++k) v[k] = 0.0;
+k_finalize(const double* partials, int nparts, double* __restrict__ out) {
+    // launched over the tail of the kernel that writes the partials
+    asm volatile("griddepcontrol.wait;" : "+l"(partials) : : "memory");
+    const int k = blockIdx.x;
+    double v = 0.0;
     // unrolled so several partials are in flight; the order of the adds is unchanged
 #pragma unroll 4
-    for (int b = threadIdx.x; b < nparts; b += kFinThreads) {
-#pragma unroll
-        for (int k = 0; k < kNumStats; ++k) v[k] += partials[(int64_t)b * kNumStats + k];
-    }
-    __shared__ double sm[kFinThreads / 32][kNumStats];
+    for (int b = threadIdx.x; b < nparts; b += kFinThreads) v += partials[(int64_t)b * kNumStats + k];
+    __shared__ double sm[kFinThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < kNumStats; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-        for (int k = 0; k < kNumStats; ++k) sm[warp][k] = v[k];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) sm[warp] = v;
     __syncthreads();
     if (warp == 0) {
-        for (int k = 0; k < kNumStats; ++k) {
-            double t = (lane < kFinThreads / 32) ? sm[lane][k] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-            if (lane == 0) out[k] = t;
-        }
+        double t = (lane < kFinThreads / 32) ? sm[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) out[k] = t;
     }
 }
 
 cudaError_t launch_finalize(const double* partials, int nparts, double* out, cudaStream_t st) {
-    k_finalize<<<1, kFinThreads, 0, st>>>(partials, nparts, out);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kNumStats);
+    cfg.blockDim = dim3(kFinThreads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_finalize, partials, nparts, out);
 }
 
 template <class T>
