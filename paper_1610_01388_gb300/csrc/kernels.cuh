@@ -257,8 +257,14 @@ __device__ __forceinline__ float root(float x) {
     asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// a > b for numbers >= 0, whose bits order as integers: an FP64 compare would
+// take its turn on the FP64 pipe like an add
+__device__ __forceinline__ bool above(float a, float b) { return a > b; }
+__device__ __forceinline__ bool above(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
 // (below 1e-290 the root counts as 0: the flush to zero of its start)
-__device__ __forceinline__ double root(double x) { return x > 1e-290 ? mul(x, rcp_root(x)) : 0.0 * x; }
+__device__ __forceinline__ double root(double x) { return above(x, 1e-290) ? mul(x, rcp_root(x)) : 0.0; }
 
 // ---------------------------------------------------------------------------
 // storage.  R is the arithmetic type.  ld / st move population i between
@@ -359,9 +365,11 @@ template <class R> struct Coef {
     R ir_b;    // 1 / (1 + 6 nu_p)
     R six_nu;  // 6 nu_p
     R s2y2;    // 2 sigma_y^2, the square of the IR yield threshold
-    R ir_as;   // s2y ir_a
     R ir_bn;   // six_nu ir_b
     R ir_bs;   // s2y ir_b
+    R ir_k;    // ir_bn - ir_a / 2 - 1
+    R ir_ks;   // s2y (ir_a / 2 + ir_b)
+    R hg[3];   // g / 2
     int newton;  // PR: Newton iterations of the implicit tau update
     R cg[13];   // c_i . g of direction i = 2p + 1 (PR force terms of the class form), per pair p
     R cgg[13];  // (c_i . g)^2
@@ -860,27 +868,28 @@ __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R
 }
 
 // ---------------------------------------------------------------------------
-// IR yield solve, per cell: s = as T, sigma = asg T (eq. Vikh_sigmaS_tensor)
-// from |T|^2.  Both factors are linear in 1 / |T|: -(|T| - sqrt2 sigma_y) a / |T|
-// = sqrt2 sigma_y a / |T| - a, so one reciprocal square root is all it takes.
+// IR yield solve, per cell: with s = as T, sigma = asg T (eq. Vikh_sigmaS_tensor)
+// from |T|^2, returns k1 = as / 2 - asg - 1 and asg.  Both factors are linear in
+// 1 / |T| (-(|T| - sqrt2 sigma_y) a / |T| = sqrt2 sigma_y a / |T| - a), and so is
+// k1: one reciprocal square root and two multiply-adds.
 template <class R>
-__device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R tn2, R& as_out,
+__device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R tn2, R& k1_out,
                                          R& asg_out) {
     using Sc = typename Lanes<R>::Sc;
-    Sc as[Lanes<R>::n], asg[Lanes<R>::n];
+    Sc k1[Lanes<R>::n], asg[Lanes<R>::n];
 #pragma unroll
     for (int k = 0; k < Lanes<R>::n; ++k) {
         const Sc t2 = Lanes<R>::get(tn2, k);
-        as[k] = Sc(0);
+        k1[k] = Sc(0);
         asg[k] = Sc(-1);
         // (an FP64 |T| below 1e-145 counts as not yielded: see rcp_root)
-        if (t2 > Sc(sizeof(Sc) == 8 ? 1e-290 : 0.0) && t2 >= c.s2y2) {
+        if (above(t2, Sc(sizeof(Sc) == 8 ? 1e-290 : 0.0)) && !above(c.s2y2, t2)) {
             const Sc it = rcp_root(t2);
-            as[k] = mad(c.ir_as, it, -c.ir_a);
+            k1[k] = mad(c.ir_ks, it, c.ir_k);
             asg[k] = mad(-c.ir_bs, it, -c.ir_bn);
         }
     }
-    as_out = Lanes<R>::make(as);
+    k1_out = Lanes<R>::make(k1);
     asg_out = Lanes<R>::make(asg);
 }
 
@@ -896,21 +905,19 @@ __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc
     const R gx = R(c.g[0]), gy = R(c.g[1]);
     R gz = R(0);
     if constexpr (L::D == 3) gz = R(c.g[2]);
-    const R half = mul(R(0.5), rho);
-    const R px = mad(half, gx, m.jx), py = mad(half, gy, m.jy);   // rho u
+    const R px = mad(rho, R(c.hg[0]), m.jx), py = mad(rho, R(c.hg[1]), m.jy);   // rho u
     R pz = R(0);
-    if constexpr (L::D == 3) pz = mad(half, gz, m.jz);
+    if constexpr (L::D == 3) pz = mad(rho, R(c.hg[2]), m.jz);
     const R ux = mul(px, inv), uy = mul(py, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(pz, inv);
     const Tens<R> P = dynamic<L, R>(m);
     const Tens<R> T = noneq<L, R>(P, -px, -py, -pz, ux, uy, uz, flags);
-    R as, asg;
-    ir_yield<R>(c, square<L, R>(T), as, asg);
+    R k1, asg;   // k1 - 1 with the k1 below
+    ir_yield<R>(c, square<L, R>(T), k1, asg);
     // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I;
     // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i,
     // and rho u u = P - T
-    const R k1 = sub(mad(R(0.5), as, -asg), R(1));
     const R k2 = mul(asg, mul(trace<L, R>(T), R(1.0 / L::D)));
     Tens<R> N;
     N.xx = mad(k1, T.xx, add(P.xx, k2));
@@ -1017,14 +1024,14 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>&
     Sc tau_[Lanes<R>::n], wp_[Lanes<R>::n], wm_[Lanes<R>::n];
 #pragma unroll
     for (int k = 0; k < Lanes<R>::n; ++k) {
-        const Sc tt = mul(Sc(1.5), root(mul(Sc(2), Lanes<R>::get(tn2, k))));
+        const Sc tt = root(mul(Sc(4.5), Lanes<R>::get(tn2, k)));   // 1.5 sqrt(2 T:T)
         Sc gd = mul(Lanes<R>::get(itau, k), tt);
         const Sc sy_rho = mul(c.sigma_y, Lanes<R>::get(inv, k));
         if constexpr (IMPLICIT) gd = pr_newton(c, tt, gd, sy_rho);
         Sc nu;
-        if (gd >= c.gdot_c) {
+        if (!above(c.gdot_c, gd)) {
             const Sc y = mul(sy_rho, -expm1(mul(-c.m, gd)));
-            if (sizeof(Sc) == 4 || gd > Sc(1e-290)) nu = mad(y, rcp(gd), c.nu_p);
+            if (sizeof(Sc) == 4 || above(gd, Sc(1e-290))) nu = mad(y, rcp(gd), c.nu_p);
             else nu = add(c.nu_p, y / gd);
         } else {
             const Sc nu0 = mad(c.m, sy_rho, c.nu_p);
@@ -1036,7 +1043,7 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>&
         // 1 / tau_odd with tau_odd = 1/2 + Lambda / (tau - 1/2) is tm / odd
         const Sc tm = sub(tn, Sc(0.5));
         const Sc odd = mad(Sc(0.5), tm, c.magic);
-        if (sizeof(Sc) == 8 && tn < Sc(1e30)) {
+        if (sizeof(Sc) == 8 && !above(tn, Sc(1e30))) {
             const Sc r = rcp(mul(tn, odd));
             wp_[k] = mul(r, odd);
             wm_[k] = mul(tm, mul(r, tn));
@@ -1112,7 +1119,7 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     const R qx = mad(wm, m.jx, Fx), qy = mad(wm, m.jy, Fy);
     R qz = R(0);
     if constexpr (L::D == 3) qz = mad(wm, m.jz, Fz);
-    f[0] = axpy(Store<S>::template gam<L, 0>(), K0, mul(sub(R(1), wp), f[0]));
+    f[0] = axpy(Store<S>::template gam<L, 0>(), K0, mad(-wp, f[0], f[0]));
     pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
         const R E = mad(omp, f[i], e);
@@ -2445,14 +2452,18 @@ template <class R> inline Coef<R> make_coef(const KParams& kp) {
     c.inv_gc = (R)(1.0 / kp.gdot_c);
     c.e_c = (R)(kp.m * kp.gdot_c > 0.0 ? -expm1(-kp.m * kp.gdot_c) / kp.gdot_c : 0.0);
     c.magic = (R)kp.magic;
-    for (int d = 0; d < 3; ++d) c.g[d] = (R)kp.g[d];
+    for (int d = 0; d < 3; ++d) {
+        c.g[d] = (R)kp.g[d];
+        c.hg[d] = (R)(0.5 * kp.g[d]);
+    }
     const double s2y = 1.4142135623730951 * kp.sigma_y;
     c.s2y = (R)s2y;
     c.ir_a = (R)(1.0 / (0.5 + 3.0 * nu));
     c.ir_b = (R)(1.0 / (1.0 + 6.0 * nu));
     c.six_nu = (R)(6.0 * nu);
     c.s2y2 = (R)(2.0 * kp.sigma_y * kp.sigma_y);
-    c.ir_as = (R)(s2y / (0.5 + 3.0 * nu));
+    c.ir_k = (R)(6.0 * nu / (1.0 + 6.0 * nu) - 0.5 / (0.5 + 3.0 * nu) - 1.0);
+    c.ir_ks = (R)(s2y * (0.5 / (0.5 + 3.0 * nu) + 1.0 / (1.0 + 6.0 * nu)));
     c.ir_bn = (R)(6.0 * nu / (1.0 + 6.0 * nu));
     c.ir_bs = (R)(s2y / (1.0 + 6.0 * nu));
     c.newton = kp.newton;
