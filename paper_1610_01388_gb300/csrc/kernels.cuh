@@ -1780,23 +1780,39 @@ k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ lin
 // reads one word per neighbouring row, 8 (D3Q15, D3Q19, D3Q27) instead of 14,
 // 18 and 26.  The wrap in x is the exception: a warp that holds a cell at
 // either end of a row looks every neighbour up.
+//
+// ROWS = false leaves the row paths out.
+//
+// In the 16-bit forms, bound by issue, the link word says whether the cell
+// lies at any face of the box (kFaceBit); a warp without such cells needs no
+// coordinates, its rows being at constant offsets (D3Q19 256^3 porous box: IR
+// 248 -> 225 us, PR 281 -> 261).  In the FP32 IR step, bound by latency, that form
+// spilled (323 -> 332 us).
 template <class L> __host__ __device__ constexpr int dir_index(int cx, int cy, int cz) {
     for (int i = 0; i < L::Q; ++i)
         if (L::cx(i) == cx && L::cy(i) == cy && L::cz(i) == cz) return i;
     return -1;
 }
-template <class L, class S, class Src>
+template <class L, class S, bool ROWS = true, class Src>
 __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, uint32_t lk,
                                                int idx, int slot, const int* __restrict__ rank,
                                                typename Store<S>::R (&v)[L::Q]) {
-    const PullOffsets o = pull_offsets(kp, idx);
+    constexpr bool by_face = sizeof(S) == 2;
+    PullOffsets o{0, 0, 0, 0, 0, 0};
+    bool edge;   // this lane's cell keeps the warp from the row paths
+    if constexpr (by_face) {
+        edge = (lk & kFaceBit) != 0u;
+    } else {
+        o = pull_offsets(kp, idx);
+        edge = o.dxm != -1 || o.dxp != 1;   // the x neighbours wrap
+    }
     // the cell's own rank word: each neighbour's is one multiply-add from it
     // (against an add and a sign-extended 64-bit address per neighbour: 2-8 %
     // faster steps on 256^3 porous boxes)
     const int* __restrict__ rk = rank + idx;
     v[0] = Store<S>::template ld<L, 0>(P.template at<0>(slot));
-    const bool edge = o.dxm != -1 || o.dxp != 1;   // the x neighbours wrap
     const unsigned warp = __activemask();
+    const int nx = kp.nx, nxy = kp.nx * kp.ny;
     // by rows (cy, cz): f(direction, slot of its source if that is fluid)
     auto rows = [&](bool solid_free, auto&& f) {
         static_for<0, 9>([&](auto J) {
@@ -1807,10 +1823,14 @@ __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, 
                 int c = slot, after = slot + 1;
                 if constexpr (cy != 0 || cz != 0) {
                     int off = 0;
-                    if constexpr (cy > 0) off += o.dym;
-                    if constexpr (cy < 0) off += o.dyp;
-                    if constexpr (cz > 0) off += o.dzm;
-                    if constexpr (cz < 0) off += o.dzp;
+                    if constexpr (by_face) {
+                        off = -(cy * nx + cz * nxy);
+                    } else {
+                        if constexpr (cy > 0) off += o.dym;
+                        if constexpr (cy < 0) off += o.dyp;
+                        if constexpr (cz > 0) off += o.dzm;
+                        if constexpr (cz < 0) off += o.dzp;
+                    }
                     c = __ldg(rk + off);
                     if (i0 >= 0 && solid_free) {     // the row's own cell is a source, hence fluid
                         after = c + 1;
@@ -1826,25 +1846,35 @@ __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, 
             }
         });
     };
-    if (__all_sync(warp, lk == 0u && !edge)) {
+    if constexpr (!ROWS) edge = true;
+    if (ROWS && __all_sync(warp, lk == 0u && !edge)) {
         rows(true, [&](auto I, int k) {
             constexpr int i = decltype(I)::value;
             v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
         });
-    } else if (__all_sync(warp, !edge)) {
+    } else if (ROWS && __all_sync(warp, !edge)) {
         rows(false, [&](auto I, int k) {
             constexpr int i = decltype(I)::value;
             const S* p = ((lk >> i) & 1u) ? P.template at<L::opp(i)>(slot) : P.template at<i>(k);
             v[i] = Store<S>::template ld<L, i>(p);   // opposite planes share w_i
         });
     } else {
+        const PullOffsets w = by_face ? pull_offsets(kp, idx) : o;
+        if (!ROWS && __all_sync(warp, lk == 0u)) {
+            static_for<1, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                const int k = __ldg(rk + w.template of<L, i>());
+                v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
+            });
+            return;
+        }
         static_for<1, L::Q>([&](auto I) {
             constexpr int i = decltype(I)::value;
             const S* p;
             if ((lk >> i) & 1u)
                 p = P.template at<L::opp(i)>(slot);
             else
-                p = P.template at<i>(__ldg(rk + o.template of<L, i>()));
+                p = P.template at<i>(__ldg(rk + w.template of<L, i>()));
             v[i] = Store<S>::template ld<L, i>(p);
         });
     }
@@ -1865,7 +1895,11 @@ __device__ __forceinline__ void compact_cell(const KParams& kp, const Coef<typen
         for (int d = 0; d < 3; ++d) up[d] = usnap[(int64_t)d * kp.plane + slot];
     }
     R f[L::Q];
-    gather_compact<L, S>(kp, src, lk, idx, slot, rank, f);
+    // D3Q27 FP32 IR looks every neighbour up: beside the row paths the compiler
+    // contracts its class-sum collision differently, and its results would move
+    // by a rounding (124 us on the 160^3 porous box, 118 with the row paths)
+    constexpr bool rows = !(sizeof(S) == 4 && L::Q == 27 && MODEL == LBM_MODEL_IR);
+    gather_compact<L, S, rows>(kp, src, lk, idx, slot, rank, f);
     R drho, ur[3];
     if constexpr (MODEL != LBM_MODEL_IR) {
         R t = tau[slot];
@@ -1891,7 +1925,8 @@ template <class L, int MODEL, class S, bool CHECK> constexpr int compact_min_blo
     // the allocator's 38 registers.  D3Q27 IR: 4 blocks (64 registers; 48
     // spilled and ran slower).  PR keeps the dense step's budget (6 blocks
     // spilled and made the D3Q19 FP16 step 7 % slower).
-    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q <= 19 ? 6 : 4;
+    // 16-bit IR up to 19 velocities spills at 6 (its large domains run the loop).
+    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q == 27 ? 4 : sizeof(S) == 2 ? 5 : 6;
     return step_min_blocks<L, MODEL, S, CHECK, kBlock>();
 }
 
@@ -1906,9 +1941,9 @@ template <class L, int MODEL, class S, bool CHECK> constexpr int compact_min_blo
 #ifndef BLBM_COMPACT_BLOCK
 #define BLBM_COMPACT_BLOCK 0
 #endif
-template <class L, int MODEL> constexpr int compact_block() {
+template <class L, int MODEL, class S> constexpr int compact_block() {
     if (BLBM_COMPACT_BLOCK > 0) return BLBM_COMPACT_BLOCK;
-    if (MODEL != LBM_MODEL_IR) return 128;
+    if (MODEL != LBM_MODEL_IR || sizeof(S) == 2) return 128;
     return L::Q <= 19 ? 512 : 256;
 }
 
@@ -1955,26 +1990,27 @@ k_step_compact(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
 // slot, slot + stride, ... and loads the next slot's cell index and link word
 // before it steps the current one, so of the three dependent loads of a slot
 // (cell index, neighbour slots, populations) only the last two are on the
-// critical path.  It pays for the IR step of the 16-bit forms (256^3 porous
-// box, D3Q19 FP16: 306 -> 268 us).  The FP32 forms need more registers for it
-// than their budgets hold: IR spilled at 6 blocks per SM (417 us) and ran at
-// 391 us with 5, against 364 us for the one-slot kernel; PR gained nothing.
-template <int MODEL, class S> constexpr bool compact_loop() {
-    return MODEL == LBM_MODEL_IR && sizeof(S) == 2;
-}
-// (BLBM_COMPACT_LOOP_MINB overrides its register budget at build time.)
+// critical path.  It pays for the 16-bit forms.  The FP32 forms need more
+// registers for it than their budgets hold (D3Q19 IR, 256^3 porous box: 323 us
+// by one-slot threads, 349-386 by the loop).
+template <class S> constexpr bool compact_loop() { return sizeof(S) == 2; }
+// ... and for domains of several rounds of the grid only (D3Q19 PR FP16, 48^3
+// box: 3.4 us by one-slot threads, 4.1 by the loop).
+constexpr int kLoopRounds = 4;
+// Register budget in resident blocks (BLBM_COMPACT_LOOP_MINB overrides it at
+// build time), FP16, us at 4 / 5 / 6 blocks: D3Q19 256^3 porous box IR 235 / 225 /
+// 279 and PR 277 / 261 / 313; D3Q15 160^3 box PR 66 / 59 / 64; D3Q27 160^3 box PR
+// 88 / 99 / 120 and IR 79 / 91 / 106.
 #ifndef BLBM_COMPACT_LOOP_MINB
 #define BLBM_COMPACT_LOOP_MINB -1
 #endif
-// D3Q27: 4 blocks (64 registers; at 5 blocks it spills 68 bytes).
-template <class L, int MODEL, class S> constexpr int compact_loop_min_blocks() {
+template <class L> constexpr int compact_loop_min_blocks() {
     if (BLBM_COMPACT_LOOP_MINB >= 0) return BLBM_COMPACT_LOOP_MINB;
-    if (L::Q == 27) return 4;
-    return compact_min_blocks<L, MODEL, S, false>();
+    return L::Q == 27 ? 4 : 5;
 }
 
 template <class L, int MODEL, class S>
-__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L, MODEL, S>())
+__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L>())
 k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
                     const uint32_t* __restrict__ links, const int* __restrict__ cellidx,
                     const int* __restrict__ rank, typename Store<S>::R* __restrict__ tau,
@@ -2016,10 +2052,11 @@ k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> ds
 }
 
 // link words of the compact layout: slot k gets the bits of cell cellidx[k]
+// (face_bits: and kFaceBit, for the 16-bit forms)
 template <class L>
 __global__ void __launch_bounds__(kBlock)
 k_links_compact(const KParams kp, const uint8_t* __restrict__ mask,
-                const int* __restrict__ cellidx, uint32_t* __restrict__ links) {
+                const int* __restrict__ cellidx, uint32_t* __restrict__ links, bool face_bits) {
     const int slot = blockIdx.x * kBlock + threadIdx.x;
     if (slot >= kp.nslots) return;
     const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
@@ -2033,6 +2070,9 @@ k_links_compact(const KParams kp, const uint8_t* __restrict__ mask,
         const int zs = (z - L::cz(i) + nz) % nz;
         if (mask[xs + nx * (ys + ny * zs)]) bits |= 1u << i;
     }
+    if (face_bits && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1 ||
+                      (L::D == 3 && (z == 0 || z == nz - 1))))
+        bits |= kFaceBit;
     links[slot] = bits;
 }
 
@@ -2679,8 +2719,9 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
         return launch_overlapped(k_step_compact<L, MODEL, S, true>, grid, kBlock, st, a, src, dst,
                                  s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials,
                                  s.rng_ctr, s.parity);
-    } else if constexpr (compact_loop<MODEL, S>()) {
-        // persistent: as many blocks as are resident at once, at most one per 256 slots
+    }
+    if constexpr (compact_loop<S>()) {
+        // persistent: as many blocks as are resident at once
         static const int resident = [] {   // blocks per SM (per instantiation)
             int r = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_step_compact_loop<L, MODEL, S>,
@@ -2693,15 +2734,19 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int pgrid = std::min(grid, std::max(1, resident * sms));
-        return launch_overlapped(k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
-                                 s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
-    } else {
-        constexpr int B = compact_block<L, MODEL>();
-        return launch_overlapped(k_step_compact<L, MODEL, S, false, B>, (kp.nslots + B - 1) / B, B, st,
-                                 a, src, dst, s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap,
-                                 s.partials, s.rng_ctr, s.parity);
+        const int pgrid = std::max(1, resident * sms);
+        if (grid >= kLoopRounds * pgrid)
+            return launch_overlapped(k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
+                                     s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
     }
+    auto one = [&](auto kernel, int b) {
+        return launch_overlapped(kernel, (kp.nslots + b - 1) / b, b, st, a, src, dst, s.links, s.cellidx,
+                                 s.rank, (R*)s.tau, (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
+    };
+    // few slots: finer blocks spread over the SMs (see untuned_block)
+    if (kp.nslots <= 8 * 152 * kBlock) return one(k_step_compact<L, MODEL, S, false, 128>, 128);
+    constexpr int B = compact_block<L, MODEL, S>();
+    return one(k_step_compact<L, MODEL, S, false, B>, B);
 }
 
 // The compact layout has its own kernel.  In the dense one the copy-through
@@ -2788,9 +2833,9 @@ cudaError_t launch_batch_lat(int model, int storage, bool check, const BatchDesc
 
 template <class L>
 cudaError_t launch_links_lat(const KParams& kp, const uint8_t* mask, uint32_t* links,
-                             const int* cellidx, cudaStream_t st) {
+                             const int* cellidx, bool face_bits, cudaStream_t st) {
     if (cellidx)
-        k_links_compact<L><<<step_grid(kp.nslots), kBlock, 0, st>>>(kp, mask, cellidx, links);
+        k_links_compact<L><<<step_grid(kp.nslots), kBlock, 0, st>>>(kp, mask, cellidx, links, face_bits);
     else
         k_links<L><<<step_grid(kp.ncells), kBlock, 0, st>>>(kp, mask, links);
     return cudaGetLastError();
@@ -2920,8 +2965,8 @@ template <class L> void lattice_table(int* c, double* w) {
         return launch_step_lat<L>(model, storage, check, kp, a, st);                            \
     }                                                                                           \
     cudaError_t launch_links_##L(const KParams& kp, const uint8_t* mask, uint32_t* links,      \
-                                 const int* cellidx, cudaStream_t st) {                         \
-        return launch_links_lat<L>(kp, mask, links, cellidx, st);                               \
+                                 const int* cellidx, bool face_bits, cudaStream_t st) {         \
+        return launch_links_lat<L>(kp, mask, links, cellidx, face_bits, st);                    \
     }                                                                                           \
     cudaError_t launch_fields_##L(int storage, const KParams& kp, const void* f,               \
                                   const uint32_t* links, const int* rank, double* rho,         \

@@ -234,11 +234,12 @@ bool resident_fits(const lbm_solver* s) {
 }
 
 cudaError_t launch_links(lbm_solver* s, const uint8_t* mask) {
+    const bool face = storage_bytes(s->p.storage) == 2;
     switch (s->lat) {
-    case LBM_D2Q9: return launch_links_D2Q9(s->kp, mask, s->links, s->cellidx, s->stream);
-    case LBM_D3Q15: return launch_links_D3Q15(s->kp, mask, s->links, s->cellidx, s->stream);
-    case LBM_D3Q19: return launch_links_D3Q19(s->kp, mask, s->links, s->cellidx, s->stream);
-    default: return launch_links_D3Q27(s->kp, mask, s->links, s->cellidx, s->stream);
+    case LBM_D2Q9: return launch_links_D2Q9(s->kp, mask, s->links, s->cellidx, face, s->stream);
+    case LBM_D3Q15: return launch_links_D3Q15(s->kp, mask, s->links, s->cellidx, face, s->stream);
+    case LBM_D3Q19: return launch_links_D3Q19(s->kp, mask, s->links, s->cellidx, face, s->stream);
+    default: return launch_links_D3Q27(s->kp, mask, s->links, s->cellidx, face, s->stream);
     }
 }
 

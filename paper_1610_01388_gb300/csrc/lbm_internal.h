@@ -14,6 +14,7 @@ namespace blbm {
 constexpr int kBlock = 256;          // threads per block of the cell kernels
 constexpr int kNumStats = 8;         // doubles per reduction partial
 constexpr uint32_t kSolidBit = 1u << 31;
+constexpr uint32_t kFaceBit = 1u << 30;   // compact link words: the cell lies at a face of the box
 // Kernel-side model code: PR with the Newton-implicit tau update is its own
 // instantiation, so the explicit kernels carry none of its code.
 constexpr int kModelPRImplicit = 2;
@@ -71,7 +72,7 @@ struct BatchDesc;   // per-domain descriptor of a batched launch (kernels.cuh)
     cudaError_t launch_step_##L(int model, int storage, bool check, const KParams& kp,          \
                                 const StepArgs& a, cudaStream_t st);                            \
     cudaError_t launch_links_##L(const KParams& kp, const uint8_t* mask, uint32_t* links,       \
-                                 const int* cellidx, cudaStream_t st);                          \
+                                 const int* cellidx, bool face_bits, cudaStream_t st);          \
     cudaError_t launch_fields_##L(int storage, const KParams& kp, const void* f,                \
                                   const uint32_t* links, const int* rank, double* rho,          \
                                   double* ux, double* uy, double* uz, cudaStream_t st);         \
