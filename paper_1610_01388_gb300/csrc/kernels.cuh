@@ -620,6 +620,28 @@ template <class L> constexpr bool fam_order() {
 static_assert(fam_order<D2Q9>() && fam_order<D3Q15>() && fam_order<D3Q19>() && fam_order<D3Q27>(),
               "direction families");
 
+// Parts a cell's pair-form collision can be divided into, one warp each (see
+// k_step_split), by families: the axis pairs with the rest population, and the
+// diagonals.  pair_part() owns pair p.
+template <class L> __host__ __device__ constexpr int parts() { return L::Q >= 19 ? 4 : 2; }
+template <class L> __host__ __device__ constexpr int pair_part(int p) {
+    if (p < L::D) return 0;
+    if (L::Q == 9 || L::Q == 15) return 1;
+    if (L::Q == 19) return 1 + (p - 3) / 2;                  // a part per face plane
+    return p < 7 ? 1 : p < 9 ? 2 : 3;                        // xy and xz, yz, corners
+}
+// pair k of a part (-1: it has fewer), and the place of pair p in its part
+template <class L> __host__ __device__ constexpr int part_pair(int part, int k) {
+    for (int p = 0; p < (L::Q - 1) / 2; ++p)
+        if (pair_part<L>(p) == part && k-- == 0) return p;
+    return -1;
+}
+template <class L> __host__ __device__ constexpr int part_place(int p) {
+    int k = 0;
+    for (int q = 0; q < p; ++q) k += pair_part<L>(q) == pair_part<L>(p);
+    return k;
+}
+
 // b x and y + b x for a compile-time factor b (a plain x, y + x where it is 1)
 template <class R, class B> __device__ __forceinline__ R scale(B b, R x) {
     if (b == B(1)) return x;
@@ -803,7 +825,8 @@ template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t)
 // (weighted) and its odd part wo cq.  Where w_i in memory units is the same for
 // every direction (the 16-bit forms) it goes into the six numbers and q once,
 // and wo = 1.
-template <class L, class S, class R, class Put>
+// PART >= 0: only the pairs of that part (the compiler drops the rest).
+template <class L, class S, class R, int PART = -1, class Put>
 __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R qz, Put&& put) {
     constexpr int F = Fam<L>::face, C = Fam<L>::corner;
     constexpr bool same = sizeof(S) == 2;   // gam, god do not depend on the direction
@@ -827,7 +850,8 @@ __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R
     const R kF = R(B(9) * gF * unit), kC = R(B(9) * gC * unit);
     auto pair = [&](auto I, R e, R cq) {
         constexpr int i = decltype(I)::value;
-        if constexpr (same) put(I, e, cq, B(1));
+        if constexpr (PART >= 0 && pair_part<L>((i - 1) / 2) != PART) return;
+        else if constexpr (same) put(I, e, cq, B(1));
         else put(I, e, cq, Store<S>::template god<L, i>());
     };
     const R eA = scale(gA, e0);
@@ -896,10 +920,10 @@ __device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R
 // ---------------------------------------------------------------------------
 // IR collision (Secs. 2.3, 3.2).  f: memory units in, memory units out.  R is
 // the arithmetic type: one cell (float, double) or two cells (F2).
-template <class L, class S, class R>
-__device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
-                                           R (&f)[L::Q], R& drho, R (&ur)[3]) {
-    const Mom<R> m = moments<L, S, R>(f);
+// What the pairs need from the moments: e0, N and q of pair_terms.
+template <class L, class R>
+__device__ __forceinline__ void ir_terms(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                         const Mom<R>& m, R& e0, Tens<R>& N, R (&q)[3], R (&ur)[3]) {
     const R rho = add(R(1), m.d);
     const R inv = rcp(rho);
     const R gx = R(c.g[0]), gy = R(c.g[1]);
@@ -919,7 +943,6 @@ __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc
     // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i,
     // and rho u u = P - T
     const R k2 = mul(asg, mul(trace<L, R>(T), R(1.0 / L::D)));
-    Tens<R> N;
     N.xx = mad(k1, T.xx, add(P.xx, k2));
     N.yy = mad(k1, T.yy, add(P.yy, k2));
     N.xy = mad(k1, T.xy, P.xy);
@@ -932,21 +955,31 @@ __device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc
         N.yz = mad(k1, T.yz, P.yz);
     }
     if (flags & LBM_FLAG_BURNETT_X) N.xx = add(mul(px, ux), k2);   // T.xx was dropped
-    const R e0 = mad(R(-1.5), trace<L, R>(N), m.d);
+    e0 = mad(R(-1.5), trace<L, R>(N), m.d);
     // odd part: w_i (3 rho c.u + 3/2 c.F) = 3 w_i c.(j + F), since rho u = j + F/2
-    const R qx = mad(rho, gx, m.jx), qy = mad(rho, gy, m.jy);
-    R qz = R(0);
-    if constexpr (L::D == 3) qz = mad(rho, gz, m.jz);
+    q[0] = mad(rho, gx, m.jx);
+    q[1] = mad(rho, gy, m.jy);
+    q[2] = R(0);
+    if constexpr (L::D == 3) q[2] = mad(rho, gz, m.jz);
+    ur[0] = ux;
+    ur[1] = uy;
+    ur[2] = uz;
+}
+
+template <class L, class S, class R>
+__device__ __forceinline__ void pair_collide_ir(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                                R (&f)[L::Q], R& drho, R (&ur)[3]) {
+    const Mom<R> m = moments<L, S, R>(f);
+    R e0, q[3];
+    Tens<R> N;
+    ir_terms<L, R>(c, flags, m, e0, N, q, ur);
     f[0] = scale(Store<S>::template gam<L, 0>(), e0);
-    pair_terms<L, S, R>(e0, N, qx, qy, qz, [&](auto I, R e, R cq, auto wo) {
+    pair_terms<L, S, R>(e0, N, q[0], q[1], q[2], [&](auto I, R e, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
         f[i] = axpy(wo, cq, e);
         f[i + 1] = axpy(-wo, cq, e);
     });
     drho = m.d;
-    ur[0] = ux;
-    ur[1] = uy;
-    ur[2] = uz;
 }
 
 // ---------------------------------------------------------------------------
@@ -1062,16 +1095,17 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>&
 // PR collision (Sec. 3.1 + TRT + EDM).  tau: previous step's relaxation time
 // in, this step's out.  f: memory units in, memory units out (the TRT update is
 // linear and opposite populations share their unit).  R as for collide_ir.
-template <class L, class S, bool IMPLICIT, class R>
-__device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
-                                           R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
-    const Mom<R> m = moments<L, S, R>(f);
+// What the pairs need from the moments: K0, N and q of pair_terms and the rates.
+template <class L, bool IMPLICIT, class R>
+__device__ __forceinline__ void pr_terms(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                         const Mom<R>& m, R& tau, R& K0, Tens<R>& N, R (&q)[3], R& wp,
+                                         R& wm, R (&ur)[3]) {
     const R rho = add(R(1), m.d);
     R inv, itau;   // 1 / rho, 1 / tau_old
     if constexpr (sizeof(typename Lanes<R>::Sc) == 8) {
-        const R q = rcp(mul(rho, tau));   // one FP64 reciprocal for both
-        inv = mul(q, tau);
-        itau = mul(q, rho);
+        const R both = rcp(mul(rho, tau));   // one FP64 reciprocal for both
+        inv = mul(both, tau);
+        itau = mul(both, rho);
     } else {
         inv = rcp(rho);
         itau = rcp(tau);
@@ -1079,7 +1113,6 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     const R ux = mul(m.jx, inv), uy = mul(m.jy, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(m.jz, inv);
-    R wp, wm;
     {
         const Tens<R> T = noneq<L, R>(dynamic<L, R>(m), -m.jx, -m.jy, -m.jz, ux, uy, uz, flags);
         pair_pr_rates<IMPLICIT, R>(c, square<L, R>(T), inv, itau, tau, wp, wm);
@@ -1097,7 +1130,6 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
     //   O = f^- - wm (f^- - f_eq^-) + F^- = (1 - wm)/2 (f_i - f_o) + 3 w_i c.(wm j + F),
     // the odd equilibrium and force parts from j and F directly (3 w_i rho c.u
     // = 3 w_i c.j exactly).  f holds the pair sums and differences.
-    Tens<R> N;
     {
         const R vx = mad(wp, ux, gx), vy = mad(wp, uy, gy), zx = add(ux, gx), zy = add(uy, gy);
         N.xx = mad(m.jx, vx, mul(Fx, zx));
@@ -1113,14 +1145,27 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
             N.yz = mad(m.jy, vz, mul(Fy, zz));
         }
     }
+    K0 = mad(R(-1.5), trace<L, R>(N), mul(wp, m.d));
+    q[0] = mad(wm, m.jx, Fx);
+    q[1] = mad(wm, m.jy, Fy);
+    q[2] = R(0);
+    if constexpr (L::D == 3) q[2] = mad(wm, m.jz, Fz);
+    ur[0] = mad(R(0.5), gx, ux);
+    ur[1] = mad(R(0.5), gy, uy);
+    ur[2] = mad(R(0.5), gz, uz);
+}
+
+template <class L, class S, bool IMPLICIT, class R>
+__device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
+                                                R (&f)[L::Q], R& tau, R& drho, R (&ur)[3]) {
+    const Mom<R> m = moments<L, S, R>(f);
+    R K0, q[3], wp, wm;
+    Tens<R> N;
+    pr_terms<L, IMPLICIT, R>(c, flags, m, tau, K0, N, q, wp, wm, ur);
     const R omp = mad(R(-0.5), wp, R(0.5));
     const R omm = mad(R(-0.5), wm, R(0.5));
-    const R K0 = mad(R(-1.5), trace<L, R>(N), mul(wp, m.d));
-    const R qx = mad(wm, m.jx, Fx), qy = mad(wm, m.jy, Fy);
-    R qz = R(0);
-    if constexpr (L::D == 3) qz = mad(wm, m.jz, Fz);
     f[0] = axpy(Store<S>::template gam<L, 0>(), K0, mad(-wp, f[0], f[0]));
-    pair_terms<L, S, R>(K0, N, qx, qy, qz, [&](auto I, R e, R cq, auto wo) {
+    pair_terms<L, S, R>(K0, N, q[0], q[1], q[2], [&](auto I, R e, R cq, auto wo) {
         constexpr int i = decltype(I)::value;
         const R E = mad(omp, f[i], e);
         const R O = mad(omm, f[i + 1], scale(wo, cq));
@@ -1128,9 +1173,6 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
         f[i + 1] = sub(E, O);
     });
     drho = m.d;
-    ur[0] = mad(R(0.5), gx, ux);
-    ur[1] = mad(R(0.5), gy, uy);
-    ur[2] = mad(R(0.5), gz, uz);
 }
 
 // ---------------------------------------------------------------------------
@@ -1637,6 +1679,257 @@ k_step2(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
 }
 
 // ---------------------------------------------------------------------------
+// Divided FP64 steps.  An FP64 warp instruction holds its SM sub-partition's
+// FP64 pipe for 64 cycles whatever it has in flight, so a small domain, one warp
+// on each of a few sub-partitions, takes as long as its longest warp however
+// many others idle.  Here the cells of one warp are stepped by parts<L>() warps:
+// each gathers, pairs up and stores the populations of its part (see
+// pair_part); the family sums that pair_moments combines go through shared
+// memory, its combining adds are dealt out to the warps, and what follows from
+// the moments is done by every warp for itself.  The expressions are those of
+// pair_moments, ir_terms, pr_terms and pair_terms, so the results are the bits of
+// the undivided step.  FP64 operations of the longest warp, D3Q27 IR: about 96
+// against 215.
+enum { kExFace = 0, kExCorner = 12, kExAxis = 19, kExRest = 25, kExCount = 26 };
+struct SplitShared {
+    double ex[kExCount][32];   // family sums: 4 per face plane, 7 of the corners, the axis pairs, f_0
+    double mo[10][32];         // d, j, p
+};
+// f(part as a constant)
+template <class L, class F> __device__ __forceinline__ void by_part(int part, F&& f) {
+    if (part == 0) f(std::integral_constant<int, 0>{});
+    else if (part == 1) f(std::integral_constant<int, 1>{});
+    if constexpr (parts<L>() == 4) {
+        if (part == 2) f(std::integral_constant<int, 2>{});
+        else if (part == 3) f(std::integral_constant<int, 3>{});
+    }
+}
+// r[2 k], r[2 k + 1]: populations (i, i + 1) of a part's pair k; f(i, place in r)
+template <class L, int PART, class F> __device__ __forceinline__ void part_pops(F&& f) {
+    static_for<0, 4>([&](auto K) {
+        constexpr int k = decltype(K)::value, p = part_pair<L>(PART, k);
+        if constexpr (p >= 0) {
+            f(std::integral_constant<int, 2 * p + 1>{}, std::integral_constant<int, 2 * k>{});
+            f(std::integral_constant<int, 2 * p + 2>{}, std::integral_constant<int, 2 * k + 1>{});
+        }
+    });
+}
+// pair form of a part, and its family sums
+template <class L, int PART>
+__device__ __forceinline__ void part_sums(double (&r)[8], double f0, SplitShared& sh, int lane) {
+    static_for<0, 4>([&](auto K) {
+        constexpr int k = 2 * decltype(K)::value;
+        if constexpr (part_pair<L>(PART, k / 2) >= 0) {
+            const double a = r[k], b = r[k + 1];
+            r[k] = add(a, b);
+            r[k + 1] = sub(a, b);
+        }
+    });
+    if constexpr (PART == 0) {
+#pragma unroll
+        for (int d = 0; d < L::D; ++d) {
+            sh.ex[kExAxis + d][lane] = r[2 * d];
+            sh.ex[kExAxis + 3 + d][lane] = r[2 * d + 1];
+        }
+        sh.ex[kExRest][lane] = f0;
+    }
+    constexpr int F = Fam<L>::face, C = Fam<L>::corner;
+    if constexpr (F != 0) {
+        static_for<0, L::D == 2 ? 1 : 3>([&](auto J) {
+            constexpr int j = decltype(J)::value, p = (F - 1) / 2 + 2 * j;
+            if constexpr (pair_part<L>(p) == PART) {
+                constexpr int k = 2 * part_place<L>(p);
+                sh.ex[kExFace + 4 * j][lane] = add(r[k], r[k + 2]);
+                sh.ex[kExFace + 4 * j + 1][lane] = sub(r[k], r[k + 2]);
+                sh.ex[kExFace + 4 * j + 2][lane] = add(r[k + 1], r[k + 3]);
+                sh.ex[kExFace + 4 * j + 3][lane] = sub(r[k + 1], r[k + 3]);
+            }
+        });
+    }
+    if constexpr (C != 0) {
+        if constexpr (pair_part<L>((C - 1) / 2) == PART) {
+            constexpr int k = 2 * part_place<L>((C - 1) / 2);
+            const double ab = add(r[k], r[k + 2]), amb = sub(r[k], r[k + 2]);
+            const double ce = add(r[k + 4], r[k + 6]), cme = sub(r[k + 4], r[k + 6]);
+            const double dp = add(r[k + 1], r[k + 3]), dq = sub(r[k + 5], r[k + 7]);
+            sh.ex[kExCorner][lane] = add(ab, ce);
+            sh.ex[kExCorner + 1][lane] = sub(ab, ce);
+            sh.ex[kExCorner + 2][lane] = add(amb, cme);
+            sh.ex[kExCorner + 3][lane] = sub(amb, cme);
+            sh.ex[kExCorner + 4][lane] = add(dp, dq);
+            sh.ex[kExCorner + 5][lane] = sub(dp, dq);
+            sh.ex[kExCorner + 6][lane] = add(sub(r[k + 1], r[k + 3]), add(r[k + 5], r[k + 7]));
+        }
+    }
+}
+// the combining adds of pair_moments, dealt out by moment
+template <class L, int PART> __device__ __forceinline__ void part_moments(SplitShared& sh, int lane) {
+    constexpr bool F = Fam<L>::face != 0, C = Fam<L>::corner != 0;
+    auto e = [&](int k) { return sh.ex[k][lane]; };
+    auto face = [&](int j, int k) { return e(kExFace + 4 * j + k); };   // k: sum, difference; odd ones
+    if constexpr (L::D == 2) {
+        if constexpr (PART == 0) {
+            const double xx = add(face(0, 0), e(kExAxis));
+            sh.mo[4][lane] = xx;
+            sh.mo[0][lane] = add(xx, add(e(kExAxis + 1), e(kExRest)));
+        } else {
+            sh.mo[5][lane] = add(face(0, 0), e(kExAxis + 1));
+            sh.mo[7][lane] = face(0, 1);
+            sh.mo[1][lane] = add(face(0, 2), e(kExAxis + 3));
+            sh.mo[2][lane] = add(face(0, 3), e(kExAxis + 4));
+        }
+    } else {
+        // diagonal sum beyond the axis pair: corners, then the two planes of the axis
+        auto diag = [&](int j, int k) {
+            if constexpr (F && C) return add(e(kExCorner), add(face(j, 0), face(k, 0)));
+            else if constexpr (F) return add(face(j, 0), face(k, 0));
+            else return e(kExCorner);
+        };
+        auto off = [&](int j) {
+            if constexpr (F && C) return add(e(kExCorner + 1 + j), face(j, 1));
+            else if constexpr (F) return face(j, 1);
+            else return e(kExCorner + 1 + j);
+        };
+        // odd sum of an axis: corners, then two planes' terms a and b
+        auto odd = [&](int axis, int ja, int ka, int jb, int kb) {
+            double v;
+            if constexpr (F) {
+                v = add(face(ja, ka), face(jb, kb));
+                if constexpr (C) v = add(e(kExCorner + 4 + axis), v);
+            } else {
+                v = e(kExCorner + 4 + axis);
+            }
+            return add(v, e(kExAxis + 3 + axis));
+        };
+        constexpr bool two = parts<L>() == 2;
+        if constexpr (PART == 0) {
+            const double xx = add(diag(0, 1), e(kExAxis));
+            double rest = add(e(kExAxis + 1), e(kExAxis + 2));
+            if constexpr (F) rest = add(rest, face(2, 0));
+            sh.mo[4][lane] = xx;
+            sh.mo[0][lane] = add(xx, add(rest, e(kExRest)));
+        }
+        if constexpr (PART == 1) {
+            sh.mo[5][lane] = add(diag(0, 2), e(kExAxis + 1));
+            sh.mo[6][lane] = add(diag(1, 2), e(kExAxis + 2));
+            sh.mo[7][lane] = off(0);
+        }
+        if constexpr (PART == (two ? 0 : 2)) {
+            sh.mo[1][lane] = odd(0, 0, 2, 1, 2);
+            sh.mo[2][lane] = odd(1, 0, 3, 2, 2);
+            sh.mo[8][lane] = off(1);
+        }
+        if constexpr (PART == (two ? 1 : 3)) {
+            sh.mo[3][lane] = odd(2, 1, 3, 2, 3);
+            sh.mo[9][lane] = off(2);
+        }
+    }
+}
+// The divided collision of a warp's cells: r, f0 in and out as populations, tau in
+// and out.  Every thread of the block calls it (two block barriers); `on`:
+// this lane's cell collides.
+template <class L, int MODEL>
+__device__ __forceinline__ void split_collide(const Coef<double>& c, uint32_t flags, int part, int lane,
+                                              bool on, SplitShared& sh, double (&r)[8], double& f0,
+                                              double& tau) {
+    if (on) by_part<L>(part, [&](auto P) { part_sums<L, decltype(P)::value>(r, f0, sh, lane); });
+    __syncthreads();
+    if (on) by_part<L>(part, [&](auto P) { part_moments<L, decltype(P)::value>(sh, lane); });
+    __syncthreads();
+    if (!on) return;
+    Mom<double> m;
+    m.d = sh.mo[0][lane];
+    m.jx = sh.mo[1][lane];
+    m.jy = sh.mo[2][lane];
+    m.xx = sh.mo[4][lane];
+    m.yy = sh.mo[5][lane];
+    m.xy = sh.mo[7][lane];
+    m.jz = L::D == 3 ? sh.mo[3][lane] : 0.0;
+    m.zz = L::D == 3 ? sh.mo[6][lane] : 0.0;
+    m.xz = L::D == 3 ? sh.mo[8][lane] : 0.0;
+    m.yz = L::D == 3 ? sh.mo[9][lane] : 0.0;
+    double e0, q[3], ur[3];
+    Tens<double> N;
+    if constexpr (MODEL == LBM_MODEL_IR) {
+        ir_terms<L, double>(c, flags, m, e0, N, q, ur);
+        by_part<L>(part, [&](auto P) {
+            constexpr int PART = decltype(P)::value;
+            if constexpr (PART == 0) f0 = scale(Store<double>::template gam<L, 0>(), e0);
+            pair_terms<L, double, double, PART>(e0, N, q[0], q[1], q[2], [&](auto I, double e, double cq, auto wo) {
+                constexpr int k = 2 * part_place<L>((decltype(I)::value - 1) / 2);
+                r[k] = axpy(wo, cq, e);
+                r[k + 1] = axpy(-wo, cq, e);
+            });
+        });
+    } else {
+        double wp, wm;
+        pr_terms<L, false, double>(c, flags, m, tau, e0, N, q, wp, wm, ur);
+        const double omp = mad(-0.5, wp, 0.5);
+        const double omm = mad(-0.5, wm, 0.5);
+        by_part<L>(part, [&](auto P) {
+            constexpr int PART = decltype(P)::value;
+            if constexpr (PART == 0)
+                f0 = axpy(Store<double>::template gam<L, 0>(), e0, mad(-wp, f0, f0));
+            pair_terms<L, double, double, PART>(e0, N, q[0], q[1], q[2], [&](auto I, double e, double cq, auto wo) {
+                constexpr int k = 2 * part_place<L>((decltype(I)::value - 1) / 2);
+                const double E = mad(omp, r[k], e);
+                const double O = mad(omm, r[k + 1], scale(wo, cq));
+                r[k] = add(E, O);
+                r[k + 1] = sub(E, O);
+            });
+        });
+    }
+}
+
+// Plain FP64 step, the 32 cells of a block by parts<L>() warps.
+template <class L, int MODEL>
+__global__ void __launch_bounds__(32 * parts<L>())
+k_step_split(const KArgs a, const SrcPlanes<double> src, const DstPlanes<double> dst,
+             const uint32_t* __restrict__ links, double* __restrict__ tau) {
+    __shared__ SplitShared sh;
+    const KParams& kp = a.kp;
+    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    int idx = blockIdx.x * 32 + lane;
+    const bool inside = idx < kp.ncells;
+    const uint32_t lk = inside ? __ldg(links + idx) : kSolidBit;
+    step_begin(idx);
+    const bool on = !(lk & kSolidBit);
+    // as k_step: the solid cells of a group with fluid copy through
+    const bool go = group_has_fluid(on, idx) && inside;
+    if (!__any_sync(0xffffffffu, go)) return;   // the same cells in every warp
+    double r[8], f0 = 0.0, t = 0.0;
+    if (go) {
+        PullOffsets o{0, 0, 0, 0, 0, 0};
+        if (on) o = pull_offsets(kp, idx);
+        const uint32_t wall = on ? lk : 0u;
+        by_part<L>(part, [&](auto P) {
+            constexpr int PART = decltype(P)::value;
+            if constexpr (PART == 0) f0 = *src.template at<0>(idx);
+            part_pops<L, PART>([&](auto I, auto K) {
+                constexpr int i = decltype(I)::value;
+                r[decltype(K)::value] = ((wall >> i) & 1u) ? *src.template at<L::opp(i)>(idx)
+                                                           : *src.template at<i>(idx + o.template of<L, i>());
+            });
+        });
+        if constexpr (MODEL != LBM_MODEL_IR)
+            if (on) t = tau[idx];
+    }
+    split_collide<L, MODEL>(a.cd, kp.flags, part, lane, on, sh, r, f0, t);
+    if (!go) return;
+    by_part<L>(part, [&](auto P) {
+        constexpr int PART = decltype(P)::value;
+        if constexpr (PART == 0) {
+            *dst.template at<0>(idx) = f0;
+            if constexpr (MODEL != LBM_MODEL_IR)
+                if (on) tau[idx] = t;
+        }
+        part_pops<L, PART>([&](auto I, auto K) {
+            *dst.template at<decltype(I)::value>(idx) = r[decltype(K)::value];
+        });
+    });
+}
+
+// ---------------------------------------------------------------------------
 // Resident steps: a run of plain steps of a small domain in one launch, its
 // populations held in the shared memory of one cluster.  A step of such a
 // domain is almost only launch and memory latency (256 cells: 1.6 us of which
@@ -1756,6 +2049,106 @@ k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ lin
     if constexpr (Store<S>::kStochastic)
         // as after nsteps launches: the counter of the buffer now current
         if (blockIdx.x == 0 && t == 0) rng_ctr[parity ^ (nsteps & 1)] = seed + (uint32_t)nsteps;
+}
+
+// The FP64 run of a domain small enough to have a cluster's sub-partitions to
+// spare, its collision divided (see k_step_split): blocks of T cells, T parts<L>()
+// threads, warp w working on part w % parts of the 32 cells w / parts.
+template <class L> struct SplitRun {
+    static constexpr int np = parts<L>();
+    static constexpr int most_cells = 128 / np;            // of a block: a warp per sub-partition
+    static constexpr size_t bytes(int T) {
+        return sizeof(double) * 2 * L::Q * (size_t)T + sizeof(SplitShared) * (size_t)(T / 32);
+    }
+};
+template <class L, int MODEL>
+__global__ void __launch_bounds__(128)
+k_resident_split(const KArgs a, const double* src, double* dst, const uint32_t* __restrict__ links,
+                 double* __restrict__ tau, int nsteps) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const KParams& kp = a.kp;
+    constexpr int np = parts<L>();
+    const int T = (int)blockDim.x / np;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int part = warp % np, t = (warp / np) * 32 + lane;
+    int idx = (int)blockIdx.x * T + t;
+    const bool inside = idx < kp.ncells;
+    const uint32_t lk = inside ? __ldg(links + idx) : kSolidBit;
+    const bool on = !(lk & kSolidBit);
+    step_begin(idx);
+    double* const buf = reinterpret_cast<double*>(smem);
+    const int half = L::Q * T;
+    SplitShared& sh = reinterpret_cast<SplitShared*>(smem + sizeof(double) * 2 * half)[warp / np];
+    uint32_t from[8];
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+    by_part<L>(part, [&](auto P) {
+        constexpr int PART = decltype(P)::value;
+        auto load = [&](int i) {   // both buffers, as k_resident
+            if (!inside) return;
+            const double v = src[(int64_t)i * kp.plane + idx];
+            buf[i * T + t] = v;
+            buf[half + i * T + t] = v;
+        };
+        if constexpr (PART == 0) load(0);
+        PullOffsets o{0, 0, 0, 0, 0, 0};
+        if (on) o = pull_offsets(kp, idx);
+        part_pops<L, PART>([&](auto I, auto K) {
+            constexpr int i = decltype(I)::value;
+            load(i);
+            const bool wall = (lk >> i) & 1u;
+            const int n = on && !wall ? idx + o.template of<L, i>() : inside ? idx : 0;
+            const int b = n / T;
+            const uint32_t own = base + (uint32_t)(((wall ? L::opp(i) : i) * T + n - b * T) * (int)sizeof(double));
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(from[decltype(K)::value]) : "r"(own), "r"(b));
+        });
+    });
+    double tc = 0.0;
+    if constexpr (MODEL != LBM_MODEL_IR)
+        if (on) tc = tau[idx];
+    cluster_barrier();
+    uint32_t rd = 0u;                        // byte offset of the buffer this step reads
+    const uint32_t bytes = (uint32_t)half * (uint32_t)sizeof(double);
+    for (int k = 0; k < nsteps; ++k) {
+        double r[8], f0 = 0.0;
+        if (on) {
+            const double* in = reinterpret_cast<const double*>(smem + rd);
+            by_part<L>(part, [&](auto P) {
+                constexpr int PART = decltype(P)::value;
+                if constexpr (PART == 0) f0 = in[t];
+                part_pops<L, PART>([&](auto, auto K) {
+                    constexpr int j = decltype(K)::value;
+                    r[j] = ld_cluster<double>(from[j] + rd);
+                });
+            });
+        }
+        split_collide<L, MODEL>(a.cd, kp.flags, part, lane, on, sh, r, f0, tc);
+        if (on) {
+            double* out = reinterpret_cast<double*>(smem + (bytes - rd));
+            by_part<L>(part, [&](auto P) {
+                constexpr int PART = decltype(P)::value;
+                if constexpr (PART == 0) out[t] = f0;
+                part_pops<L, PART>([&](auto I, auto K) {
+                    out[decltype(I)::value * T + t] = r[decltype(K)::value];
+                });
+            });
+        }
+        rd = bytes - rd;
+        cluster_barrier();
+    }
+    if (on) {
+        const double* last = reinterpret_cast<const double*>(smem + rd);
+        by_part<L>(part, [&](auto P) {
+            constexpr int PART = decltype(P)::value;
+            if constexpr (PART == 0) {
+                dst[idx] = last[t];
+                if constexpr (MODEL != LBM_MODEL_IR) tau[idx] = tc;
+            }
+            part_pops<L, PART>([&](auto I, auto) {
+                constexpr int i = decltype(I)::value;
+                dst[(int64_t)i * kp.plane + idx] = last[i * T + t];
+            });
+        });
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2544,6 +2937,10 @@ template <class L, class S> inline DstPlanes<S> dst_planes(void* f, int64_t plan
     return P;
 }
 
+// Lanes of one warp on every FP64 pipe (152 SMs of four sub-partitions): the
+// most that divided steps fill (cells times parts).
+constexpr int64_t kSplitLanes = 608 * 32;
+
 // Launch of a step kernel that calls step_begin() (overlapped launches).
 template <class... K, class... A>
 inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, cudaStream_t st,
@@ -2598,6 +2995,19 @@ template <class L, int MODEL, class S> bool resident_ready() {
         cfg.numAttrs = 1;
         int clusters = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+        if constexpr (std::is_same<S, double>::value) {
+            auto divided = k_resident_split<L, MODEL>;
+            cfg.blockDim = dim3(128);
+            cfg.dynamicSmemBytes = SplitRun<L>::bytes(SplitRun<L>::most_cells);
+            int more = 0;
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(divided, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)cfg.dynamicSmemBytes);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(divided, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&more, divided, &cfg);
+            clusters = std::min(clusters, more);
+        }
         if (e != cudaSuccess) cudaGetLastError();
         return e == cudaSuccess && clusters > 0;
     }();
@@ -2611,6 +3021,8 @@ cudaError_t launch_resident_t(const KParams& kp, const StepArgs& s, int nsteps, 
     int threads = 0, blocks = 0;
     if (!resident_shape<L, S>(kp.ncells, threads, blocks)) return cudaErrorNotSupported;
     const KArgs a = make_args<L>(kp);
+    bool divided = false;
+    if constexpr (std::is_same<S, double>::value) divided = threads <= SplitRun<L>::most_cells;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -2625,6 +3037,14 @@ cudaError_t launch_resident_t(const KParams& kp, const StepArgs& s, int nsteps, 
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
+    if constexpr (std::is_same<S, double>::value) {
+        if (divided) {
+            cfg.blockDim = dim3((unsigned)(threads * parts<L>()));
+            cfg.dynamicSmemBytes = SplitRun<L>::bytes(threads);
+            return cudaLaunchKernelEx(&cfg, k_resident_split<L, MODEL>, a, (const double*)s.fsrc,
+                                      (double*)s.fdst, s.links, (double*)s.tau, nsteps);
+        }
+    }
     return cudaLaunchKernelEx(&cfg, kernel, a, (const S*)s.fsrc, (S*)s.fdst, s.links, (R*)s.tau,
                               s.rng_ctr, s.parity, nsteps);
 }
@@ -2695,6 +3115,13 @@ cudaError_t launch_step_c(bool check, const KParams& kp, const StepArgs& s, cuda
                                  (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
     };
     if (check) return go(k_step<L, MODEL, S, true, kBlock, COPY>, kBlock);
+    // FP64 domains that leave sub-partitions idle
+    if constexpr (f64 && MODEL != kModelPRImplicit) {
+        if (s.split && kp.cell_begin == 0 && kp.cell_end == kp.ncells &&
+            (int64_t)kp.ncells * parts<L>() <= kSplitLanes)
+            return launch_overlapped(k_step_split<L, MODEL>, (kp.ncells + 31) / 32, 32 * parts<L>(), st,
+                                     a, src, dst, s.links, (R*)s.tau);
+    }
     // one part of a step taken in parts (256 threads)
     if (kp.cell_begin != 0 || kp.cell_end != kp.ncells)
         return go(k_step<L, MODEL, S, false, kBlock, COPY, true>, kBlock);

@@ -194,6 +194,7 @@ StepArgs step_args(const lbm_solver* s, int flip) {
     a.parity = s->cur;
     a.block = s->block;
     a.cpt = s->cpt;
+    a.split = s->split;
     a.copy = s->copy;
     a.cellidx = s->cellidx;
     a.rank = s->rank;
@@ -713,6 +714,7 @@ void apply_tuning(lbm_solver* s) {
     Shape sh = tune_lookup(s->lat, s->p.model, s->p.storage, s->ncells);
     if (!sh.set) sh.block = untuned_block(s);
     // an entry of the table keeps its launch shape
+    s->split = !sh.set;
     s->resident = !sh.set && !s->rank && resident_fits(s);
     if (sh.block != s->block || sh.cpt != s->cpt) {
         for (int k = 0; k < 2; ++k)
@@ -854,6 +856,7 @@ lbm_status lbm_step_cells(lbm_solver* s, int64_t cell_begin, int64_t cell_end) {
     a.parity = s->cur;
     a.block = kBlock;
     a.cpt = 1;
+    a.split = 0;
     a.copy = s->copy;
     a.cellidx = nullptr;
     a.rank = nullptr;

@@ -58,6 +58,7 @@ struct StepArgs {
     int parity;          // which of the two counters this launch reads
     int block;           // threads per block of plain steps (128, 256 or 512)
     int cpt;             // cells per thread of plain steps (1, or 2 with block 128 / 256)
+    int split;           // FP64: small domains may divide a cell's work over warps
     int copy;            // 16-bit PR: solid cells of mixed groups copy through (geometry choice)
     const int* cellidx;  // compact layout: cell index of each slot (nullptr: dense layout)
     const int* rank;     // compact layout: slot of each cell, negative for solid cells

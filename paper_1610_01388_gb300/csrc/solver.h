@@ -66,6 +66,7 @@ struct lbm_solver {
     int block = 256;                   // threads per block of plain steps (tuning table)
     int cpt = 1;                       // cells per thread of plain steps (tuning table)
     int copy = 1;                      // at least 1 % of the warps with fluid also hold solid cells
+    bool split = false;                // small FP64 steps may be divided over warps
     bool resident = false;             // runs of plain steps may stay in shared memory
     uint64_t tune_version = ~uint64_t(0);
 };

@@ -83,3 +83,27 @@ def test_table_entry_keeps_its_launch_shape():
         _same(a, b, "IR")
     finally:
         lbm.lbm_tuning_clear()
+
+
+@pytest.mark.parametrize("model", ["IR", "PR"])
+@pytest.mark.parametrize("lat,shape", [("D2Q9", (1, 13, 11)), ("D2Q9", (1, 33, 31)), ("D2Q9", (1, 79, 80)),
+                                       ("D3Q15", (5, 6, 7)), ("D3Q15", (20, 21, 19)),
+                                       ("D3Q19", (5, 6, 7)), ("D3Q19", (15, 16, 17)),
+                                       ("D3Q27", (5, 6, 7)), ("D3Q27", (15, 16, 17))])
+@pytest.mark.parametrize("flags", [0, lbm.LBM_FLAG_BURNETT_X, lbm.LBM_FLAG_Z_GHOSTS])
+def test_divided_fp64_steps_equal_undivided_ones(lat, shape, model, flags):
+    """Small FP64 domains divide a cell's work over warps; a table entry keeps
+    the undivided kernel.  Same expressions, same bits."""
+    if flags == lbm.LBM_FLAG_Z_GHOSTS and lat == "D2Q9":
+        pytest.skip("ghost planes need a 3D lattice")
+    _, _, cls = lbm.lbm_tuning_get_shape(lat, model, "F64", int(np.prod(shape)))
+    try:
+        a = _state(lat, shape, model, "F64", flags=flags)
+        a.step(3)                         # single steps
+        a.step(21)                        # a run
+        lbm.lbm_tuning_set(lat, model, "F64", cls, 128)
+        b = _state(lat, shape, model, "F64", flags=flags)
+        b.step(24)
+        _same(a, b, model)
+    finally:
+        lbm.lbm_tuning_clear()
