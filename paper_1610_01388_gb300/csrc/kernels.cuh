@@ -29,6 +29,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <type_traits>
 #include <utility>
@@ -2973,9 +2974,14 @@ template <class L, class S> inline bool resident_shape(int ncells, int& threads,
 
 // Raises the kernel's limits (shared memory and blocks per cluster above the
 // defaults) and asks whether the device can hold its largest cluster; once per
-// instantiation.
+// instantiation and device (the limits belong to the device's copy).
 template <class L, int MODEL, class S> bool resident_ready() {
-    static const bool ready = [] {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];   // 0: not asked, 1: yes, 2: no
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
+    if (const int k = known[dev].load()) return k == 1;
+    const bool ready = [] {
         auto kernel = k_resident<L, MODEL, S>;
         constexpr int threads = resident_threads<L, S>();
         constexpr int bytes = (int)sizeof(S) * 2 * L::Q * threads;
@@ -3011,6 +3017,7 @@ template <class L, int MODEL, class S> bool resident_ready() {
         if (e != cudaSuccess) cudaGetLastError();
         return e == cudaSuccess && clusters > 0;
     }();
+    known[dev].store(ready ? 1 : 2);
     return ready;
 }
 

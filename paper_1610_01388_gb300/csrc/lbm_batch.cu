@@ -587,7 +587,11 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     if (b->dirty && (v = rebuild(b)) != LBM_OK) return v;
     int active = 0;
     for (const auto& g : b->groups) active += !g.ids.empty();
-    const bool branches = b->concurrent && active > 1;
+    // a caller that captures the stream gets plain launches (a graph cannot be
+    // launched into a capture)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &capturing) != cudaSuccess) cudaGetLastError();
+    const bool branches = b->concurrent && active > 1 && capturing == cudaStreamCaptureStatusNone;
     // one launch of the graph with this content, at the current phase
     auto replay = [&](int content) {
         cudaGraphExec_t& g = b->graph[content][b->phase];
