@@ -2027,10 +2027,17 @@ k_resident(const KArgs a, const S* src, S* dst, const uint32_t* __restrict__ lin
                 f[i] = ld_cluster<S>(from[i] + rd);
             });
             R drho, ur[3];
-            if constexpr (MODEL != LBM_MODEL_IR)
+            if constexpr (MODEL != LBM_MODEL_IR) {
                 collide_pr<L, S, false>(coef<R>(a), kp.flags, f, tc, drho, ur);
-            else
+            } else if constexpr (pair_form<S>()) {
                 collide_ir<L, S>(coef<R>(a), kp.flags, f, drho, ur);
+            } else {
+                // behind a branch of its own, as in k_step: merged with the
+                // gather the compiler contracts the class sums differently
+                int go = 1;
+                asm volatile("" : "+r"(go));
+                if (go) collide_ir<L, S>(coef<R>(a), kp.flags, f, drho, ur);
+            }
             uint32_t rnd = 0u;
             if constexpr (Store<S>::kStochastic)
                 rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ ((seed + (uint32_t)k) * 0x9e3779b9u));
@@ -3056,11 +3063,18 @@ cudaError_t launch_resident_t(const KParams& kp, const StepArgs& s, int nsteps, 
                               s.rng_ctr, s.parity, nsteps);
 }
 
+// Left out: the Newton-implicit step, and FP32 IR on D3Q15 and D3Q27, whose
+// class-sum collision the compiler contracts differently here than in k_step
+// (every other form gives the same bits).
+template <class L, class S> constexpr bool resident_ir() {
+    return pair_form<S>() || L::Q == 9 || L::Q == 19;
+}
+
 template <class L, class S>
 cudaError_t launch_resident_model(int model, const KParams& kp, const StepArgs& s, int nsteps,
                                   cudaStream_t st) {
     if (model == LBM_MODEL_PR) return launch_resident_t<L, LBM_MODEL_PR, S>(kp, s, nsteps, st);
-    if constexpr (pair_form<S>()) return launch_resident_t<L, LBM_MODEL_IR, S>(kp, s, nsteps, st);
+    if constexpr (resident_ir<L, S>()) return launch_resident_t<L, LBM_MODEL_IR, S>(kp, s, nsteps, st);
     return cudaErrorNotSupported;
 }
 
@@ -3076,15 +3090,12 @@ cudaError_t launch_resident_lat(int model, int storage, const KParams& kp, const
     }
 }
 
-// Left out: FP32 IR, whose class-sum collision the compiler contracts
-// differently here than in k_step (the other forms give the same bits), and the
-// Newton-implicit step.
 template <class L, class S> bool resident_fits_model(int model, int ncells) {
     int threads = 0, blocks = 0;
     if (!resident_shape<L, S>(ncells, threads, blocks)) return false;
-    if (model == kModelPRImplicit || (!pair_form<S>() && model == LBM_MODEL_IR)) return false;
+    if (model == kModelPRImplicit) return false;
     if (model == LBM_MODEL_PR) return resident_ready<L, LBM_MODEL_PR, S>();
-    if constexpr (pair_form<S>()) return resident_ready<L, LBM_MODEL_IR, S>();
+    if constexpr (resident_ir<L, S>()) return resident_ready<L, LBM_MODEL_IR, S>();
     return false;
 }
 
