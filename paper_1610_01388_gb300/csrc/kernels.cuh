@@ -357,6 +357,28 @@ template <> struct Store<__nv_bfloat16> {
     static __device__ __forceinline__ double dec(__nv_bfloat16 v, double w) { return (double)__bfloat162float(v) * w; }
 };
 
+// The same storage, stepped with the pair-form collision (see pair_form).
+struct PairHalf {
+    __half v;
+};
+struct PairBf16 {
+    __nv_bfloat16 v;
+};
+template <class T, class B> struct PairStore : Store<B> {
+    template <class L, int i> static __device__ __forceinline__ float ld(const T* p) {
+        return Store<B>::template ld<L, i>(&p->v);
+    }
+    template <class L, int i> static __device__ __forceinline__ void st(T* p, float v, uint32_t rnd) {
+        Store<B>::template st<L, i>(&p->v, v, rnd);
+    }
+    template <class L, int i>
+    static __device__ __forceinline__ void st2(T* pi, T* po, float vi, float vo, uint32_t rnd) {
+        Store<B>::template st2<L, i>(&pi->v, &po->v, vi, vo, rnd);
+    }
+};
+template <> struct Store<PairHalf> : PairStore<PairHalf, __half> {};
+template <> struct Store<PairBf16> : PairStore<PairBf16, __nv_bfloat16> {};
+
 // Rheology constants in the arithmetic type, derived on the host in FP64.
 template <class R> struct Coef {
     R nu_p, sigma_y, m, gdot_c, inv_gc, e_c, magic;
@@ -524,16 +546,20 @@ template <class R> struct Tens {
     R xx, yy, zz, xy, xz, yz;
 };
 
-// Which form of the collision a storage form runs.  Pair form (below): FP64,
-// whose step is bound by the FP64 pipe (D3Q27 IR, duct 1 x 64 x 64: 24.5 ->
-// 19.0 us a step; D2Q9 PR, 80 x 80: 15.6 -> 13.5), and the 16-bit forms, whose
-// step is bound by instruction issue (D3Q27 PR FP16: 703 -> 607 instructions a
-// warp; BF16 IR, duct 256 x 128 x 128: 96.1 -> 90.7 us; D3Q19 PR FP16, compact
-// porous 256^3: 326 -> 311).  Errors against FP64 did not grow.  FP32 storage
-// keeps the class sums, which are bit for bit the results it has always had:
-// the pair form gained it 0.4-3 % (its large steps are bound by HBM), and near
-// a steady state the residual shows any change of rounding.
-template <class S> __host__ __device__ constexpr bool pair_form() { return sizeof(S) != 4; }
+// Which form of the collision a domain runs.  Pair form (below): FP64, whose
+// step is bound by the FP64 pipe (D3Q27 IR, duct 1 x 64 x 64: 24.5 -> 19.0 us a
+// step; D2Q9 PR, 80 x 80: 15.6 -> 13.5), and the 16-bit forms of domains with large
+// x-y planes (kPairPlane), whose step is bound by instruction issue (us a step,
+// class -> pair form, D3Q27 duct 256 x 128 x 128: PR FP16 109.9 -> 99.1, IR 91.9 ->
+// 87.0; D3Q19 PR FP16, compact porous 256^3: 319 -> 260).  Errors against FP64 did
+// not grow.  FP32 storage and the 16-bit forms of smaller domains keep the
+// class sums, which are bit for bit the results they have always had: the pair
+// form gained FP32 0.4-3 % (its large steps are bound by HBM), small domains are
+// bound by latency, and near a steady state, which they reach, the residual
+// shows any change of rounding.
+template <class S> __host__ __device__ constexpr bool pair_form() {
+    return sizeof(S) == 8 || std::is_same<S, PairHalf>::value || std::is_same<S, PairBf16>::value;
+}
 
 // Grouped sums: populations are added once per velocity class (c_x = +1, -1,
 // 0; c_y = +-1; c_z = +-1; sign of c_x c_y, c_x c_z, c_y c_z) and the moments
@@ -1416,7 +1442,9 @@ __device__ __forceinline__ void step_begin(int& n) {
 // smaller lattices keep 1280 (10 x 128, 5 x 256, 2 x 512): D3Q19 PR then
 // takes 48 registers without spilling and measured 7-9 % faster than at 64
 // (porous box 256^3: FP32 466 -> 430 us, FP16 440 -> 401 us; duct
-// 256 x 128 x 128: FP32 113.5 -> 105.7 us).  IR (40-48 registers) and FP64
+// 256 x 128 x 128: FP32 113.5 -> 105.7 us).  Their 16-bit PR steps in the pair form
+// keep 1536 (40 registers, up to 16 bytes spilled): duct 256 x 128 x 128, D3Q19
+// 87.0 -> 80.3 us, D3Q15 74.6 -> 70.0; porous 160^3 D3Q19 91.8 -> 86.0.  IR (40-48 registers) and FP64
 // arithmetic (which these caps would make spill) are left to the allocator.
 // BLBM_PR_MINB / BLBM_IR_MINB override at build time.
 #ifndef BLBM_PR_MINB
@@ -1431,7 +1459,7 @@ template <class L, int MODEL, class S, bool CHECK, int BLOCK> constexpr int step
     if (std::is_same<typename Store<S>::R, double>::value) return 0;
     if (BLBM_PR_MINB >= 0) return BLBM_PR_MINB;
     if (L::Q == 27 || CHECK) return BLOCK == 128 ? 9 : 1024 / BLOCK;   // check steps: no spill
-    return 1280 / BLOCK;
+    return (sizeof(S) == 2 && pair_form<S>() ? 1536 : 1280) / BLOCK;
 }
 
 // Stores one cell's outgoing populations at element n of the planes: the
@@ -2184,7 +2212,7 @@ k_resident_split(const KArgs a, const double* src, double* dst, const uint32_t* 
 //
 // ROWS = false leaves the row paths out.
 //
-// In the 16-bit forms, bound by issue, the link word says whether the cell
+// In the pair-form 16-bit steps, bound by issue, the link word says whether the cell
 // lies at any face of the box (kFaceBit); a warp without such cells needs no
 // coordinates, its rows being at constant offsets (D3Q19 256^3 porous box: IR
 // 248 -> 225 us, PR 281 -> 261).  In the FP32 IR step, bound by latency, that form
@@ -2198,7 +2226,7 @@ template <class L, class S, bool ROWS = true, class Src>
 __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, uint32_t lk,
                                                int idx, int slot, const int* __restrict__ rank,
                                                typename Store<S>::R (&v)[L::Q]) {
-    constexpr bool by_face = sizeof(S) == 2;
+    constexpr bool by_face = sizeof(S) == 2 && pair_form<S>();
     PullOffsets o{0, 0, 0, 0, 0, 0};
     bool edge;   // this lane's cell keeps the warp from the row paths
     if constexpr (by_face) {
@@ -2296,10 +2324,11 @@ __device__ __forceinline__ void compact_cell(const KParams& kp, const Coef<typen
         for (int d = 0; d < 3; ++d) up[d] = usnap[(int64_t)d * kp.plane + slot];
     }
     R f[L::Q];
-    // D3Q27 FP32 IR looks every neighbour up: beside the row paths the compiler
-    // contracts its class-sum collision differently, and its results would move
-    // by a rounding (124 us on the 160^3 porous box, 118 with the row paths)
-    constexpr bool rows = !(sizeof(S) == 4 && L::Q == 27 && MODEL == LBM_MODEL_IR);
+    // The class sums of D3Q27 FP32 IR and of the 16-bit forms look every neighbour
+    // up: beside the row paths the compiler contracts them differently, and
+    // results would move by a rounding (D3Q27 FP32 IR, 160^3 porous box: 124 us, 118
+    // with the row paths)
+    constexpr bool rows = pair_form<S>() || (sizeof(S) == 4 && !(L::Q == 27 && MODEL == LBM_MODEL_IR));
     gather_compact<L, S, rows>(kp, src, lk, idx, slot, rank, f);
     R drho, ur[3];
     if constexpr (MODEL != LBM_MODEL_IR) {
@@ -2326,8 +2355,8 @@ template <class L, int MODEL, class S, bool CHECK> constexpr int compact_min_blo
     // the allocator's 38 registers.  D3Q27 IR: 4 blocks (64 registers; 48
     // spilled and ran slower).  PR keeps the dense step's budget (6 blocks
     // spilled and made the D3Q19 FP16 step 7 % slower).
-    // 16-bit IR up to 19 velocities spills at 6 (its large domains run the loop).
-    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q == 27 ? 4 : sizeof(S) == 2 ? 5 : 6;
+    // Pair-form 16-bit IR up to 19 velocities spills at 6 (large domains run the loop).
+    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q == 27 ? 4 : pair_form<S>() ? 5 : 6;
     return step_min_blocks<L, MODEL, S, CHECK, kBlock>();
 }
 
@@ -2394,7 +2423,10 @@ k_step_compact(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
 // critical path.  It pays for the 16-bit forms.  The FP32 forms need more
 // registers for it than their budgets hold (D3Q19 IR, 256^3 porous box: 323 us
 // by one-slot threads, 349-386 by the loop).
-template <class S> constexpr bool compact_loop() { return sizeof(S) == 2; }
+// (class sums: the IR step, at every size)
+template <int MODEL, class S> constexpr bool compact_loop() {
+    return sizeof(S) == 2 && (pair_form<S>() || MODEL == LBM_MODEL_IR);
+}
 // ... and for domains of several rounds of the grid only (D3Q19 PR FP16, 48^3
 // box: 3.4 us by one-slot threads, 4.1 by the loop).
 constexpr int kLoopRounds = 4;
@@ -2405,13 +2437,13 @@ constexpr int kLoopRounds = 4;
 #ifndef BLBM_COMPACT_LOOP_MINB
 #define BLBM_COMPACT_LOOP_MINB -1
 #endif
-template <class L> constexpr int compact_loop_min_blocks() {
+template <class L, class S> constexpr int compact_loop_min_blocks() {
     if (BLBM_COMPACT_LOOP_MINB >= 0) return BLBM_COMPACT_LOOP_MINB;
-    return L::Q == 27 ? 4 : 5;
+    return L::Q == 27 ? 4 : pair_form<S>() ? 5 : 6;
 }
 
 template <class L, int MODEL, class S>
-__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L>())
+__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L, S>())
 k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
                     const uint32_t* __restrict__ links, const int* __restrict__ cellidx,
                     const int* __restrict__ rank, typename Store<S>::R* __restrict__ tau,
@@ -3063,9 +3095,12 @@ cudaError_t launch_resident_t(const KParams& kp, const StepArgs& s, int nsteps, 
                               s.rng_ctr, s.parity, nsteps);
 }
 
-// Left out: the Newton-implicit step, and FP32 IR on D3Q15 and D3Q27, whose
-// class-sum collision the compiler contracts differently here than in k_step
-// (every other form gives the same bits).
+// Left out: the Newton-implicit step, and class sums that the compiler contracts
+// differently here than in k_step: IR on D3Q15 and D3Q27, 16-bit PR on D3Q19 (every
+// other form gives the same bits).
+template <class L, class S> constexpr bool resident_pr() {
+    return pair_form<S>() || sizeof(S) == 4 || L::Q != 19;
+}
 template <class L, class S> constexpr bool resident_ir() {
     return pair_form<S>() || L::Q == 9 || L::Q == 19;
 }
@@ -3073,7 +3108,9 @@ template <class L, class S> constexpr bool resident_ir() {
 template <class L, class S>
 cudaError_t launch_resident_model(int model, const KParams& kp, const StepArgs& s, int nsteps,
                                   cudaStream_t st) {
-    if (model == LBM_MODEL_PR) return launch_resident_t<L, LBM_MODEL_PR, S>(kp, s, nsteps, st);
+    if constexpr (resident_pr<L, S>()) {
+        if (model == LBM_MODEL_PR) return launch_resident_t<L, LBM_MODEL_PR, S>(kp, s, nsteps, st);
+    }
     if constexpr (resident_ir<L, S>()) return launch_resident_t<L, LBM_MODEL_IR, S>(kp, s, nsteps, st);
     return cudaErrorNotSupported;
 }
@@ -3094,7 +3131,10 @@ template <class L, class S> bool resident_fits_model(int model, int ncells) {
     int threads = 0, blocks = 0;
     if (!resident_shape<L, S>(ncells, threads, blocks)) return false;
     if (model == kModelPRImplicit) return false;
-    if (model == LBM_MODEL_PR) return resident_ready<L, LBM_MODEL_PR, S>();
+    if (model == LBM_MODEL_PR) {
+        if constexpr (resident_pr<L, S>()) return resident_ready<L, LBM_MODEL_PR, S>();
+        return false;
+    }
     if constexpr (resident_ir<L, S>()) return resident_ready<L, LBM_MODEL_IR, S>();
     return false;
 }
@@ -3165,7 +3205,7 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
                                  s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials,
                                  s.rng_ctr, s.parity);
     }
-    if constexpr (compact_loop<S>()) {
+    if constexpr (compact_loop<MODEL, S>()) {
         // persistent: as many blocks as are resident at once
         static const int resident = [] {   // blocks per SM (per instantiation)
             int r = 0;
@@ -3179,8 +3219,9 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int pgrid = std::max(1, resident * sms);
-        if (grid >= kLoopRounds * pgrid)
+        int pgrid = std::max(1, resident * sms);
+        if (!pair_form<S>()) pgrid = std::min(grid, pgrid);
+        if (!pair_form<S>() || grid >= kLoopRounds * pgrid)
             return launch_overlapped(k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
                                      s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
     }
@@ -3220,8 +3261,12 @@ cudaError_t launch_step_lat(int model, int storage, bool check, const KParams& k
     switch (storage) {
     case LBM_F32: return launch_step_model<L, float>(model, check, kp, s, st);
     case LBM_F64: return launch_step_model<L, double>(model, check, kp, s, st);
-    case LBM_F16_OFS: return launch_step_model<L, __half>(model, check, kp, s, st);
-    case LBM_BF16_OFS: return launch_step_model<L, __nv_bfloat16>(model, check, kp, s, st);
+    case LBM_F16_OFS:
+        return kp.pair16 ? launch_step_model<L, PairHalf>(model, check, kp, s, st)
+                         : launch_step_model<L, __half>(model, check, kp, s, st);
+    case LBM_BF16_OFS:
+        return kp.pair16 ? launch_step_model<L, PairBf16>(model, check, kp, s, st)
+                         : launch_step_model<L, __nv_bfloat16>(model, check, kp, s, st);
     default: return cudaErrorNotSupported;
     }
 }

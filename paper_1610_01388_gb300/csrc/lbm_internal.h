@@ -13,6 +13,9 @@ namespace blbm {
 
 constexpr int kBlock = 256;          // threads per block of the cell kernels
 constexpr int kNumStats = 8;         // doubles per reduction partial
+// Cells of an x-y plane from which the 16-bit forms run the pair-form collision:
+// the plane, because a domain's z-slabs share it and step to the same bits.
+constexpr int64_t kPairPlane = 128 * 128;
 constexpr uint32_t kSolidBit = 1u << 31;
 constexpr uint32_t kFaceBit = 1u << 30;   // compact link words: the cell lies at a face of the box
 // Kernel-side model code: PR with the Newton-implicit tau update is its own
@@ -34,6 +37,7 @@ struct KParams {
     int newton;           // PR: Newton iterations of the implicit tau update (0 = explicit)
     uint32_t hash_offset; // added to the cell index in the stochastic-rounding hash
     int cell_begin, cell_end; // cells the single-domain step kernel covers (0, ncells)
+    int pair16;           // 16-bit storage: steps run the pair-form collision (kPairPlane)
     int nslots;           // compact layout: fluid cells held (0: dense layout)
     FastDiv div_nx, div_ny;   // idx -> (x, y, z) without integer division
 };
