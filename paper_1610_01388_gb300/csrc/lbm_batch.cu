@@ -144,7 +144,7 @@ int sched_ctas(int lat, int model, int storage, int unset = 0) {
 // out by the bytes of their steps, at least one each.  With one CTA per tile a
 // large group's blocks, and those of its next step that already wait for it,
 // keep the other groups off the SMs (48 domains of the serving mix, us per step:
-// 52 with a CTA per tile, 42 shared out).
+// 52 with a CTA per tile, 42 shared out, with pair-form 16-bit groups).
 constexpr int kSharedCtas = 8;
 
 // bytes a group's plain step moves at least
