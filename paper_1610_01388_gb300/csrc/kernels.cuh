@@ -209,43 +209,22 @@ __device__ __forceinline__ F2 recip(F2 x) { return F2(1.0f / x.lo(), 1.0f / x.hi
 // Arithmetic with every rounding spelled out (mad: one, fused).  The compiler
 // may neither fuse these nor take a fused one apart, so a collision written in
 // them gives the same bits in every kernel it is compiled into.
-__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ F2 add(F2 a, F2 b) { return f2_add(a, b); }
-__device__ __forceinline__ F2 sub(F2 a, F2 b) { return f2_sub(a, b); }
-__device__ __forceinline__ F2 mul(F2 a, F2 b) { return f2_mul(a, b); }
-__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) { return f2_fma(a, b, c); }
 
 // Reciprocal and (reciprocal) square root of the pair-form collision: the
 // hardware's approximation refined by the residual of its defining equation.
 // With e = 1 - x r, 1 / x = r (1 + e + e^2 + ...); with e = 1 - x r^2, 1 / sqrt(x)
-// = r (1 + e/2 + 3/8 e^2 + ...).  FP32 starts within 2^-23 (one term of the
-// first series makes it correct to an ulp; the roots are used as they are);
-// FP64 starts within 2^-19 and takes two terms, 3 and 5 operations on the FP64
-// pipe where the division and the root take 9 to 10.  Arguments are normal
-// numbers (callers guard the rest).
-__device__ __forceinline__ float rcp(float x) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return mad(r, mad(-x, r, 1.0f), r);
-}
+// = r (1 + e/2 + 3/8 e^2 + ...).  They start within 2^-19 and take two terms, 3
+// and 5 operations on the FP64 pipe where the division and the root take 9 to
+// 10.  Arguments are normal numbers (callers guard the rest).
 __device__ __forceinline__ double rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = mad(-x, r, 1.0);
     return mad(r, mad(e, e, e), r);
-}
-__device__ __forceinline__ F2 rcp(F2 x) { return F2(rcp(x.lo()), rcp(x.hi())); }
-__device__ __forceinline__ float rcp_root(float x) {
-    float r;
-    asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
 }
 __device__ __forceinline__ double rcp_root(double x) {
     double r;
@@ -253,14 +232,8 @@ __device__ __forceinline__ double rcp_root(double x) {
     const double e = mad(-mul(x, r), r, 1.0);
     return mad(mul(r, e), mad(0.375, e, 0.5), r);
 }
-__device__ __forceinline__ float root(float x) {
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 // a > b for numbers >= 0, whose bits order as integers: an FP64 compare would
 // take its turn on the FP64 pipe like an add
-__device__ __forceinline__ bool above(float a, float b) { return a > b; }
 __device__ __forceinline__ bool above(double a, double b) {
     return __double_as_longlong(a) > __double_as_longlong(b);
 }
@@ -356,28 +329,6 @@ template <> struct Store<__nv_bfloat16> {
     static __device__ __forceinline__ __nv_bfloat16 enc(double off, double w) { return __double2bfloat16(off / w); }
     static __device__ __forceinline__ double dec(__nv_bfloat16 v, double w) { return (double)__bfloat162float(v) * w; }
 };
-
-// The same storage, stepped with the pair-form collision (see pair_form).
-struct PairHalf {
-    __half v;
-};
-struct PairBf16 {
-    __nv_bfloat16 v;
-};
-template <class T, class B> struct PairStore : Store<B> {
-    template <class L, int i> static __device__ __forceinline__ float ld(const T* p) {
-        return Store<B>::template ld<L, i>(&p->v);
-    }
-    template <class L, int i> static __device__ __forceinline__ void st(T* p, float v, uint32_t rnd) {
-        Store<B>::template st<L, i>(&p->v, v, rnd);
-    }
-    template <class L, int i>
-    static __device__ __forceinline__ void st2(T* pi, T* po, float vi, float vo, uint32_t rnd) {
-        Store<B>::template st2<L, i>(&pi->v, &po->v, vi, vo, rnd);
-    }
-};
-template <> struct Store<PairHalf> : PairStore<PairHalf, __half> {};
-template <> struct Store<PairBf16> : PairStore<PairBf16, __nv_bfloat16> {};
 
 // Rheology constants in the arithmetic type, derived on the host in FP64.
 template <class R> struct Coef {
@@ -546,20 +497,14 @@ template <class R> struct Tens {
     R xx, yy, zz, xy, xz, yz;
 };
 
-// Which form of the collision a domain runs.  Pair form (below): FP64, whose
+// Which form of the collision a storage runs.  Pair form (below): FP64, whose
 // step is bound by the FP64 pipe (D3Q27 IR, duct 1 x 64 x 64: 24.5 -> 19.0 us a
-// step; D2Q9 PR, 80 x 80: 15.6 -> 13.5), and the 16-bit forms of domains with large
-// x-y planes (kPairPlane), whose step is bound by instruction issue (us a step,
-// class -> pair form, D3Q27 duct 256 x 128 x 128: PR FP16 109.9 -> 99.1, IR 91.9 ->
-// 87.0; D3Q19 PR FP16, compact porous 256^3: 319 -> 260).  Errors against FP64 did
-// not grow.  FP32 storage and the 16-bit forms of smaller domains keep the
-// class sums, which are bit for bit the results they have always had: the pair
-// form gained FP32 0.4-3 % (its large steps are bound by HBM), small domains are
-// bound by latency, and near a steady state, which they reach, the residual
-// shows any change of rounding.
-template <class S> __host__ __device__ constexpr bool pair_form() {
-    return sizeof(S) == 8 || std::is_same<S, PairHalf>::value || std::is_same<S, PairBf16>::value;
-}
+// step; D2Q9 PR, 80 x 80: 15.6 -> 13.5).  FP32 arithmetic keeps the class sums.  The
+// pair form gained FP32 storage 0.4-3 % (its large steps are bound by HBM) and
+// the 16-bit forms 5-20 %, but it rounds in another order: near a steady state the
+// FP32 residual shows that, and 16-bit storage picks the other neighbour here and
+// there, so that a domain would depend on which form its size, or a batch, runs.
+template <class S> __host__ __device__ constexpr bool pair_form() { return sizeof(S) == 8; }
 
 // Grouped sums: populations are added once per velocity class (c_x = +1, -1,
 // 0; c_y = +-1; c_z = +-1; sign of c_x c_y, c_x c_z, c_y c_z) and the moments
@@ -670,13 +615,9 @@ template <class L> __host__ __device__ constexpr int part_place(int p) {
 }
 
 // b x and y + b x for a compile-time factor b (a plain x, y + x where it is 1)
-template <class R, class B> __device__ __forceinline__ R scale(B b, R x) {
-    if (b == B(1)) return x;
-    return mul(x, R(b));
-}
-template <class R, class B> __device__ __forceinline__ R axpy(B b, R x, R y) {
-    if (b == B(1)) return add(y, x);
-    return mad(x, R(b), y);
+__device__ __forceinline__ double scale(double b, double x) { return b == 1.0 ? x : mul(x, b); }
+__device__ __forceinline__ double axpy(double b, double x, double y) {
+    return b == 1.0 ? add(y, x) : mad(x, b, y);
 }
 
 // Pair form: f[i] = f_i + f_o and f[o] = f_i - f_o for every opposite pair
@@ -693,45 +634,38 @@ template <class L, class R> __device__ __forceinline__ void to_pairs(R (&f)[L::Q
 
 // Moments from the pair form.  Per family the members are first combined by
 // sums and differences (xx + yy against xy of a face plane; the four corners
-// by one 4-point butterfly), then scaled once by the family's beta (memory
-// units to offsets) and added to the axis terms.  On D3Q27 this takes 82 adds
-// where adding every population to its velocity classes took 96, and 26 of
-// them are the pair sums that the TRT collision needs anyway; in the 16-bit
-// forms the classes' 96 multiply-adds by beta become 20.
-template <class L, class S, class R>
-__device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
+// by one 4-point butterfly), then added to the axis terms.  On D3Q27 this takes
+// 82 adds where adding every population to its velocity classes took 96, and 26
+// of them are the pair sums that the TRT collision needs anyway.
+template <class L, class R> __device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
     constexpr int F = Fam<L>::face, C = Fam<L>::corner;
-    constexpr auto b0 = Store<S>::template beta<L, 0>();
-    constexpr auto bA = Store<S>::template beta<L, 1>();
-    constexpr auto bF = Store<S>::template beta<L, (F ? F : 1)>();
-    constexpr auto bC = Store<S>::template beta<L, (C ? C : 1)>();
     Mom<R> m;
     if constexpr (L::D == 2) {
-        const R XY = scale(bF, add(f[F], f[F + 2]));
-        m.xx = axpy(bA, f[1], XY);
-        m.yy = axpy(bA, f[3], XY);
-        m.d = add(m.xx, axpy(b0, f[0], scale(bA, f[3])));
-        m.xy = scale(bF, sub(f[F], f[F + 2]));
-        m.jx = axpy(bA, f[2], scale(bF, add(f[F + 1], f[F + 3])));
-        m.jy = axpy(bA, f[4], scale(bF, sub(f[F + 1], f[F + 3])));
+        const R XY = add(f[F], f[F + 2]);
+        m.xx = add(XY, f[1]);
+        m.yy = add(XY, f[3]);
+        m.d = add(m.xx, add(f[3], f[0]));
+        m.xy = sub(f[F], f[F + 2]);
+        m.jx = add(add(f[F + 1], f[F + 3]), f[2]);
+        m.jy = add(sub(f[F + 1], f[F + 3]), f[4]);
         m.zz = R(0);
         m.jz = R(0);
         m.xz = R(0);
         m.yz = R(0);
     } else {
-        R X, Y, Z, rest = scale(bA, add(f[3], f[5]));   // X: diagonal sums beyond the axis pairs
+        R X, Y, Z, rest = add(f[3], f[5]);   // X: diagonal sums beyond the axis pairs
         R jx, jy, jz;
         if constexpr (C != 0) {
             const R ab = add(f[C], f[C + 2]), amb = sub(f[C], f[C + 2]);
             const R ce = add(f[C + 4], f[C + 6]), cme = sub(f[C + 4], f[C + 6]);
-            X = scale(bC, add(ab, ce));
-            m.xy = scale(bC, sub(ab, ce));
-            m.xz = scale(bC, add(amb, cme));
-            m.yz = scale(bC, sub(amb, cme));
+            X = add(ab, ce);
+            m.xy = sub(ab, ce);
+            m.xz = add(amb, cme);
+            m.yz = sub(amb, cme);
             const R dp = add(f[C + 1], f[C + 3]), dq = sub(f[C + 5], f[C + 7]);
-            jx = scale(bC, add(dp, dq));
-            jy = scale(bC, sub(dp, dq));
-            jz = scale(bC, add(sub(f[C + 1], f[C + 3]), add(f[C + 5], f[C + 7])));
+            jx = add(dp, dq);
+            jy = sub(dp, dq);
+            jz = add(sub(f[C + 1], f[C + 3]), add(f[C + 5], f[C + 7]));
             Y = X;
             Z = X;
         }
@@ -742,36 +676,36 @@ __device__ __forceinline__ Mom<R> pair_moments(const R (&f)[L::Q]) {
             const R fy = add(sub(f[F + 1], f[F + 3]), add(f[F + 9], f[F + 11]));
             const R fz = add(sub(f[F + 5], f[F + 7]), sub(f[F + 9], f[F + 11]));
             const R xs = add(sxy, sxz), ys = add(sxy, syz), zs = add(sxz, syz);
-            rest = axpy(bF, syz, rest);
+            rest = add(rest, syz);
             if constexpr (C != 0) {
-                X = axpy(bF, xs, X);
-                Y = axpy(bF, ys, Y);
-                Z = axpy(bF, zs, Z);
-                m.xy = axpy(bF, oxy, m.xy);
-                m.xz = axpy(bF, oxz, m.xz);
-                m.yz = axpy(bF, oyz, m.yz);
-                jx = axpy(bF, fx, jx);
-                jy = axpy(bF, fy, jy);
-                jz = axpy(bF, fz, jz);
+                X = add(X, xs);
+                Y = add(Y, ys);
+                Z = add(Z, zs);
+                m.xy = add(m.xy, oxy);
+                m.xz = add(m.xz, oxz);
+                m.yz = add(m.yz, oyz);
+                jx = add(jx, fx);
+                jy = add(jy, fy);
+                jz = add(jz, fz);
             } else {
-                X = scale(bF, xs);
-                Y = scale(bF, ys);
-                Z = scale(bF, zs);
-                m.xy = scale(bF, oxy);
-                m.xz = scale(bF, oxz);
-                m.yz = scale(bF, oyz);
-                jx = scale(bF, fx);
-                jy = scale(bF, fy);
-                jz = scale(bF, fz);
+                X = xs;
+                Y = ys;
+                Z = zs;
+                m.xy = oxy;
+                m.xz = oxz;
+                m.yz = oyz;
+                jx = fx;
+                jy = fy;
+                jz = fz;
             }
         }
-        m.xx = axpy(bA, f[1], X);
-        m.yy = axpy(bA, f[3], Y);
-        m.zz = axpy(bA, f[5], Z);
-        m.d = add(m.xx, axpy(b0, f[0], rest));
-        m.jx = axpy(bA, f[2], jx);
-        m.jy = axpy(bA, f[4], jy);
-        m.jz = axpy(bA, f[6], jz);
+        m.xx = add(X, f[1]);
+        m.yy = add(Y, f[3]);
+        m.zz = add(Z, f[5]);
+        m.d = add(m.xx, add(rest, f[0]));
+        m.jx = add(jx, f[2]);
+        m.jy = add(jy, f[4]);
+        m.jz = add(jz, f[6]);
     }
     return m;
 }
@@ -781,7 +715,7 @@ template <class L, class S, class R = typename Store<S>::R>
 __device__ __forceinline__ Mom<R> moments(R (&f)[L::Q]) {
     if constexpr (pair_form<S>()) {
         to_pairs<L>(f);
-        return pair_moments<L, S, R>(f);
+        return pair_moments<L, R>(f);
     } else {
         return class_moments<L, S, R>(f);
     }
@@ -849,36 +783,21 @@ template <class L, class R> __device__ __forceinline__ R trace(const Tens<R>& t)
 // sum per axis pair, two per face plane, one 4-point butterfly for the
 // corners, instead of c.u, its square and c.T.c per pair (D3Q27: 23 adds
 // against 150 operations).  put(i, e, cq, wo) stores pair i, its even part e
-// (weighted) and its odd part wo cq.  Where w_i in memory units is the same for
-// every direction (the 16-bit forms) it goes into the six numbers and q once,
-// and wo = 1.
+// (weighted) and its odd part wo cq.
 // PART >= 0: only the pairs of that part (the compiler drops the rest).
 template <class L, class S, class R, int PART = -1, class Put>
 __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R qz, Put&& put) {
     constexpr int F = Fam<L>::face, C = Fam<L>::corner;
-    constexpr bool same = sizeof(S) == 2;   // gam, god do not depend on the direction
-    constexpr auto g0 = Store<S>::template gam<L, 1>();
-    constexpr auto o0 = Store<S>::template god<L, 1>();
-    using B = std::remove_const_t<decltype(g0)>;
-    if constexpr (same) {
-        e0 = scale(g0, e0);
-        qx = scale(o0, qx);
-        qy = scale(o0, qy);
-        if constexpr (L::D == 3) qz = scale(o0, qz);
-    }
 #define BLBM_I(n) std::integral_constant<int, (n)>{}
     // Even parts carry their weights: per family gam enters e0's sums once (the
     // axis family through its constants) and the off-diagonal terms' constant.
-    constexpr B gA = same ? B(1) : Store<S>::template gam<L, 1>();
-    constexpr B gF = same ? B(1) : Store<S>::template gam<L, (F ? F : 1)>();
-    constexpr B gC = same ? B(1) : Store<S>::template gam<L, (C ? C : 1)>();
-    constexpr B unit = same ? g0 : B(1);
-    const R k = R(B(4.5) * unit), kA = R(B(4.5) * gA * unit);
-    const R kF = R(B(9) * gF * unit), kC = R(B(9) * gC * unit);
+    constexpr R gA = Store<S>::template gam<L, 1>();
+    constexpr R gF = Store<S>::template gam<L, (F ? F : 1)>();
+    constexpr R gC = Store<S>::template gam<L, (C ? C : 1)>();
+    constexpr R k = 4.5, kA = 4.5 * gA, kF = 9.0 * gF, kC = 9.0 * gC;
     auto pair = [&](auto I, R e, R cq) {
         constexpr int i = decltype(I)::value;
         if constexpr (PART >= 0 && pair_part<L>((i - 1) / 2) != PART) return;
-        else if constexpr (same) put(I, e, cq, B(1));
         else put(I, e, cq, Store<S>::template god<L, i>());
     };
     const R eA = scale(gA, e0);
@@ -923,30 +842,19 @@ __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R
 // from |T|^2, returns k1 = as / 2 - asg - 1 and asg.  Both factors are linear in
 // 1 / |T| (-(|T| - sqrt2 sigma_y) a / |T| = sqrt2 sigma_y a / |T| - a), and so is
 // k1: one reciprocal square root and two multiply-adds.
-template <class R>
-__device__ __forceinline__ void ir_yield(const Coef<typename Lanes<R>::Sc>& c, R tn2, R& k1_out,
-                                         R& asg_out) {
-    using Sc = typename Lanes<R>::Sc;
-    Sc k1[Lanes<R>::n], asg[Lanes<R>::n];
-#pragma unroll
-    for (int k = 0; k < Lanes<R>::n; ++k) {
-        const Sc t2 = Lanes<R>::get(tn2, k);
-        k1[k] = Sc(0);
-        asg[k] = Sc(-1);
-        // (an FP64 |T| below 1e-145 counts as not yielded: see rcp_root)
-        if (above(t2, Sc(sizeof(Sc) == 8 ? 1e-290 : 0.0)) && !above(c.s2y2, t2)) {
-            const Sc it = rcp_root(t2);
-            k1[k] = mad(c.ir_ks, it, c.ir_k);
-            asg[k] = mad(-c.ir_bs, it, -c.ir_bn);
-        }
+__device__ __forceinline__ void ir_yield(const Coef<double>& c, double t2, double& k1, double& asg) {
+    k1 = 0.0;
+    asg = -1.0;
+    // (|T| below 1e-145 counts as not yielded: see rcp_root)
+    if (above(t2, 1e-290) && !above(c.s2y2, t2)) {
+        const double it = rcp_root(t2);
+        k1 = mad(c.ir_ks, it, c.ir_k);
+        asg = mad(-c.ir_bs, it, -c.ir_bn);
     }
-    k1_out = Lanes<R>::make(k1);
-    asg_out = Lanes<R>::make(asg);
 }
 
 // ---------------------------------------------------------------------------
-// IR collision (Secs. 2.3, 3.2).  f: memory units in, memory units out.  R is
-// the arithmetic type: one cell (float, double) or two cells (F2).
+// IR collision (Secs. 2.3, 3.2).  f: memory units in, memory units out.
 // What the pairs need from the moments: e0, N and q of pair_terms.
 template <class L, class R>
 __device__ __forceinline__ void ir_terms(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
@@ -965,7 +873,7 @@ __device__ __forceinline__ void ir_terms(const Coef<typename Lanes<R>::Sc>& c, u
     const Tens<R> P = dynamic<L, R>(m);
     const Tens<R> T = noneq<L, R>(P, -px, -py, -pz, ux, uy, uz, flags);
     R k1, asg;   // k1 - 1 with the k1 below
-    ir_yield<R>(c, square<L, R>(T), k1, asg);
+    ir_yield(c, square<L, R>(T), k1, asg);
     // A = -sigma_bar + s/2 = k1 T + k2 I with sigma_bar = sigma - tr(sigma)/D I;
     // N = rho u u + A gives f_eq + f^sigma = w_i (d - 3/2 tr N + 9/2 c.N.c + 3 rho c.u) + w_i,
     // and rho u u = P - T
@@ -1074,48 +982,39 @@ __device__ __forceinline__ void pr_rates(const Coef<typename Lanes<R>::Sc>& c, R
     wm_out = Lanes<R>::make(wm_);
 }
 
-// The same for the pair form.  itau: 1 / (previous step's tau).  FP64 takes
-// both rates from one division (a product of two moderate numbers; beyond that
-// range, which only an extreme m reaches, from two).
-template <bool IMPLICIT, class R>
-__device__ __forceinline__ void pair_pr_rates(const Coef<typename Lanes<R>::Sc>& c, R tn2, R inv,
-                                              R itau, R& tau, R& wp_out, R& wm_out) {
-    using Sc = typename Lanes<R>::Sc;
-    Sc tau_[Lanes<R>::n], wp_[Lanes<R>::n], wm_[Lanes<R>::n];
-#pragma unroll
-    for (int k = 0; k < Lanes<R>::n; ++k) {
-        const Sc tt = root(mul(Sc(4.5), Lanes<R>::get(tn2, k)));   // 1.5 sqrt(2 T:T)
-        Sc gd = mul(Lanes<R>::get(itau, k), tt);
-        const Sc sy_rho = mul(c.sigma_y, Lanes<R>::get(inv, k));
-        if constexpr (IMPLICIT) gd = pr_newton(c, tt, gd, sy_rho);
-        Sc nu;
-        if (!above(c.gdot_c, gd)) {
-            const Sc y = mul(sy_rho, -expm1(mul(-c.m, gd)));
-            if (sizeof(Sc) == 4 || above(gd, Sc(1e-290))) nu = mad(y, rcp(gd), c.nu_p);
-            else nu = add(c.nu_p, y / gd);
-        } else {
-            const Sc nu0 = mad(c.m, sy_rho, c.nu_p);
-            const Sc nuc = mad(sy_rho, c.e_c, c.nu_p);
-            const Sc s = mul(gd, c.inv_gc);
-            nu = mad(mul(sub(c.gdot_c, gd), c.inv_gc), nu0, mul(s, nuc));
-        }
-        const Sc tn = mad(Sc(3), nu, Sc(0.5));
-        // 1 / tau_odd with tau_odd = 1/2 + Lambda / (tau - 1/2) is tm / odd
-        const Sc tm = sub(tn, Sc(0.5));
-        const Sc odd = mad(Sc(0.5), tm, c.magic);
-        if (sizeof(Sc) == 8 && !above(tn, Sc(1e30))) {
-            const Sc r = rcp(mul(tn, odd));
-            wp_[k] = mul(r, odd);
-            wm_[k] = mul(tm, mul(r, tn));
-        } else {
-            wp_[k] = rcp(tn);
-            wm_[k] = mul(tm, rcp(odd));
-        }
-        tau_[k] = tn;
+// The same for the pair form.  itau: 1 / (previous step's tau).  Both rates from
+// one reciprocal (a product of two moderate numbers; beyond that range, which
+// only an extreme m reaches, from two).
+template <bool IMPLICIT>
+__device__ __forceinline__ void pair_pr_rates(const Coef<double>& c, double tn2, double inv, double itau,
+                                              double& tau, double& wp, double& wm) {
+    const double tt = root(mul(4.5, tn2));   // 1.5 sqrt(2 T:T)
+    double gd = mul(itau, tt);
+    const double sy_rho = mul(c.sigma_y, inv);
+    if constexpr (IMPLICIT) gd = pr_newton(c, tt, gd, sy_rho);
+    double nu;
+    if (!above(c.gdot_c, gd)) {
+        const double y = mul(sy_rho, -expm1(mul(-c.m, gd)));
+        if (above(gd, 1e-290)) nu = mad(y, rcp(gd), c.nu_p);
+        else nu = add(c.nu_p, y / gd);
+    } else {
+        const double nu0 = mad(c.m, sy_rho, c.nu_p);
+        const double nuc = mad(sy_rho, c.e_c, c.nu_p);
+        const double s = mul(gd, c.inv_gc);
+        nu = mad(mul(sub(c.gdot_c, gd), c.inv_gc), nu0, mul(s, nuc));
     }
-    tau = Lanes<R>::make(tau_);
-    wp_out = Lanes<R>::make(wp_);
-    wm_out = Lanes<R>::make(wm_);
+    tau = mad(3.0, nu, 0.5);
+    // 1 / tau_odd with tau_odd = 1/2 + Lambda / (tau - 1/2) is tm / odd
+    const double tm = sub(tau, 0.5);
+    const double odd = mad(0.5, tm, c.magic);
+    if (!above(tau, 1e30)) {
+        const double r = rcp(mul(tau, odd));
+        wp = mul(r, odd);
+        wm = mul(tm, mul(r, tau));
+    } else {
+        wp = rcp(tau);
+        wm = mul(tm, rcp(odd));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1128,21 +1027,14 @@ __device__ __forceinline__ void pr_terms(const Coef<typename Lanes<R>::Sc>& c, u
                                          const Mom<R>& m, R& tau, R& K0, Tens<R>& N, R (&q)[3], R& wp,
                                          R& wm, R (&ur)[3]) {
     const R rho = add(R(1), m.d);
-    R inv, itau;   // 1 / rho, 1 / tau_old
-    if constexpr (sizeof(typename Lanes<R>::Sc) == 8) {
-        const R both = rcp(mul(rho, tau));   // one FP64 reciprocal for both
-        inv = mul(both, tau);
-        itau = mul(both, rho);
-    } else {
-        inv = rcp(rho);
-        itau = rcp(tau);
-    }
+    const R both = rcp(mul(rho, tau));   // one reciprocal for both 1 / rho and 1 / tau_old
+    const R inv = mul(both, tau), itau = mul(both, rho);
     const R ux = mul(m.jx, inv), uy = mul(m.jy, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(m.jz, inv);
     {
         const Tens<R> T = noneq<L, R>(dynamic<L, R>(m), -m.jx, -m.jy, -m.jz, ux, uy, uz, flags);
-        pair_pr_rates<IMPLICIT, R>(c, square<L, R>(T), inv, itau, tau, wp, wm);
+        pair_pr_rates<IMPLICIT>(c, square<L, R>(T), inv, itau, tau, wp, wm);
     }
     const R gx = R(c.g[0]), gy = R(c.g[1]);
     R gz = R(0);
@@ -1203,7 +1095,8 @@ __device__ __forceinline__ void pair_collide_pr(const Coef<typename Lanes<R>::Sc
 }
 
 // ---------------------------------------------------------------------------
-// The same two collisions on class sums, for FP32 storage (see pair_form).
+// The same two collisions on class sums, for FP32 arithmetic (see pair_form).  R is
+// the arithmetic type: one cell (float) or two cells (F2).
 template <class L, class R> __device__ __forceinline__ R tnorm2(const Tens<R>& T) {
     R s = T.xx * T.xx + T.yy * T.yy + R(2) * T.xy * T.xy;
     if constexpr (L::D == 3) s += T.zz * T.zz + R(2) * (T.xz * T.xz + T.yz * T.yz);
@@ -1442,9 +1335,7 @@ __device__ __forceinline__ void step_begin(int& n) {
 // smaller lattices keep 1280 (10 x 128, 5 x 256, 2 x 512): D3Q19 PR then
 // takes 48 registers without spilling and measured 7-9 % faster than at 64
 // (porous box 256^3: FP32 466 -> 430 us, FP16 440 -> 401 us; duct
-// 256 x 128 x 128: FP32 113.5 -> 105.7 us).  Their 16-bit PR steps in the pair form
-// keep 1536 (40 registers, up to 16 bytes spilled): duct 256 x 128 x 128, D3Q19
-// 87.0 -> 80.3 us, D3Q15 74.6 -> 70.0; porous 160^3 D3Q19 91.8 -> 86.0.  IR (40-48 registers) and FP64
+// 256 x 128 x 128: FP32 113.5 -> 105.7 us).  IR (40-48 registers) and FP64
 // arithmetic (which these caps would make spill) are left to the allocator.
 // BLBM_PR_MINB / BLBM_IR_MINB override at build time.
 #ifndef BLBM_PR_MINB
@@ -1459,7 +1350,7 @@ template <class L, int MODEL, class S, bool CHECK, int BLOCK> constexpr int step
     if (std::is_same<typename Store<S>::R, double>::value) return 0;
     if (BLBM_PR_MINB >= 0) return BLBM_PR_MINB;
     if (L::Q == 27 || CHECK) return BLOCK == 128 ? 9 : 1024 / BLOCK;   // check steps: no spill
-    return (sizeof(S) == 2 && pair_form<S>() ? 1536 : 1280) / BLOCK;
+    return 1280 / BLOCK;
 }
 
 // Stores one cell's outgoing populations at element n of the planes: the
@@ -1587,14 +1478,20 @@ k_step(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
     const KParams& kp = a.kp;
     int idx = (RANGE ? kp.cell_begin : 0) + (int)(blockIdx.x * BLOCK + threadIdx.x);
     const bool inside = idx < (RANGE ? kp.cell_end : kp.ncells);
-    const uint32_t lk = inside ? __ldg(links + idx) : kSolidBit;
-    step_begin(idx);
-    uint32_t rnd = 0u;
-    if constexpr (Store<S>::kStochastic) {
+    uint32_t lk = kSolidBit, rnd = 0u;
+    if constexpr (!Store<S>::kStochastic) {
+        if (inside) lk = __ldg(links + idx);
+        step_begin(idx);
+    } else {
+        step_begin(idx);
         // this launch reads counter[parity] and leaves counter + 1 for the next
         const uint32_t seed = rng_ctr[parity];
         if (blockIdx.x == 0 && threadIdx.x == 0) rng_ctr[parity ^ 1] = seed + 1u;
         rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ (seed * 0x9e3779b9u));
+        // behind the hash: before it, the PR step is slower than the wait it hides
+        // (FP16 duct 256 x 128 x 128, D3Q19 92.6 us against 88.8; D3Q27 at 256 threads
+        // 128.4 against 119.0)
+        if (inside) lk = __ldg(links + idx);
     }
     const bool active = !(lk & kSolidBit);
     R acc[kNumStats];
@@ -2210,102 +2107,96 @@ k_resident_split(const KArgs a, const double* src, double* dst, const uint32_t* 
 // 18 and 26.  The wrap in x is the exception: a warp that holds a cell at
 // either end of a row looks every neighbour up.
 //
-// ROWS = false leaves the row paths out.
-//
-// In the pair-form 16-bit steps, bound by issue, the link word says whether the cell
-// lies at any face of the box (kFaceBit); a warp without such cells needs no
-// coordinates, its rows being at constant offsets (D3Q19 256^3 porous box: IR
-// 248 -> 225 us, PR 281 -> 261).  In the FP32 IR step, bound by latency, that form
-// spilled (323 -> 332 us).
+// ROWS = false leaves the row paths out: beside them the compiler contracts some
+// class sums differently, and results would move by a rounding.  So the 16-bit
+// forms look every neighbour up, in a step and in a read-back alike.
 template <class L> __host__ __device__ constexpr int dir_index(int cx, int cy, int cz) {
     for (int i = 0; i < L::Q; ++i)
         if (L::cx(i) == cx && L::cy(i) == cy && L::cz(i) == cz) return i;
     return -1;
 }
-template <class L, class S, bool ROWS = true, class Src>
+template <class L, class S, bool ROWS = sizeof(S) != 2, class Src>
 __device__ __forceinline__ void gather_compact(const KParams& kp, const Src& P, uint32_t lk,
                                                int idx, int slot, const int* __restrict__ rank,
                                                typename Store<S>::R (&v)[L::Q]) {
-    constexpr bool by_face = sizeof(S) == 2 && pair_form<S>();
-    PullOffsets o{0, 0, 0, 0, 0, 0};
-    bool edge;   // this lane's cell keeps the warp from the row paths
-    if constexpr (by_face) {
-        edge = (lk & kFaceBit) != 0u;
-    } else {
-        o = pull_offsets(kp, idx);
-        edge = o.dxm != -1 || o.dxp != 1;   // the x neighbours wrap
-    }
+    const PullOffsets o = pull_offsets(kp, idx);
     // the cell's own rank word: each neighbour's is one multiply-add from it
     // (against an add and a sign-extended 64-bit address per neighbour: 2-8 %
     // faster steps on 256^3 porous boxes)
     const int* __restrict__ rk = rank + idx;
     v[0] = Store<S>::template ld<L, 0>(P.template at<0>(slot));
-    const unsigned warp = __activemask();
-    const int nx = kp.nx, nxy = kp.nx * kp.ny;
-    // by rows (cy, cz): f(direction, slot of its source if that is fluid)
-    auto rows = [&](bool solid_free, auto&& f) {
-        static_for<0, 9>([&](auto J) {
-            constexpr int cy = decltype(J)::value % 3 - 1, cz = decltype(J)::value / 3 - 1;
-            constexpr int im = dir_index<L>(1, cy, cz), i0 = dir_index<L>(0, cy, cz),
-                          ip = dir_index<L>(-1, cy, cz);
-            if constexpr (im >= 0 || i0 >= 0 || ip >= 0) {
-                int c = slot, after = slot + 1;
-                if constexpr (cy != 0 || cz != 0) {
-                    int off = 0;
-                    if constexpr (by_face) {
-                        off = -(cy * nx + cz * nxy);
-                    } else {
+    if constexpr (ROWS) {
+        // by rows (cy, cz): f(direction, slot of its source if that is fluid)
+        auto rows = [&](bool solid_free, auto&& f) {
+            static_for<0, 9>([&](auto J) {
+                constexpr int cy = decltype(J)::value % 3 - 1, cz = decltype(J)::value / 3 - 1;
+                constexpr int im = dir_index<L>(1, cy, cz), i0 = dir_index<L>(0, cy, cz),
+                              ip = dir_index<L>(-1, cy, cz);
+                if constexpr (im >= 0 || i0 >= 0 || ip >= 0) {
+                    int c = slot, after = slot + 1;
+                    if constexpr (cy != 0 || cz != 0) {
+                        int off = 0;
                         if constexpr (cy > 0) off += o.dym;
                         if constexpr (cy < 0) off += o.dyp;
                         if constexpr (cz > 0) off += o.dzm;
                         if constexpr (cz < 0) off += o.dzp;
+                        c = __ldg(rk + off);
+                        if (i0 >= 0 && solid_free) {     // the row's own cell is a source, hence fluid
+                            after = c + 1;
+                        } else {
+                            const int s = c >> 31;       // -1 for a solid cell
+                            c ^= s;
+                            after = c + 1 + s;
+                        }
                     }
-                    c = __ldg(rk + off);
-                    if (i0 >= 0 && solid_free) {     // the row's own cell is a source, hence fluid
-                        after = c + 1;
-                    } else {
-                        const int s = c >> 31;       // -1 for a solid cell
-                        c ^= s;
-                        after = c + 1 + s;
-                    }
+                    if constexpr (im >= 0) f(std::integral_constant<int, im>{}, c - 1);
+                    if constexpr (i0 > 0) f(std::integral_constant<int, i0>{}, c);
+                    if constexpr (ip >= 0) f(std::integral_constant<int, ip>{}, after);
                 }
-                if constexpr (im >= 0) f(std::integral_constant<int, im>{}, c - 1);
-                if constexpr (i0 > 0) f(std::integral_constant<int, i0>{}, c);
-                if constexpr (ip >= 0) f(std::integral_constant<int, ip>{}, after);
-            }
-        });
-    };
-    if constexpr (!ROWS) edge = true;
-    if (ROWS && __all_sync(warp, lk == 0u && !edge)) {
-        rows(true, [&](auto I, int k) {
-            constexpr int i = decltype(I)::value;
-            v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
-        });
-    } else if (ROWS && __all_sync(warp, !edge)) {
-        rows(false, [&](auto I, int k) {
-            constexpr int i = decltype(I)::value;
-            const S* p = ((lk >> i) & 1u) ? P.template at<L::opp(i)>(slot) : P.template at<i>(k);
-            v[i] = Store<S>::template ld<L, i>(p);   // opposite planes share w_i
-        });
-    } else {
-        const PullOffsets w = by_face ? pull_offsets(kp, idx) : o;
-        if (!ROWS && __all_sync(warp, lk == 0u)) {
-            static_for<1, L::Q>([&](auto I) {
+            });
+        };
+        const bool edge = o.dxm != -1 || o.dxp != 1;   // the x neighbours wrap
+        const unsigned warp = __activemask();
+        if (__all_sync(warp, lk == 0u && !edge)) {
+            rows(true, [&](auto I, int k) {
                 constexpr int i = decltype(I)::value;
-                const int k = __ldg(rk + w.template of<L, i>());
                 v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
             });
-            return;
+        } else if (__all_sync(warp, !edge)) {
+            rows(false, [&](auto I, int k) {
+                constexpr int i = decltype(I)::value;
+                const S* p = ((lk >> i) & 1u) ? P.template at<L::opp(i)>(slot) : P.template at<i>(k);
+                v[i] = Store<S>::template ld<L, i>(p);   // opposite planes share w_i
+            });
+        } else {
+            static_for<1, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                const S* p;
+                if ((lk >> i) & 1u)
+                    p = P.template at<L::opp(i)>(slot);
+                else
+                    p = P.template at<i>(__ldg(rk + o.template of<L, i>()));
+                v[i] = Store<S>::template ld<L, i>(p);
+            });
         }
-        static_for<1, L::Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            const S* p;
-            if ((lk >> i) & 1u)
-                p = P.template at<L::opp(i)>(slot);
-            else
-                p = P.template at<i>(__ldg(rk + w.template of<L, i>()));
-            v[i] = Store<S>::template ld<L, i>(p);
-        });
+    } else {
+        if (__all_sync(__activemask(), lk == 0u)) {
+            static_for<1, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                const int k = __ldg(rk + o.template of<L, i>());
+                v[i] = Store<S>::template ld<L, i>(P.template at<i>(k));
+            });
+        } else {
+            static_for<1, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                const S* p;
+                if ((lk >> i) & 1u)
+                    p = P.template at<L::opp(i)>(slot);
+                else
+                    p = P.template at<i>(__ldg(rk + o.template of<L, i>()));
+                v[i] = Store<S>::template ld<L, i>(p);
+            });
+        }
     }
 }
 
@@ -2324,11 +2215,8 @@ __device__ __forceinline__ void compact_cell(const KParams& kp, const Coef<typen
         for (int d = 0; d < 3; ++d) up[d] = usnap[(int64_t)d * kp.plane + slot];
     }
     R f[L::Q];
-    // The class sums of D3Q27 FP32 IR and of the 16-bit forms look every neighbour
-    // up: beside the row paths the compiler contracts them differently, and
-    // results would move by a rounding (D3Q27 FP32 IR, 160^3 porous box: 124 us, 118
-    // with the row paths)
-    constexpr bool rows = pair_form<S>() || (sizeof(S) == 4 && !(L::Q == 27 && MODEL == LBM_MODEL_IR));
+    // so does the D3Q27 FP32 IR step (160^3 porous box: 124 us, 118 with the row paths)
+    constexpr bool rows = sizeof(S) != 2 && !(sizeof(S) == 4 && L::Q == 27 && MODEL == LBM_MODEL_IR);
     gather_compact<L, S, rows>(kp, src, lk, idx, slot, rank, f);
     R drho, ur[3];
     if constexpr (MODEL != LBM_MODEL_IR) {
@@ -2355,8 +2243,7 @@ template <class L, int MODEL, class S, bool CHECK> constexpr int compact_min_blo
     // the allocator's 38 registers.  D3Q27 IR: 4 blocks (64 registers; 48
     // spilled and ran slower).  PR keeps the dense step's budget (6 blocks
     // spilled and made the D3Q19 FP16 step 7 % slower).
-    // Pair-form 16-bit IR up to 19 velocities spills at 6 (large domains run the loop).
-    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q == 27 ? 4 : pair_form<S>() ? 5 : 6;
+    if (MODEL == LBM_MODEL_IR && !CHECK) return L::Q <= 19 ? 6 : 4;
     return step_min_blocks<L, MODEL, S, CHECK, kBlock>();
 }
 
@@ -2371,9 +2258,9 @@ template <class L, int MODEL, class S, bool CHECK> constexpr int compact_min_blo
 #ifndef BLBM_COMPACT_BLOCK
 #define BLBM_COMPACT_BLOCK 0
 #endif
-template <class L, int MODEL, class S> constexpr int compact_block() {
+template <class L, int MODEL> constexpr int compact_block() {
     if (BLBM_COMPACT_BLOCK > 0) return BLBM_COMPACT_BLOCK;
-    if (MODEL != LBM_MODEL_IR || sizeof(S) == 2) return 128;
+    if (MODEL != LBM_MODEL_IR) return 128;
     return L::Q <= 19 ? 512 : 256;
 }
 
@@ -2389,14 +2276,14 @@ k_step_compact(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
     const KParams& kp = a.kp;
     int slot = blockIdx.x * BLOCK + threadIdx.x;
     int idx = 0;
-    uint32_t lk = 0u;
-    if (slot < kp.nslots) {
-        idx = __ldg(cellidx + slot);
-        lk = __ldg(links + slot);
-    }
-    step_begin(slot);
-    uint32_t seed = 0u;
-    if constexpr (Store<S>::kStochastic) {
+    uint32_t lk = 0u, seed = 0u;
+    if constexpr (!Store<S>::kStochastic) {
+        if (slot < kp.nslots) {
+            idx = __ldg(cellidx + slot);
+            lk = __ldg(links + slot);
+        }
+        step_begin(slot);
+    } else {
         // this launch reads counter[parity] and leaves counter + 1 for the next
         seed = rng_ctr[parity];
         if (blockIdx.x == 0 && threadIdx.x == 0) rng_ctr[parity ^ 1] = seed + 1u;
@@ -2408,8 +2295,11 @@ k_step_compact(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
     }
     if (slot < kp.nslots) {
         uint32_t rnd = 0u;
-        if constexpr (Store<S>::kStochastic)
+        if constexpr (Store<S>::kStochastic) {
+            idx = __ldg(cellidx + slot);
+            lk = __ldg(links + slot);
             rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ (seed * 0x9e3779b9u));
+        }
         compact_cell<L, MODEL, S, CHECK>(kp, coef<R>(a), src, dst, lk, idx, slot, rank, tau, usnap,
                                          rnd, acc);
     }
@@ -2420,30 +2310,26 @@ k_step_compact(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
 // slot, slot + stride, ... and loads the next slot's cell index and link word
 // before it steps the current one, so of the three dependent loads of a slot
 // (cell index, neighbour slots, populations) only the last two are on the
-// critical path.  It pays for the 16-bit forms.  The FP32 forms need more
-// registers for it than their budgets hold (D3Q19 IR, 256^3 porous box: 323 us
-// by one-slot threads, 349-386 by the loop).
-// (class sums: the IR step, at every size)
+// critical path.  It pays for the IR step of the 16-bit forms (256^3 porous
+// box, D3Q19 FP16: 306 -> 268 us).  The FP32 forms need more registers for it
+// than their budgets hold (D3Q19 IR, 256^3 porous box: 323 us by one-slot
+// threads, 349-386 by the loop); 16-bit PR gained nothing.
 template <int MODEL, class S> constexpr bool compact_loop() {
-    return sizeof(S) == 2 && (pair_form<S>() || MODEL == LBM_MODEL_IR);
+    return MODEL == LBM_MODEL_IR && sizeof(S) == 2;
 }
-// ... and for domains of several rounds of the grid only (D3Q19 PR FP16, 48^3
-// box: 3.4 us by one-slot threads, 4.1 by the loop).
-constexpr int kLoopRounds = 4;
-// Register budget in resident blocks (BLBM_COMPACT_LOOP_MINB overrides it at
-// build time), FP16, us at 4 / 5 / 6 blocks: D3Q19 256^3 porous box IR 235 / 225 /
-// 279 and PR 277 / 261 / 313; D3Q15 160^3 box PR 66 / 59 / 64; D3Q27 160^3 box PR
-// 88 / 99 / 120 and IR 79 / 91 / 106.
+// (BLBM_COMPACT_LOOP_MINB overrides its register budget at build time.)
 #ifndef BLBM_COMPACT_LOOP_MINB
 #define BLBM_COMPACT_LOOP_MINB -1
 #endif
-template <class L, class S> constexpr int compact_loop_min_blocks() {
+// D3Q27: 4 blocks (64 registers; at 5 blocks it spills 68 bytes).
+template <class L, int MODEL, class S> constexpr int compact_loop_min_blocks() {
     if (BLBM_COMPACT_LOOP_MINB >= 0) return BLBM_COMPACT_LOOP_MINB;
-    return L::Q == 27 ? 4 : pair_form<S>() ? 5 : 6;
+    if (L::Q == 27) return 4;
+    return compact_min_blocks<L, MODEL, S, false>();
 }
 
 template <class L, int MODEL, class S>
-__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L, S>())
+__global__ void __launch_bounds__(kBlock, compact_loop_min_blocks<L, MODEL, S>())
 k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> dst,
                     const uint32_t* __restrict__ links, const int* __restrict__ cellidx,
                     const int* __restrict__ rank, typename Store<S>::R* __restrict__ tau,
@@ -2452,18 +2338,17 @@ k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> ds
     const KParams& kp = a.kp;
     const int n = kp.nslots, stride = gridDim.x * kBlock;
     int slot = blockIdx.x * kBlock + threadIdx.x;
-    int idx = 0;
-    uint32_t lk = 0u;
-    if (slot < n) {
-        idx = __ldg(cellidx + slot);
-        lk = __ldg(links + slot);
-    }
-    step_begin(slot);
     uint32_t seed = 0u;
     if constexpr (Store<S>::kStochastic) {
         // this launch reads counter[parity] and leaves counter + 1 for the next
         seed = rng_ctr[parity];
         if (blockIdx.x == 0 && threadIdx.x == 0) rng_ctr[parity ^ 1] = seed + 1u;
+    }
+    int idx = 0;
+    uint32_t lk = 0u;
+    if (slot < n) {
+        idx = __ldg(cellidx + slot);
+        lk = __ldg(links + slot);
     }
     R acc[kNumStats];
     for (; slot < n; slot += stride) {
@@ -2485,11 +2370,10 @@ k_step_compact_loop(const KArgs a, const SrcPlanes<S> src, const DstPlanes<S> ds
 }
 
 // link words of the compact layout: slot k gets the bits of cell cellidx[k]
-// (face_bits: and kFaceBit, for the 16-bit forms)
 template <class L>
 __global__ void __launch_bounds__(kBlock)
 k_links_compact(const KParams kp, const uint8_t* __restrict__ mask,
-                const int* __restrict__ cellidx, uint32_t* __restrict__ links, bool face_bits) {
+                const int* __restrict__ cellidx, uint32_t* __restrict__ links) {
     const int slot = blockIdx.x * kBlock + threadIdx.x;
     if (slot >= kp.nslots) return;
     const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
@@ -2503,9 +2387,6 @@ k_links_compact(const KParams kp, const uint8_t* __restrict__ mask,
         const int zs = (z - L::cz(i) + nz) % nz;
         if (mask[xs + nx * (ys + ny * zs)]) bits |= 1u << i;
     }
-    if (face_bits && (x == 0 || x == nx - 1 || y == 0 || y == ny - 1 ||
-                      (L::D == 3 && (z == 0 || z == nz - 1))))
-        bits |= kFaceBit;
     links[slot] = bits;
 }
 
@@ -2981,10 +2862,11 @@ template <class L, class S> inline DstPlanes<S> dst_planes(void* f, int64_t plan
 // most that divided steps fill (cells times parts).
 constexpr int64_t kSplitLanes = 608 * 32;
 
-// Launch of a step kernel that calls step_begin() (overlapped launches).
+// Launch of a step kernel; overlap: over the tail of the one before (it calls
+// step_begin()).
 template <class... K, class... A>
-inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, cudaStream_t st,
-                                     A&&... args) {
+inline cudaError_t launch_kernel(bool overlap, void (*kernel)(K...), int grid, int block,
+                                 cudaStream_t st, A&&... args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -2993,8 +2875,13 @@ inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, 
     cfg.blockDim = dim3((unsigned)block);
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <class... K, class... A>
+inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, cudaStream_t st,
+                                     A&&... args) {
+    return launch_kernel(true, kernel, grid, block, st, std::forward<A>(args)...);
 }
 
 // Threads per block and blocks of a resident run of ncells cells, and whether
@@ -3200,13 +3087,17 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
     const int grid = step_grid(kp.nslots);
     const SrcPlanes<S> src = src_planes<L, S>(s.fsrc, kp.plane);
     const DstPlanes<S> dst = dst_planes<L, S>(s.fdst, kp.plane);
-    if (check) {
-        return launch_overlapped(k_step_compact<L, MODEL, S, true>, grid, kBlock, st, a, src, dst,
-                                 s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials,
-                                 s.rng_ctr, s.parity);
-    }
+    // The 16-bit steps are not overlapped: with their loads in front of the wait the
+    // compiler orders the rest worse (D3Q27 FP16, 160^3 porous box: PR 109.3 -> 115.5 us;
+    // 100^3, IR 21.7 -> 23.4) and contracts the class sums of D3Q15 and D3Q19 IR
+    // differently; behind it an overlapped launch gains nothing.
+    constexpr bool overlap = !Store<S>::kStochastic;
+    if (check)
+        return launch_kernel(overlap, k_step_compact<L, MODEL, S, true>, grid, kBlock, st, a, src, dst,
+                             s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials,
+                             s.rng_ctr, s.parity);
     if constexpr (compact_loop<MODEL, S>()) {
-        // persistent: as many blocks as are resident at once
+        // persistent: as many blocks as are resident at once, at most one per 256 slots
         static const int resident = [] {   // blocks per SM (per instantiation)
             int r = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, k_step_compact_loop<L, MODEL, S>,
@@ -3219,19 +3110,17 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        int pgrid = std::max(1, resident * sms);
-        if (!pair_form<S>()) pgrid = std::min(grid, pgrid);
-        if (!pair_form<S>() || grid >= kLoopRounds * pgrid)
-            return launch_overlapped(k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
-                                     s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
+        const int pgrid = std::min(grid, std::max(1, resident * sms));
+        return launch_kernel(overlap, k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
+                             s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
     }
     auto one = [&](auto kernel, int b) {
-        return launch_overlapped(kernel, (kp.nslots + b - 1) / b, b, st, a, src, dst, s.links, s.cellidx,
-                                 s.rank, (R*)s.tau, (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
+        return launch_kernel(overlap, kernel, (kp.nslots + b - 1) / b, b, st, a, src, dst, s.links,
+                             s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
     };
     // few slots: finer blocks spread over the SMs (see untuned_block)
     if (kp.nslots <= 8 * 152 * kBlock) return one(k_step_compact<L, MODEL, S, false, 128>, 128);
-    constexpr int B = compact_block<L, MODEL, S>();
+    constexpr int B = compact_block<L, MODEL>();
     return one(k_step_compact<L, MODEL, S, false, B>, B);
 }
 
@@ -3261,12 +3150,8 @@ cudaError_t launch_step_lat(int model, int storage, bool check, const KParams& k
     switch (storage) {
     case LBM_F32: return launch_step_model<L, float>(model, check, kp, s, st);
     case LBM_F64: return launch_step_model<L, double>(model, check, kp, s, st);
-    case LBM_F16_OFS:
-        return kp.pair16 ? launch_step_model<L, PairHalf>(model, check, kp, s, st)
-                         : launch_step_model<L, __half>(model, check, kp, s, st);
-    case LBM_BF16_OFS:
-        return kp.pair16 ? launch_step_model<L, PairBf16>(model, check, kp, s, st)
-                         : launch_step_model<L, __nv_bfloat16>(model, check, kp, s, st);
+    case LBM_F16_OFS: return launch_step_model<L, __half>(model, check, kp, s, st);
+    case LBM_BF16_OFS: return launch_step_model<L, __nv_bfloat16>(model, check, kp, s, st);
     default: return cudaErrorNotSupported;
     }
 }
@@ -3323,9 +3208,9 @@ cudaError_t launch_batch_lat(int model, int storage, bool check, const BatchDesc
 
 template <class L>
 cudaError_t launch_links_lat(const KParams& kp, const uint8_t* mask, uint32_t* links,
-                             const int* cellidx, bool face_bits, cudaStream_t st) {
+                             const int* cellidx, cudaStream_t st) {
     if (cellidx)
-        k_links_compact<L><<<step_grid(kp.nslots), kBlock, 0, st>>>(kp, mask, cellidx, links, face_bits);
+        k_links_compact<L><<<step_grid(kp.nslots), kBlock, 0, st>>>(kp, mask, cellidx, links);
     else
         k_links<L><<<step_grid(kp.ncells), kBlock, 0, st>>>(kp, mask, links);
     return cudaGetLastError();
@@ -3455,8 +3340,8 @@ template <class L> void lattice_table(int* c, double* w) {
         return launch_step_lat<L>(model, storage, check, kp, a, st);                            \
     }                                                                                           \
     cudaError_t launch_links_##L(const KParams& kp, const uint8_t* mask, uint32_t* links,      \
-                                 const int* cellidx, bool face_bits, cudaStream_t st) {         \
-        return launch_links_lat<L>(kp, mask, links, cellidx, face_bits, st);                    \
+                                 const int* cellidx, cudaStream_t st) {                         \
+        return launch_links_lat<L>(kp, mask, links, cellidx, st);                               \
     }                                                                                           \
     cudaError_t launch_fields_##L(int storage, const KParams& kp, const void* f,               \
                                   const uint32_t* links, const int* rank, double* rho,         \

@@ -235,12 +235,11 @@ bool resident_fits(const lbm_solver* s) {
 }
 
 cudaError_t launch_links(lbm_solver* s, const uint8_t* mask) {
-    const bool face = s->kp.pair16 != 0;
     switch (s->lat) {
-    case LBM_D2Q9: return launch_links_D2Q9(s->kp, mask, s->links, s->cellidx, face, s->stream);
-    case LBM_D3Q15: return launch_links_D3Q15(s->kp, mask, s->links, s->cellidx, face, s->stream);
-    case LBM_D3Q19: return launch_links_D3Q19(s->kp, mask, s->links, s->cellidx, face, s->stream);
-    default: return launch_links_D3Q27(s->kp, mask, s->links, s->cellidx, face, s->stream);
+    case LBM_D2Q9: return launch_links_D2Q9(s->kp, mask, s->links, s->cellidx, s->stream);
+    case LBM_D3Q15: return launch_links_D3Q15(s->kp, mask, s->links, s->cellidx, s->stream);
+    case LBM_D3Q19: return launch_links_D3Q19(s->kp, mask, s->links, s->cellidx, s->stream);
+    default: return launch_links_D3Q27(s->kp, mask, s->links, s->cellidx, s->stream);
     }
 }
 
@@ -544,7 +543,6 @@ static lbm_status create_impl(lbm_solver** out, lbm_lattice lat, int nx, int ny,
     kp.ncells = s->ncells;
     kp.cell_begin = 0;
     kp.cell_end = s->ncells;
-    kp.pair16 = storage_bytes(p->storage) == 2 && (int64_t)nx * ny >= kPairPlane;
     kp.nslots = compact ? (int)s->nfluid : 0;
     kp.plane = s->lay.plane;
     kp.nu_p = p->mu_p;   // rho_0 = 1

@@ -13,11 +13,7 @@ namespace blbm {
 
 constexpr int kBlock = 256;          // threads per block of the cell kernels
 constexpr int kNumStats = 8;         // doubles per reduction partial
-// Cells of an x-y plane from which the 16-bit forms run the pair-form collision:
-// the plane, because a domain's z-slabs share it and step to the same bits.
-constexpr int64_t kPairPlane = 128 * 128;
 constexpr uint32_t kSolidBit = 1u << 31;
-constexpr uint32_t kFaceBit = 1u << 30;   // compact link words: the cell lies at a face of the box
 // Kernel-side model code: PR with the Newton-implicit tau update is its own
 // instantiation, so the explicit kernels carry none of its code.
 constexpr int kModelPRImplicit = 2;
@@ -37,7 +33,6 @@ struct KParams {
     int newton;           // PR: Newton iterations of the implicit tau update (0 = explicit)
     uint32_t hash_offset; // added to the cell index in the stochastic-rounding hash
     int cell_begin, cell_end; // cells the single-domain step kernel covers (0, ncells)
-    int pair16;           // 16-bit storage: steps run the pair-form collision (kPairPlane)
     int nslots;           // compact layout: fluid cells held (0: dense layout)
     FastDiv div_nx, div_ny;   // idx -> (x, y, z) without integer division
 };
@@ -77,7 +72,7 @@ struct BatchDesc;   // per-domain descriptor of a batched launch (kernels.cuh)
     cudaError_t launch_step_##L(int model, int storage, bool check, const KParams& kp,          \
                                 const StepArgs& a, cudaStream_t st);                            \
     cudaError_t launch_links_##L(const KParams& kp, const uint8_t* mask, uint32_t* links,       \
-                                 const int* cellidx, bool face_bits, cudaStream_t st);          \
+                                 const int* cellidx, cudaStream_t st);                          \
     cudaError_t launch_fields_##L(int storage, const KParams& kp, const void* f,                \
                                   const uint32_t* links, const int* rank, double* rho,          \
                                   double* ux, double* uy, double* uz, cudaStream_t st);         \
