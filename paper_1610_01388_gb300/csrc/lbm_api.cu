@@ -714,7 +714,9 @@ void apply_tuning(lbm_solver* s) {
     if (!sh.set) sh.block = untuned_block(s);
     // an entry of the table keeps its launch shape
     s->split = !sh.set;
-    s->resident = !sh.set && !s->rank && resident_fits(s);
+    // a run reads one buffer's ghost planes at every step, single steps each
+    // buffer's own (an exchange fills the current one's)
+    s->resident = !sh.set && !s->rank && !(s->p.flags & LBM_FLAG_Z_GHOSTS) && resident_fits(s);
     if (sh.block != s->block || sh.cpt != s->cpt) {
         for (int k = 0; k < 2; ++k)
             if (s->graph[k]) {
