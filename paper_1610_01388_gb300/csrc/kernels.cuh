@@ -214,12 +214,23 @@ __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, 
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// a > b for numbers >= 0, whose bits order as integers: an FP64 compare would
+// take its turn on the FP64 pipe like an add
+__device__ __forceinline__ bool above(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
+// x in [2^-960, 2^960), by its high word: neither x nor its reciprocal or root is
+// near what the starts below flush to zero
+__device__ __forceinline__ bool moderate(double x) {
+    return (uint32_t)__double2hiint(x) - 0x03f00000u < 0x78000000u;
+}
 // Reciprocal and (reciprocal) square root of the pair-form collision: the
 // hardware's approximation refined by the residual of its defining equation.
 // With e = 1 - x r, 1 / x = r (1 + e + e^2 + ...); with e = 1 - x r^2, 1 / sqrt(x)
 // = r (1 + e/2 + 3/8 e^2 + ...).  They start within 2^-19 and take two terms, 3
 // and 5 operations on the FP64 pipe where the division and the root take 9 to
-// 10.  Arguments are normal numbers (callers guard the rest).
+// 10.  x has to be moderate; callers divide and root other numbers, zeros,
+// infinities and NaN among them.
 __device__ __forceinline__ double rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -232,13 +243,7 @@ __device__ __forceinline__ double rcp_root(double x) {
     const double e = mad(-mul(x, r), r, 1.0);
     return mad(mul(r, e), mad(0.375, e, 0.5), r);
 }
-// a > b for numbers >= 0, whose bits order as integers: an FP64 compare would
-// take its turn on the FP64 pipe like an add
-__device__ __forceinline__ bool above(double a, double b) {
-    return __double_as_longlong(a) > __double_as_longlong(b);
-}
-// (below 1e-290 the root counts as 0: the flush to zero of its start)
-__device__ __forceinline__ double root(double x) { return above(x, 1e-290) ? mul(x, rcp_root(x)) : 0.0; }
+__device__ __forceinline__ double root(double x) { return moderate(x) ? mul(x, rcp_root(x)) : sqrt(x); }
 
 // ---------------------------------------------------------------------------
 // storage.  R is the arithmetic type.  ld / st move population i between
@@ -845,12 +850,17 @@ __device__ __forceinline__ void pair_terms(R e0, const Tens<R>& N, R qx, R qy, R
 __device__ __forceinline__ void ir_yield(const Coef<double>& c, double t2, double& k1, double& asg) {
     k1 = 0.0;
     asg = -1.0;
-    // (|T| below 1e-145 counts as not yielded: see rcp_root)
-    if (above(t2, 1e-290) && !above(c.s2y2, t2)) {
-        const double it = rcp_root(t2);
-        k1 = mad(c.ir_ks, it, c.ir_k);
-        asg = mad(-c.ir_bs, it, -c.ir_bn);
+    double it;
+    if (moderate(t2)) {
+        if (above(c.s2y2, t2)) return;
+        it = rcp_root(t2);
+    } else {
+        const double tn = sqrt(t2);
+        if (!(tn > 0.0 && tn >= c.s2y)) return;
+        it = 1.0 / tn;
     }
+    k1 = mad(c.ir_ks, it, c.ir_k);
+    asg = mad(-c.ir_bs, it, -c.ir_bn);
 }
 
 // ---------------------------------------------------------------------------
@@ -860,7 +870,7 @@ template <class L, class R>
 __device__ __forceinline__ void ir_terms(const Coef<typename Lanes<R>::Sc>& c, uint32_t flags,
                                          const Mom<R>& m, R& e0, Tens<R>& N, R (&q)[3], R (&ur)[3]) {
     const R rho = add(R(1), m.d);
-    const R inv = rcp(rho);
+    const R inv = moderate(rho) ? rcp(rho) : 1.0 / rho;
     const R gx = R(c.g[0]), gy = R(c.g[1]);
     R gz = R(0);
     if constexpr (L::D == 3) gz = R(c.g[2]);
@@ -982,9 +992,8 @@ __device__ __forceinline__ void pr_rates(const Coef<typename Lanes<R>::Sc>& c, R
     wm_out = Lanes<R>::make(wm_);
 }
 
-// The same for the pair form.  itau: 1 / (previous step's tau).  Both rates from
-// one reciprocal (a product of two moderate numbers; beyond that range, which
-// only an extreme m reaches, from two).
+// The same for the pair form.  itau: 1 / (previous step's tau).  Both rates come
+// from one reciprocal, of a moderate product (all but an extreme m or Lambda).
 template <bool IMPLICIT>
 __device__ __forceinline__ void pair_pr_rates(const Coef<double>& c, double tn2, double inv, double itau,
                                               double& tau, double& wp, double& wm) {
@@ -995,8 +1004,7 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<double>& c, double tn2,
     double nu;
     if (!above(c.gdot_c, gd)) {
         const double y = mul(sy_rho, -expm1(mul(-c.m, gd)));
-        if (above(gd, 1e-290)) nu = mad(y, rcp(gd), c.nu_p);
-        else nu = add(c.nu_p, y / gd);
+        nu = moderate(gd) ? mad(y, rcp(gd), c.nu_p) : add(c.nu_p, y / gd);
     } else {
         const double nu0 = mad(c.m, sy_rho, c.nu_p);
         const double nuc = mad(sy_rho, c.e_c, c.nu_p);
@@ -1007,13 +1015,14 @@ __device__ __forceinline__ void pair_pr_rates(const Coef<double>& c, double tn2,
     // 1 / tau_odd with tau_odd = 1/2 + Lambda / (tau - 1/2) is tm / odd
     const double tm = sub(tau, 0.5);
     const double odd = mad(0.5, tm, c.magic);
-    if (!above(tau, 1e30)) {
-        const double r = rcp(mul(tau, odd));
+    const double product = mul(tau, odd);
+    if (moderate(product)) {
+        const double r = rcp(product);
         wp = mul(r, odd);
         wm = mul(tm, mul(r, tau));
     } else {
-        wp = rcp(tau);
-        wm = mul(tm, rcp(odd));
+        wp = 1.0 / tau;
+        wm = tm / odd;
     }
 }
 
@@ -1027,8 +1036,16 @@ __device__ __forceinline__ void pr_terms(const Coef<typename Lanes<R>::Sc>& c, u
                                          const Mom<R>& m, R& tau, R& K0, Tens<R>& N, R (&q)[3], R& wp,
                                          R& wm, R (&ur)[3]) {
     const R rho = add(R(1), m.d);
-    const R both = rcp(mul(rho, tau));   // one reciprocal for both 1 / rho and 1 / tau_old
-    const R inv = mul(both, tau), itau = mul(both, rho);
+    R inv, itau;   // 1 / rho, 1 / tau_old, of a moderate product from one reciprocal
+    const R product = mul(rho, tau);
+    if (moderate(product)) {
+        const R both = rcp(product);
+        inv = mul(both, tau);
+        itau = mul(both, rho);
+    } else {
+        inv = 1.0 / rho;
+        itau = 1.0 / tau;
+    }
     const R ux = mul(m.jx, inv), uy = mul(m.jy, inv);
     R uz = R(0);
     if constexpr (L::D == 3) uz = mul(m.jz, inv);
