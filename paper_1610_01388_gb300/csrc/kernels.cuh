@@ -227,9 +227,11 @@ __device__ __forceinline__ bool moderate(double x) {
 // Reciprocal and (reciprocal) square root of the pair-form collision: the
 // hardware's approximation refined by the residual of its defining equation.
 // With e = 1 - x r, 1 / x = r (1 + e + e^2 + ...); with e = 1 - x r^2, 1 / sqrt(x)
-// = r (1 + e/2 + 3/8 e^2 + ...).  They start within 2^-19 and take two terms, 3
-// and 5 operations on the FP64 pipe where the division and the root take 9 to
-// 10.  x has to be moderate; callers divide and root other numbers, zeros,
+// = r (1 + e/2 + 3/8 e^2 + ...) (binomial series).  The starts read and give 20
+// mantissa bits, so e stays near 2^-19 and two terms do, 3 and 5 operations on the
+// FP64 pipe where the division and the root take 9 to 10.  Largest errors measured:
+// 0.50 ulp of 1 / x, 0.92 of 1 / sqrt(x) (the root and the division: up to 1), 1.61
+// of the root.  x has to be moderate; callers divide and root other numbers, zeros,
 // infinities and NaN among them.
 __device__ __forceinline__ double rcp(double x) {
     double r;
