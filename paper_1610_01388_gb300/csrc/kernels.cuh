@@ -2903,6 +2903,38 @@ inline cudaError_t launch_overlapped(void (*kernel)(K...), int grid, int block, 
     return launch_kernel(true, kernel, grid, block, st, std::forward<A>(args)...);
 }
 
+// Launch of a solver's step kernel, overlapped where that pays.  The blocks of a
+// launch over the tail of another share the SMs with it, so two grids that fit
+// together overlap whole, and of a grid of a wave and more some blocks start early.
+// In between, a grid that fits alone only would start in part, and in a second
+// wave.  Steps of 0.05-2 waves on D2Q9 to D3Q27, FP32 and FP16, plain over overlapped
+// us: 1.03-1.31 up to half a wave, 0.72-0.95 from there to 0.8, 1.04 from 0.9 on
+// (D3Q15 FP32 PR, 48^3: 3.7 plain, 4.7 overlapped; 40^3: 3.2 and 2.8).  FP64 steps in
+// blocks of 256, bound by the FP64 pipe of the SMs that hold two of the blocks, are
+// launched plainly: the blocks that start early take the SMs the other grid leaves
+// idle first, several to an SM (a step of 256^2 cells in two parts: 39.1 -> 32.8 us).
+template <auto Kernel, class R, class... A>
+inline cudaError_t launch_step(int grid, int block, cudaStream_t st, A&&... args) {
+    struct Wave {
+        int sms = 1, per_sm = 0;   // (unknown: overlapped)
+    };
+    static const Wave wave = [block] {   // per instantiation, which has one block size
+        Wave w;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&w.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&w.per_sm, Kernel, block, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return Wave();
+        }
+        return w;
+    }();
+    const bool both = 2 * ((grid + wave.sms - 1) / wave.sms) <= wave.per_sm;
+    const bool waves = 10 * (int64_t)grid >= 9 * (int64_t)wave.per_sm * wave.sms;
+    const bool piled = sizeof(R) == 8 && block >= kBlock;
+    return launch_kernel((both || waves) && !piled, Kernel, grid, block, st, std::forward<A>(args)...);
+}
+
 // Threads per block and blocks of a resident run of ncells cells, and whether
 // the domain takes it (fits one cluster): small domains of FP32 arithmetic
 // share one block, larger ones spread over the cluster's 16 (D2Q9 F32 IR, us a
@@ -3068,53 +3100,66 @@ cudaError_t launch_step_c(bool check, const KParams& kp, const StepArgs& s, cuda
     if constexpr (MODEL != kModelPRImplicit && std::is_same<typename Store<S>::R, float>::value) {
         if (!check && s.cpt == 2) {   // two cells per thread
             if (block == 128)
-                return launch_overlapped(k_step2<L, MODEL, S, 128>, (kp.ncells + 255) / 256, 128, st,
-                                         a, src, dst, s.links, (R*)s.tau, s.rng_ctr, s.parity);
-            return launch_overlapped(k_step2<L, MODEL, S, 256>, (kp.ncells + 511) / 512, 256, st, a,
-                                     src, dst, s.links, (R*)s.tau, s.rng_ctr, s.parity);
+                return launch_step<k_step2<L, MODEL, S, 128>, R>((kp.ncells + 255) / 256, 128, st, a, src,
+                                                              dst, s.links, (R*)s.tau, s.rng_ctr, s.parity);
+            return launch_step<k_step2<L, MODEL, S, 256>, R>((kp.ncells + 511) / 512, 256, st, a, src, dst,
+                                                          s.links, (R*)s.tau, s.rng_ctr, s.parity);
         }
     }
-    auto go = [&](auto kernel, int b) {
-        return launch_overlapped(kernel, (ncell + b - 1) / b, b, st, a, src, dst, s.links, (R*)s.tau,
-                                 (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
+    // (the block size and whether it is a check step, whole or in part)
+    auto go = [&](auto B, auto CHECK, auto PART) {
+        constexpr int b = decltype(B)::value;
+        return launch_step<k_step<L, MODEL, S, decltype(CHECK)::value, b, COPY, decltype(PART)::value>, R>(
+            (ncell + b - 1) / b, b, st, a, src, dst, s.links, (R*)s.tau, (R*)s.usnap, s.partials,
+            s.rng_ctr, s.parity);
     };
-    if (check) return go(k_step<L, MODEL, S, true, kBlock, COPY>, kBlock);
+    constexpr std::true_type yes;
+    constexpr std::false_type no;
+#define BLBM_B(n) std::integral_constant<int, n>{}
+    if (check) return go(BLBM_B(kBlock), yes, no);
     // FP64 domains that leave sub-partitions idle
     if constexpr (f64 && MODEL != kModelPRImplicit) {
         if (s.split && kp.cell_begin == 0 && kp.cell_end == kp.ncells &&
             (int64_t)kp.ncells * parts<L>() <= kSplitLanes)
-            return launch_overlapped(k_step_split<L, MODEL>, (kp.ncells + 31) / 32, 32 * parts<L>(), st,
-                                     a, src, dst, s.links, (R*)s.tau);
+            return launch_step<k_step_split<L, MODEL>, R>((kp.ncells + 31) / 32, 32 * parts<L>(), st, a, src,
+                                                       dst, s.links, (R*)s.tau);
     }
     // one part of a step taken in parts (256 threads)
     if (kp.cell_begin != 0 || kp.cell_end != kp.ncells)
-        return go(k_step<L, MODEL, S, false, kBlock, COPY, true>, kBlock);
+        return go(BLBM_B(kBlock), no, yes);
     if constexpr (MODEL != kModelPRImplicit || f64) {
-        if (block == 64) return go(k_step<L, MODEL, S, false, 64, COPY>, 64);
+        if (block == 64) return go(BLBM_B(64), no, no);
     }
     if constexpr (MODEL != kModelPRImplicit) {
-        if (block == 128) return go(k_step<L, MODEL, S, false, 128, COPY>, 128);
-        if (block == 512) return go(k_step<L, MODEL, S, false, 512, COPY>, 512);
+        if (block == 128) return go(BLBM_B(128), no, no);
+        if (block == 512) return go(BLBM_B(512), no, no);
     }
-    return go(k_step<L, MODEL, S, false, kBlock, COPY>, kBlock);
+    return go(BLBM_B(kBlock), no, no);
+#undef BLBM_B
 }
 
 template <class L, int MODEL, class S>
 cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s, cudaStream_t st) {
     using R = typename Store<S>::R;
     const KArgs a = make_args<L>(kp);
-    const int grid = step_grid(kp.nslots);
     const SrcPlanes<S> src = src_planes<L, S>(s.fsrc, kp.plane);
     const DstPlanes<S> dst = dst_planes<L, S>(s.fdst, kp.plane);
     // The 16-bit steps are not overlapped: with their loads in front of the wait the
     // compiler orders the rest worse (D3Q27 FP16, 160^3 porous box: PR 109.3 -> 115.5 us;
     // 100^3, IR 21.7 -> 23.4) and contracts the class sums of D3Q15 and D3Q19 IR
     // differently; behind it an overlapped launch gains nothing.
-    constexpr bool overlap = !Store<S>::kStochastic;
-    if (check)
-        return launch_kernel(overlap, k_step_compact<L, MODEL, S, true>, grid, kBlock, st, a, src, dst,
-                             s.links, s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials,
-                             s.rng_ctr, s.parity);
+    auto one = [&](auto B, auto CHECK) {
+        constexpr int b = decltype(B)::value;
+        constexpr auto kernel = k_step_compact<L, MODEL, S, decltype(CHECK)::value, b>;
+        const int blocks = (kp.nslots + b - 1) / b;
+        if constexpr (Store<S>::kStochastic)
+            return launch_kernel(false, kernel, blocks, b, st, a, src, dst, s.links, s.cellidx, s.rank,
+                                 (R*)s.tau, (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
+        else
+            return launch_step<kernel, R>(blocks, b, st, a, src, dst, s.links, s.cellidx, s.rank, (R*)s.tau,
+                                       (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
+    };
+    if (check) return one(std::integral_constant<int, kBlock>{}, std::true_type{});
     if constexpr (compact_loop<MODEL, S>()) {
         // persistent: as many blocks as are resident at once, at most one per 256 slots
         static const int resident = [] {   // blocks per SM (per instantiation)
@@ -3129,18 +3174,13 @@ cudaError_t launch_step_compact(bool check, const KParams& kp, const StepArgs& s
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int pgrid = std::min(grid, std::max(1, resident * sms));
-        return launch_kernel(overlap, k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
+        const int pgrid = std::min(step_grid(kp.nslots), std::max(1, resident * sms));
+        return launch_kernel(false, k_step_compact_loop<L, MODEL, S>, pgrid, kBlock, st, a, src, dst,
                              s.links, s.cellidx, s.rank, (R*)s.tau, s.rng_ctr, s.parity);
     }
-    auto one = [&](auto kernel, int b) {
-        return launch_kernel(overlap, kernel, (kp.nslots + b - 1) / b, b, st, a, src, dst, s.links,
-                             s.cellidx, s.rank, (R*)s.tau, (R*)s.usnap, s.partials, s.rng_ctr, s.parity);
-    };
     // few slots: finer blocks spread over the SMs (see untuned_block)
-    if (kp.nslots <= 8 * 152 * kBlock) return one(k_step_compact<L, MODEL, S, false, 128>, 128);
-    constexpr int B = compact_block<L, MODEL>();
-    return one(k_step_compact<L, MODEL, S, false, B>, B);
+    if (kp.nslots <= 8 * 152 * kBlock) return one(std::integral_constant<int, 128>{}, std::false_type{});
+    return one(std::integral_constant<int, compact_block<L, MODEL>()>{}, std::false_type{});
 }
 
 // The compact layout has its own kernel.  In the dense one the copy-through

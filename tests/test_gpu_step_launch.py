@@ -48,3 +48,27 @@ def test_queued_steps_equal_waited_steps(lat, model, storage, layout, make, chec
         assert a.residual() == b.residual()
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("check_every", [0, 7])
+@pytest.mark.parametrize("lat,model,storage,shape", [
+    # steps that fill more than half the GPU and less than all of it, in both
+    # layouts, and the sizes around: overlapped, plain, overlapped launches
+    ("D3Q15", "PR", "F32", (40, 40, 40)), ("D3Q15", "PR", "F32", (48, 48, 48)),
+    ("D3Q15", "PR", "F32", (64, 64, 64)), ("D3Q27", "IR", "F16", (48, 48, 48)),
+    ("D3Q27", "IR", "F16", (64, 64, 64)), ("D2Q9", "IR", "F32", (1, 400, 512)),
+    ("D3Q19", "PR", "F64", (20, 33, 33))])
+@pytest.mark.parametrize("layout", ["dense", "compact"])
+def test_overlapped_and_plain_launches_leave_the_same_bits(lat, model, storage, shape, layout, check_every):
+    rng = np.random.default_rng(6)
+    mask = (rng.random(shape) < 0.2).astype(np.uint8)
+    a, b = (_solver(lat, mask, model, storage, layout, check_every) for _ in range(2))
+    a.step(40)
+    for _ in range(40):
+        b.step(1)
+        b.sync()
+    np.testing.assert_array_equal(a.get_populations(), b.get_populations())
+    if check_every:
+        assert a.residual() == b.residual()
+    a.close()
+    b.close()
