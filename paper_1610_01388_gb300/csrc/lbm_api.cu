@@ -692,16 +692,21 @@ Shape tune_lookup(int lat, int model, int storage, int64_t cells) {
 //    64 cycles, so warps must be spread over sub-partitions, 64-thread blocks
 //    the finest that fills them: D2Q9 IR 4 x 64: 3.9 / 4.3 / 7.5; D3Q27 IR 1 x
 //    64 x 64: 8.9 / 10.2 / 18.6; D3Q19 PR 40 x 64 x 64: 75.1 / 78.3 / 86.8.
+//  - FP32 arithmetic on D2Q9: 128, where 64-thread blocks are launched slower than
+//    they run (IR F32 512^2: 4.75 / 3.94 / 3.90; PR F32 1024^2: 17.2 / 13.1 / 13.6; IR
+//    F32 128^2: 1.64 / 1.58 / 1.67).
 //  - FP32 arithmetic up to 8 blocks of 256 per SM (152 SMs): smaller blocks
 //    spread the last wave: D3Q15 PR F32 91k cells 2.85 / 2.89 / 3.07, D3Q27 IR F32
 //    80k 3.66 / 3.80 / 4.01, D3Q27 PR F32 262k 8.02 / 8.15 / 8.49.
-//  - larger 16-bit domains, bound by issue: 128 (D3Q27 PR F16 duct 256 x 128 x
-//    128: 113 / 102 / 109, porous 160^3: 117 / 116 / 123; D3Q19 IR F16: 68 / 65 / 67).
+//  - larger 16-bit domains, bound by issue: 128 (128 / 256: D3Q27 PR F16 duct 256 x
+//    128 x 128 110.6 / 119.0, porous 160^3 128 / 132; D3Q19 IR F16 duct 67.8 / 70.3).
 //  - larger FP32 domains, bound by HBM: 256 (D3Q27 IR, porous 160^3: 157 / 156 /
 //    134), where a wider block's reads meet in L1, but for the PR step of
 //    domains whose walls fill whole warps: 64 (duct: 138.7 / 139.8 / 141.2).
 int untuned_block(const lbm_solver* s) {
-    if (s->p.storage == LBM_F64 || s->ncells <= 8 * 152 * kBlock) return 64;
+    if (s->p.storage == LBM_F64) return 64;
+    if (s->lat == LBM_D2Q9) return 128;
+    if (s->ncells <= 8 * 152 * kBlock) return 64;
     if (storage_bytes(s->p.storage) == 2) return 128;
     return s->p.model == LBM_MODEL_PR && !s->copy ? 64 : kBlock;
 }
