@@ -2439,7 +2439,7 @@ template <> __device__ __forceinline__ const Coef<double>& bcoef<double>(const B
 // k_step's check step, with the copy-through for every form (the solid cells
 // of a group with fluid cells copy their populations through).
 template <class L, int MODEL, class S>
-__device__ __forceinline__ void batch_tile_check(const BatchDesc& D, int tile, int phase, uint32_t lk,
+__device__ __forceinline__ void batch_tile_check(const BatchDesc& D, int tile, int phase,
                                                  double* __restrict__ partials) {
     using R = typename Store<S>::R;
     const KParams& kp = D.kp;
@@ -2456,6 +2456,7 @@ __device__ __forceinline__ void batch_tile_check(const BatchDesc& D, int tile, i
         if (lb == 0 && threadIdx.x == 0) D.rng[cur ^ 1] = seed + 1u;
         rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ (seed * 0x9e3779b9u));
     }
+    const uint32_t lk = inside ? __ldg(D.links + idx) : kSolidBit;
     const bool active = !(lk & kSolidBit);
     const bool group_fluid = group_has_fluid(active, idx);
     R acc[kNumStats];
@@ -2471,9 +2472,8 @@ __device__ __forceinline__ void batch_tile_check(const BatchDesc& D, int tile, i
 // batch schedule sets per group): thread t steps cells base + t, base + t + T,
 // ... (C of them, one after the other), so every warp access stays
 // contiguous.  Per cell as k_step, with the copy-through for every form.
-// lk: the link word of the thread's first cell.
 template <class L, int MODEL, class S, int T, int C>
-__device__ __forceinline__ void batch_tile_plain(const BatchDesc& D, int tile, int phase, uint32_t lk) {
+__device__ __forceinline__ void batch_tile_plain(const BatchDesc& D, int tile, int phase) {
     using R = typename Store<S>::R;
     const KParams& kp = D.kp;
     const int lb = tile - D.pblock_begin;
@@ -2492,7 +2492,7 @@ __device__ __forceinline__ void batch_tile_plain(const BatchDesc& D, int tile, i
         const bool inside = idx < kp.ncells;
         uint32_t rnd = 0u;
         if constexpr (Store<S>::kStochastic) rnd = pcg_hash(((uint32_t)idx + kp.hash_offset) ^ (seed * 0x9e3779b9u));
-        if (c > 0) lk = inside ? __ldg(D.links + idx) : kSolidBit;
+        const uint32_t lk = inside ? __ldg(D.links + idx) : kSolidBit;
         const bool active = !(lk & kSolidBit);
         const bool group_fluid = group_has_fluid(active, idx);
         R acc[kNumStats];
@@ -2533,31 +2533,18 @@ template <int MODEL, class S, bool CHECK> constexpr int batch_min_blocks() {
          : sizeof(S) == 4 ? BLBM_BATCH_PR32_MINB : 0;
 }
 
-// The link word of a domain's cell idx (cells past the end count as solid).
-__device__ __forceinline__ uint32_t batch_link(const BatchDesc& D, int idx) {
-    return idx < D.kp.ncells ? __ldg(D.links + idx) : kSolidBit;
-}
-
-// Both batch kernels follow three dependent reads (tile map, descriptor, link
-// word) before a tile's populations; for a block's first tile these come
-// before step_begin(), under the tail of the step before.
+// Both batch kernels read nothing in front of step_begin(): a tile's map entry,
+// descriptor and first link word read there cost the rest of the tile more than
+// the wait hides (16 D2Q9 domains of 256^2 cells, PR: FP16 18.7 -> 21.6 us, FP32 18.7 ->
+// 20.5; D3Q27 FP32 IR 16^3: 4.5 -> 5.1).
 template <class L, int MODEL, class S>
 __global__ void __launch_bounds__(kBlock)
 k_step_batch_check(const BatchDesc* __restrict__ descs, const int* __restrict__ block_dom,
                    int ntiles, int phase, double* __restrict__ partials) {
-    int t = blockIdx.x;
-    uint32_t lk = kSolidBit;
-    if (t < ntiles) {
-        const BatchDesc& D = descs[block_dom[t]];
-        lk = batch_link(D, (t - D.block_begin) * kBlock + (int)threadIdx.x);
-    }
-    step_begin(t);
-    while (t < ntiles) {
-        batch_tile_check<L, MODEL, S>(descs[block_dom[t]], t, phase, lk, partials);
-        t += gridDim.x;
-        if (t >= ntiles) break;
-        const BatchDesc& D = descs[block_dom[t]];
-        lk = batch_link(D, (t - D.block_begin) * kBlock + (int)threadIdx.x);
+    int first = blockIdx.x;
+    step_begin(first);
+    for (int t = first; t < ntiles; t += gridDim.x) {
+        batch_tile_check<L, MODEL, S>(descs[block_dom[t]], t, phase, partials);
         __syncthreads();   // block_sum_store's shared rows are reused
     }
 }
@@ -2566,20 +2553,10 @@ template <class L, int MODEL, class S, int T, int C>
 __global__ void __launch_bounds__(T, batch_min_blocks<MODEL, S, false>() * kBlock / T)
 k_step_batch(const BatchDesc* __restrict__ descs, const int* __restrict__ tile_dom, int ntiles,
              int phase) {
-    int t = blockIdx.x;
-    uint32_t lk = kSolidBit;
-    if (t < ntiles) {
-        const BatchDesc& D = descs[tile_dom[t]];
-        lk = batch_link(D, (t - D.pblock_begin) * (C * T) + (int)threadIdx.x);
-    }
-    step_begin(t);
-    while (t < ntiles) {
-        batch_tile_plain<L, MODEL, S, T, C>(descs[tile_dom[t]], t, phase, lk);
-        t += gridDim.x;
-        if (t >= ntiles) break;
-        const BatchDesc& D = descs[tile_dom[t]];
-        lk = batch_link(D, (t - D.pblock_begin) * (C * T) + (int)threadIdx.x);
-    }
+    int first = blockIdx.x;
+    step_begin(first);
+    for (int t = first; t < ntiles; t += gridDim.x)
+        batch_tile_plain<L, MODEL, S, T, C>(descs[tile_dom[t]], t, phase);
 }
 
 // density and velocity u = (j + F/2) / rho of gathered populations
@@ -3225,19 +3202,23 @@ template <class L, int MODEL, class S>
 cudaError_t launch_batch_t(bool check, const BatchDesc* descs, const int* block_dom, int nblocks,
                            int grid, int phase, double* partials, int threads, int cpt,
                            cudaStream_t st) {
+    using R = typename Store<S>::R;
     if (check)
-        return launch_overlapped(k_step_batch_check<L, MODEL, S>, grid, kBlock, st, descs, block_dom,
-                                 nblocks, phase, partials);
-    auto go = [&](auto kernel) {
-        return launch_overlapped(kernel, grid, threads, st, descs, block_dom, nblocks, phase);
+        return launch_step<k_step_batch_check<L, MODEL, S>, R>(grid, kBlock, st, descs, block_dom, nblocks,
+                                                               phase, partials);
+    auto go = [&](auto T, auto C) {
+        return launch_step<k_step_batch<L, MODEL, S, decltype(T)::value, decltype(C)::value>, R>(
+            grid, threads, st, descs, block_dom, nblocks, phase);
     };
-    if (threads == 256 && cpt == 1) return go(k_step_batch<L, MODEL, S, 256, 1>);
+#define BLBM_I(n) std::integral_constant<int, n>{}
+    if (threads == 256 && cpt == 1) return go(BLBM_I(256), BLBM_I(1));
     if constexpr (batch_shapes_all<MODEL, S>()) {
-        if (threads == 128 && cpt == 1) return go(k_step_batch<L, MODEL, S, 128, 1>);
-        if (threads == 512 && cpt == 1) return go(k_step_batch<L, MODEL, S, 512, 1>);
-        if (threads == 128 && cpt == 2) return go(k_step_batch<L, MODEL, S, 128, 2>);
-        if (threads == 256 && cpt == 2) return go(k_step_batch<L, MODEL, S, 256, 2>);
+        if (threads == 128 && cpt == 1) return go(BLBM_I(128), BLBM_I(1));
+        if (threads == 512 && cpt == 1) return go(BLBM_I(512), BLBM_I(1));
+        if (threads == 128 && cpt == 2) return go(BLBM_I(128), BLBM_I(2));
+        if (threads == 256 && cpt == 2) return go(BLBM_I(256), BLBM_I(2));
     }
+#undef BLBM_I
     return cudaErrorInvalidValue;
 }
 
