@@ -591,7 +591,8 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     // launched into a capture)
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &capturing) != cudaSuccess) cudaGetLastError();
-    const bool branches = b->concurrent && active > 1 && capturing == cudaStreamCaptureStatusNone;
+    const bool graphs = capturing == cudaStreamCaptureStatusNone;
+    const bool branches = graphs && b->concurrent && active > 1;
     // one launch of the graph with this content, at the current phase
     auto replay = [&](int content) {
         cudaGraphExec_t& g = b->graph[content][b->phase];
@@ -603,7 +604,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     while (left > 0) {
         const int64_t to_check = b->k - (b->gstep % b->k);
         int64_t plain = std::min(to_check - 1, left);
-        while (plain >= kGraphLen) {
+        while (graphs && plain >= kGraphLen) {
             if ((v = replay(kGraphLen)) != LBM_OK) return v;
             b->gstep += kGraphLen;          // even: the phase is unchanged
             plain -= kGraphLen;

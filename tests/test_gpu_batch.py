@@ -339,3 +339,32 @@ def test_server_steady_criteria():
             changes.append(st.flow_change if crit == "flow" else st.residual)
         b.close()
         assert 0.0 <= changes[-1] < tol and not (0.0 <= changes[-2] < tol), (crit, changes[-3:])
+
+
+@pytest.mark.parametrize("forms", [1, 4])
+def test_captured_batch_steps_replay_as_uncaptured_ones(forms):
+    """A caller that captures the batch's stream gets plain launches, also for
+    runs long enough for the batch's own graphs."""
+    import torch
+    st = torch.cuda.Stream()
+    got = []
+    for capture in (True, False):
+        b = lbm.Batch(GB, check_every=50, stream=st.cuda_stream)
+        ids = [b.add(lat, mask, **prm) for lat, mask, prm in _cases()[2:2 + forms]]
+        b.step(10)
+        if capture:
+            st.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st, capture_error_mode="thread_local"):
+                b.step(40)                      # 39 plain steps and a check step
+            with torch.cuda.stream(st):
+                g.replay()
+            st.synchronize()
+        else:
+            b.step(40)
+        got.append([(lbm.lbm_get_populations(b.solver(d)), list(b.status(d).flow), b.status(d).steps)
+                    for d in ids])
+        b.close()
+    for (fa, qa, na), (fb, qb, nb) in zip(*got):
+        np.testing.assert_array_equal(fa, fb)
+        assert qa == qb and na == nb == 50
