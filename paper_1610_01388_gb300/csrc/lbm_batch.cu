@@ -96,11 +96,13 @@ struct Group {
     int user_model = 0;                    // lbm_model, the schedule key
     std::vector<int64_t> ids;
     int nblocks = 0;                       // check steps: tiles of kBlock cells
-    int grid = 0;                          // check steps: CTAs per launch
+    int grid = 0;                          // check steps: CTAs per launch beside other groups
+    int grid_alone = 0;                    // ... and one group after the other
     int tile_threads = kBlock;             // plain steps: tile shape of the schedule
     int tile_cpt = 1;
     int pnblocks = 0;                      // plain steps: tiles of tile_threads x tile_cpt cells
-    int pgrid = 0;                         // plain steps: CTAs per launch
+    int pgrid = 0;                         // plain steps, as the two above
+    int pgrid_alone = 0;
     BatchDesc* d_desc = nullptr;
     int* d_block_dom = nullptr;
     int* d_pblock_dom = nullptr;
@@ -211,6 +213,7 @@ struct lbm_batch {
     double* h_slots = nullptr;      // pinned mirror
     bool dirty = true;
     cudaGraphExec_t graph[kGraphLen + 1][2] = {};   // by content and phase
+    bool stepped = false;                 // since the groups changed
     int rows = 0;                         // stats rows in use: [0, rows)
     bool poisoned = false;
     int sms = 1;                          // multiprocessors of the device
@@ -259,6 +262,7 @@ void drop_graphs(lbm_batch* b) {
                 cudaGraphExecDestroy(g);
                 g = nullptr;
             }
+    b->stepped = false;
 }
 
 // (Re)build the per-group device tables after the set of domains or the
@@ -358,6 +362,9 @@ lbm_status rebuild(lbm_batch* b) {
         const int ctas = sched_ctas(g.lat, g.user_model, g.storage, part);
         g.grid = ctas > 0 ? std::min(blocks, ctas * b->sms) : blocks;
         g.pgrid = ctas > 0 ? std::min(pblocks, ctas * b->sms) : pblocks;
+        const int alone = sched_ctas(g.lat, g.user_model, g.storage);
+        g.grid_alone = alone > 0 ? g.grid : blocks;
+        g.pgrid_alone = alone > 0 ? g.pgrid : pblocks;
         if ((int)desc.size() > g.cap_desc) {
             if (g.d_desc) cudaFreeAsync(g.d_desc, b->stream);
             g.cap_desc = (int)desc.size() * 2;
@@ -385,12 +392,14 @@ lbm_status rebuild(lbm_batch* b) {
     return LBM_OK;
 }
 
-cudaError_t launch_group(lbm_batch* b, const Group& g, bool check, int phase, cudaStream_t st) {
+cudaError_t launch_group(lbm_batch* b, const Group& g, bool check, int phase, bool alone,
+                         cudaStream_t st) {
     cudaError_t e = check ? launch_batch(g.lat, g.model, g.storage, true, g.d_desc, g.d_block_dom,
-                                         g.nblocks, g.grid, phase, g.d_partials, kBlock, 1, st)
+                                         g.nblocks, alone ? g.grid_alone : g.grid, phase, g.d_partials,
+                                         kBlock, 1, st)
                           : launch_batch(g.lat, g.model, g.storage, false, g.d_desc,
-                                         g.d_pblock_dom, g.pnblocks, g.pgrid, phase, nullptr,
-                                         g.tile_threads, g.tile_cpt, st);
+                                         g.d_pblock_dom, g.pnblocks, alone ? g.pgrid_alone : g.pgrid,
+                                         phase, nullptr, g.tile_threads, g.tile_cpt, st);
     if (e != cudaSuccess || !check) return e;
     return launch_overlapped(k_finalize_domains, (int)g.ids.size(), kBlock, st, g.d_desc, g.d_partials,
                              b->d_slots);
@@ -399,7 +408,7 @@ cudaError_t launch_group(lbm_batch* b, const Group& g, bool check, int phase, cu
 cudaError_t launch_all(lbm_batch* b, bool check, cudaStream_t st) {
     for (auto& g : b->groups) {
         if (g.ids.empty()) continue;
-        cudaError_t e = launch_group(b, g, check, b->phase, st);
+        cudaError_t e = launch_group(b, g, check, b->phase, true, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -430,7 +439,7 @@ cudaError_t capture_branches(lbm_batch* b, int content, int par, int active) {
         cudaError_t eb = cudaStreamWaitEvent(st, b->fork, 0);
         const int steps = content == kGraphCheck ? 1 : content;
         for (int t = 0; t < steps && eb == cudaSuccess; ++t)
-            eb = launch_group(b, g, content == kGraphCheck, par ^ (t & 1), st);
+            eb = launch_group(b, g, content == kGraphCheck, par ^ (t & 1), false, st);
         cudaError_t ej = cudaEventRecord(b->join[k], st);
         if (ej == cudaSuccess) ej = cudaStreamWaitEvent(b->cap, b->join[k], 0);
         if (e == cudaSuccess) e = eb != cudaSuccess ? eb : ej;
@@ -592,7 +601,12 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &capturing) != cudaSuccess) cudaGetLastError();
     const bool graphs = capturing == cudaStreamCaptureStatusNone;
-    const bool branches = graphs && b->concurrent && active > 1;
+    // A call of one step after a change of the domains goes group by group: its
+    // graph may run once and is not worth the capture (48 domains in 10 groups:
+    // 218 us by launches, 267 by a graph; a call of three steps: as long).
+    const bool lone = nsteps == 1 && !b->stepped;
+    b->stepped = true;
+    const bool branches = graphs && b->concurrent && active > 1 && !lone;
     // one launch of the graph with this content, at the current phase
     auto replay = [&](int content) {
         cudaGraphExec_t& g = b->graph[content][b->phase];

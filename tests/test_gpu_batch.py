@@ -368,3 +368,33 @@ def test_captured_batch_steps_replay_as_uncaptured_ones(forms):
     for (fa, qa, na), (fb, qb, nb) in zip(*got):
         np.testing.assert_array_equal(fa, fb)
         assert qa == qb and na == nb == 50
+
+
+@pytest.mark.parametrize("concurrent", [True, False])
+def test_short_calls_between_changes_of_the_domains(concurrent):
+    """Calls of every length around the direct launches and the graphs, with
+    domains that come and go between them, leave what single steps leave."""
+    lengths = [1, 1, 3, 4, 4, 5, 5, 15, 16, 17, 35]
+    got = []
+    lbm.lbm_tuning_set_batch_concurrency(concurrent)
+    try:
+        for single in (False, True):
+            b = lbm.Batch(4 * GB, check_every=7)
+            ids = [b.add(lat, mask, **prm) for lat, mask, prm in _cases()[2:6]]
+            extra = None
+            for k, n in enumerate(lengths * 2):
+                if k % 5 == 4:
+                    if extra is not None:
+                        b.remove(extra)
+                    lat, mask, prm = _cases()[k % 2]
+                    extra = b.add(lat, mask, **prm)
+                for m in [1] * n if single else [n]:
+                    b.step(m)
+            got.append([(lbm.lbm_get_populations(b.solver(d)), b.status(d)) for d in ids])
+            b.close()
+    finally:
+        lbm.lbm_tuning_clear()
+    for (fa, sa), (fb, sb) in zip(*got):
+        np.testing.assert_array_equal(fa, fb)
+        assert (sa.steps, sa.checks, sa.residual) == (sb.steps, sb.checks, sb.residual)
+        assert list(sa.flow) == list(sb.flow)
