@@ -288,8 +288,8 @@ def run_ours(args):
         for model in ("IR", "PR"):
             best, times = autotune.tune(LATTICE, model, STORAGE, mask.size, steps=200, mask=mask)
             tuned[model] = {"block": best[0], "cells_per_thread": best[1],
-                            "us_per_step": {f"{b}x{c}": round(t * 1e6, 2)
-                                            for (b, c), t in times.items()}}
+                            "us_per_step": {autotune.label(shape): round(t * 1e6, 2)
+                                            for shape, t in times.items()}}
 
     solvers = {}
     for model in ("IR", "PR"):
@@ -488,7 +488,7 @@ def run_precision_record(args):
     n = CHECK_EVERY + args.precision_steps
     for storage in ("F32", "F16"):
         for model in ("IR", "PR"):
-            shape = (256, 1)
+            shape = autotune.UNTUNED
             if not args.no_tune:
                 shape, _ = autotune.tune("D3Q27", model, storage, mask.size, steps=100, mask=mask)
             s = lbm.Solver("D3Q27", mask, model=model, storage=storage, mu_p=NU_P,
@@ -508,7 +508,7 @@ def run_precision_record(args):
             gbs = b * nfluid / t / 1e9
             out[f"{model}/{storage}"] = {
                 "kernel": f"k_step<D3Q27,{model},{STORAGE_CTYPE[storage]}>",
-                "shape": f"{shape[0]}x{shape[1]}", "launch_us": round(t * 1e6, 2),
+                "shape": autotune.label(shape), "launch_us": round(t * 1e6, 2),
                 "mlups": round(nfluid / t / 1e6, 1), "bytes_per_fluid_update": b,
                 "achieved_gbs": round(gbs, 1), "frac": round(gbs / peak, 4)}
     fl = mask == 0

@@ -361,7 +361,8 @@ void lbm_destroy(lbm_solver *s);
  * ------------------------------------------------------------------------ */
 lbm_status lbm_tuning_set(lbm_lattice lat, int32_t model, int32_t storage, int32_t size_class,
                           int32_t block);
-/* Block used for a problem of `cells` cells, and its size class. */
+/* Block set for a problem of `cells` cells (256 without an entry), and its size
+ * class. */
 lbm_status lbm_tuning_get(lbm_lattice lat, int32_t model, int32_t storage, int64_t cells,
                           int32_t *block, int32_t *size_class);
 /* Launch shape with the cells each thread steps: 1, or 2 (block 128 or 256;
@@ -374,13 +375,25 @@ lbm_status lbm_tuning_set_shape(lbm_lattice lat, int32_t model, int32_t storage,
                                 int32_t size_class, int32_t block, int32_t cells_per_thread);
 lbm_status lbm_tuning_get_shape(lbm_lattice lat, int32_t model, int32_t storage, int64_t cells,
                                 int32_t *block, int32_t *cells_per_thread, int32_t *size_class);
+/* Without an entry a solver runs what the library chooses for it: other block
+ * sizes (64 threads among them), small domains in runs held in shared memory,
+ * small FP64 steps divided over warps.  An entry turns these off, also one equal
+ * to what lbm_tuning_get reports without it, so a choice of "no entry" is kept
+ * by lbm_tuning_unset, not by setting what was read. */
+lbm_status lbm_tuning_unset(lbm_lattice lat, int32_t model, int32_t storage, int32_t size_class);
+/* 1: an entry applies to problems of `cells` cells, 0: none does. */
+lbm_status lbm_tuning_is_set(lbm_lattice lat, int32_t model, int32_t storage, int64_t cells,
+                             int32_t *set);
 lbm_status lbm_tuning_clear(void);   /* also resets the batch schedule below */
 
 /* Batch schedule (no counterpart in the paper), read by every batch (and so
  * every server) at its next lbm_batch_step:
- *   ctas_per_sm -- per (lattice, model, storage) group: 0 (default) launches
- *     one CTA per tile; n > 0 launches a persistent grid of min(tiles,
- *     n x SMs) CTAs that walk the tiles.  0..32.
+ *   ctas_per_sm -- per (lattice, model, storage) group: 0 launches one CTA
+ *     per tile; n > 0 launches a persistent grid of min(tiles, n x SMs) CTAs
+ *     that walk the tiles.  0..32.  Until it is set, groups that run as
+ *     branches share the SMs' CTAs by the bytes of their steps, a group on its
+ *     own has a CTA per tile, and lbm_tuning_get_batch reports 0;
+ *     lbm_tuning_unset_batch goes back to that.
  *   concurrency -- 1: captured graphs run the groups as parallel branches
  *     (they touch disjoint memory); 0: one after another.  Until it is set, a
  *     batch of several groups runs them as branches, and
@@ -393,6 +406,8 @@ lbm_status lbm_tuning_set_batch(lbm_lattice lat, int32_t model, int32_t storage,
                                 int32_t ctas_per_sm);
 lbm_status lbm_tuning_get_batch(lbm_lattice lat, int32_t model, int32_t storage,
                                 int32_t *ctas_per_sm);
+lbm_status lbm_tuning_unset_batch(lbm_lattice lat, int32_t model, int32_t storage);
+lbm_status lbm_tuning_batch_is_set(lbm_lattice lat, int32_t model, int32_t storage, int32_t *set);
 lbm_status lbm_tuning_set_batch_concurrency(int32_t concurrent);
 lbm_status lbm_tuning_get_batch_concurrency(int32_t *concurrent);
 /* Plain-step tile shape of the batch kernel for a (lattice, model, storage,

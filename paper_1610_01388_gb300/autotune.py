@@ -1,12 +1,14 @@
 """Autotuner for the step kernel's launch shape.
 
 For a (lattice, model, storage, size class) it builds a synthetic square duct
-with about 2**size_class cells, times every candidate shape (128, 256 or 512
-threads per block at one cell per thread; 128 or 256 at two cells per
-thread, FP32 arithmetic only) for a few hundred steps with CUDA events on
-the solver's stream (after a warm-up that also captures the CUDA graphs),
-takes the fastest, and writes it into the library's tuning table
-(lbm_tuning_set_shape).  Results are cached in a JSON file keyed by the GPU
+with about 2**size_class cells, times every candidate shape (the library's own
+choice; 128, 256 or 512 threads per block at one cell per thread; 128 or 256
+at two cells per thread, FP32 arithmetic only) for a few hundred steps with
+CUDA events on the solver's stream (after a warm-up that also captures the
+CUDA graphs), takes the fastest, and writes it into the library's tuning table
+(lbm_tuning_set_shape), which it leaves without an entry where the library's
+own choice is: an entry would turn off what no entry can hold (resident runs,
+divided FP64 steps, blocks of 64).  Results are cached in a JSON file keyed by the GPU
 name so later processes skip the measurement (``load``).  All timing goes
 through the C ABI.  The block size changes only the launch; two cells per
 thread run the same collision in packed two-wide FP32 instructions (equal to
@@ -21,8 +23,21 @@ import os
 from . import lbm
 from . import workloads as W
 
-# launch shapes (threads per block, cells per thread)
-CANDIDATES = ((128, 1), (256, 1), (512, 1), (128, 2), (256, 2))
+# launch shapes (threads per block, cells per thread); UNTUNED: no entry, the
+# library chooses
+UNTUNED = (0, 0)
+CANDIDATES = (UNTUNED, (128, 1), (256, 1), (512, 1), (128, 2), (256, 2))
+
+
+def label(shape):
+    return "untuned" if tuple(shape) == UNTUNED else f"{shape[0]}x{shape[1]}"
+
+
+def _apply(lattice, model, storage, size_class, shape):
+    if tuple(shape) == UNTUNED:
+        lbm.lbm_tuning_unset(lattice, model, storage, size_class)
+    else:
+        lbm.lbm_tuning_set_shape(lattice, model, storage, size_class, *shape)
 
 
 def _gpu_name():
@@ -54,7 +69,7 @@ def measure(lattice, model, storage, size_class, steps=300, warmup=70, mask=None
     for block, cpt in CANDIDATES:
         if cpt == 2 and storage == "F64":
             continue
-        lbm.lbm_tuning_set_shape(lattice, model, storage, size_class, block, cpt)
+        _apply(lattice, model, storage, size_class, (block, cpt))
         s = lbm.Solver(lattice, mask, model=model, storage=storage, mu_p=0.1, sigma_y=1e-6,
                        m=1e6, g=(1e-6, 0.0, 0.0), use_torch=True)
         s.step(warmup)
@@ -72,16 +87,16 @@ def measure(lattice, model, storage, size_class, steps=300, warmup=70, mask=None
 def tune(lattice, model, storage, cells, cache=None, steps=300, mask=None):
     """Tune the size class of `cells` (on `mask`, the workload's geometry,
     when given); returns (best (block, cells per thread), {(block, cells per
-    thread): seconds})."""
+    thread): seconds}), UNTUNED standing for the library's own choice."""
     _, cls = lbm.lbm_tuning_get(lattice, model, storage, cells)
     times = measure(lattice, model, storage, cls, steps=steps, mask=mask)
     best = min(times, key=times.get)
-    lbm.lbm_tuning_set_shape(lattice, model, storage, cls, *best)
+    _apply(lattice, model, storage, cls, best)
     if cache:
         data = _read(cache)
         data.setdefault(_gpu_name(), {})[f"{lattice}/{model}/{storage}/{cls}"] = {
             "block": best[0], "cells_per_thread": best[1],
-            "seconds_per_step": {f"{b}x{c}": t for (b, c), t in times.items()}}
+            "seconds_per_step": {label(shape): t for shape, t in times.items()}}
         with open(cache, "w") as fh:
             json.dump(data, fh, indent=1, sort_keys=True)
     return best, times
@@ -95,21 +110,22 @@ def _read(path):
 
 
 def load(cache):
-    """Apply cached decisions for this GPU; returns how many were applied."""
+    """Apply cached decisions for this GPU; returns how many were applied.  Those
+    taken without a look at the library's own choice are left out: it may be
+    faster now."""
     n = 0
     for key, v in _read(cache).get(_gpu_name(), {}).items():
-        if key == "batch":
+        if key == "batch" or label(UNTUNED) not in v.get("seconds_per_step", {}):
             continue
         lat, model, storage, cls = key.split("/")
-        lbm.lbm_tuning_set_shape(lat, model, storage, int(cls), int(v["block"]),
-                                 int(v.get("cells_per_thread", 1)))
+        _apply(lat, model, storage, int(cls), (int(v["block"]), int(v["cells_per_thread"])))
         n += 1
     return n
 
 
 # --- batch schedule -------------------------------------------------------------
 
-BATCH_CTAS = (0, 1, 2, 4, 8)
+BATCH_CTAS = (None, 0, 1, 2, 4, 8)   # None: not set, the library chooses
 # plain-step tile shapes (threads per CTA, cells per thread), the default first
 BATCH_TILES = ((256, 1), (128, 1), (512, 1), (128, 2), (256, 2))
 
@@ -135,36 +151,45 @@ def _group_key(lat, prm):
     return (lat, prm.get("model", "IR"), prm.get("storage", "F32"))
 
 
+def _apply_ctas(key, ctas):
+    if ctas is None:
+        lbm.lbm_tuning_unset_batch(*key)
+    else:
+        lbm.lbm_tuning_set_batch(*key, ctas)
+
+
 def tune_batch(mix, steps=160, cache=None):
-    """Coordinate search over the batch schedule on `mix`: group concurrency
-    first (with one CTA per tile), then, group by group, the CTAs per SM of a
-    persistent grid, then the plain-step tile shape (threads per CTA x cells
-    per thread) for the group's size class (floor(log2) of its domains' mean
-    cell count).  Leaves the fastest schedule set; returns it with the
+    """Coordinate search over the batch schedule on `mix`, from what the library
+    runs with nothing set ("base": concurrent groups that share the SMs): groups
+    one after another first, then, group by group, the CTAs per SM (one CTA per
+    tile, or a persistent grid), then the plain-step tile shape (threads per CTA
+    x cells per thread) for the group's size class (floor(log2) of its domains'
+    mean cell count).  Leaves the fastest schedule set, groups whose unset CTAs
+    were the fastest without an entry; returns it (CTAs None: not set) with the
     measured seconds per step of every candidate tried, and records the
     choices in the JSON file `cache` under the GPU's name and
     "lattice/model/storage/size class" keys (``load_batch`` applies them)."""
     keys = sorted({_group_key(lat, prm) for lat, _, prm in mix})
-    for lat, model, storage in keys:
-        lbm.lbm_tuning_set_batch(lat, model, storage, 0)
-    lbm.lbm_tuning_set_batch_concurrency(False)
+    for key in keys:
+        lbm.lbm_tuning_unset_batch(*key)
+    lbm.lbm_tuning_set_batch_concurrency(True)     # as unset
     tried = {"base": measure_batch(mix, steps)}
     best = tried["base"]
-    lbm.lbm_tuning_set_batch_concurrency(True)
-    tried["concurrent"] = measure_batch(mix, steps)
-    concurrent = tried["concurrent"] < best
-    best = min(best, tried["concurrent"])
+    lbm.lbm_tuning_set_batch_concurrency(False)
+    tried["serial"] = measure_batch(mix, steps)
+    concurrent = best <= tried["serial"]
+    best = min(best, tried["serial"])
     lbm.lbm_tuning_set_batch_concurrency(concurrent)
     ctas = {}
     for key in keys:
-        ctas[key] = 0
+        ctas[key] = None
         for c in BATCH_CTAS[1:]:
-            lbm.lbm_tuning_set_batch(*key, c)
+            _apply_ctas(key, c)
             t = measure_batch(mix, steps)
             tried[f"{'/'.join(key)}:{c}"] = t
             if t < best:
                 best, ctas[key] = t, c
-        lbm.lbm_tuning_set_batch(*key, ctas[key])
+        _apply_ctas(key, ctas[key])
     tiles = {}
     for key in keys:
         lat, model, storage = key
@@ -182,8 +207,12 @@ def tune_batch(mix, steps=160, cache=None):
         tiles[key] = (shape, cls)
     if cache:
         data = _read(cache)
-        ent = data.setdefault(_gpu_name(), {}).setdefault("batch", {})
+        gpu = data.setdefault(_gpu_name(), {})
+        if not gpu.get("batch", {}).get("from_unset"):
+            gpu["batch"] = {}          # left out by load_batch
+        ent = gpu["batch"]
         ent["concurrent"] = bool(concurrent)
+        ent["from_unset"] = True       # the search began at what the library chooses
         for key in keys:
             (th, cpt), cls = tiles[key]
             ent[f"{'/'.join(key)}/{cls}"] = {"ctas_per_sm": ctas[key], "threads": th,
@@ -197,15 +226,21 @@ def tune_batch(mix, steps=160, cache=None):
 
 def load_batch(cache):
     """Apply cached batch schedules for this GPU; returns how many group
-    entries were applied."""
+    entries were applied: none of a cache whose search did not begin at what
+    the library chooses with nothing set, which may be faster now."""
     ent = _read(cache).get(_gpu_name(), {}).get("batch", {})
+    if not ent.get("from_unset"):
+        return 0
     n = 0
     for key, v in ent.items():
+        if key == "from_unset":
+            continue
         if key == "concurrent":
             lbm.lbm_tuning_set_batch_concurrency(bool(v))
             continue
         lat, model, storage, cls = key.split("/")
-        lbm.lbm_tuning_set_batch(lat, model, storage, int(v["ctas_per_sm"]))
+        c = v["ctas_per_sm"]
+        _apply_ctas((lat, model, storage), None if c is None else int(c))
         lbm.lbm_tuning_set_batch_tile(lat, model, storage, int(cls), int(v["threads"]),
                                       int(v["cells_per_thread"]))
         n += 1

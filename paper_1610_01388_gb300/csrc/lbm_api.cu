@@ -734,12 +734,18 @@ void apply_tuning(lbm_solver* s) {
     s->tune_version = ver;
 }
 
-lbm_status set_shape(int lat, int32_t model, int32_t storage, int32_t cls, int32_t block,
-                     int32_t cpt) {
+lbm_status check_key(int lat, int32_t model, int32_t storage, int32_t cls) {
     if (lattice_q(lat) == 0) return fail(LBM_EINVAL, "unknown lattice %d", lat);
     if (model != LBM_MODEL_PR && model != LBM_MODEL_IR) return fail(LBM_EINVAL, "unknown model %d", model);
     if (storage_bytes(storage) == 0) return fail(LBM_EINVAL, "unknown storage %d", storage);
     if (cls < 0 || cls > 62) return fail(LBM_EINVAL, "size class must be in 0..62");
+    return LBM_OK;
+}
+
+lbm_status set_shape(int lat, int32_t model, int32_t storage, int32_t cls, int32_t block,
+                     int32_t cpt) {
+    const lbm_status v = check_key(lat, model, storage, cls);
+    if (v != LBM_OK) return v;
     if (block != 128 && block != 256 && block != 512) return fail(LBM_EINVAL, "block must be 128, 256 or 512");
     if (cpt != 1 && cpt != 2) return fail(LBM_EINVAL, "cells per thread must be 1 or 2");
     if (cpt == 2 && block == 512) return fail(LBM_EINVAL, "two cells per thread need block 128 or 256");
@@ -778,6 +784,26 @@ lbm_status lbm_tuning_get_shape(lbm_lattice lat, int32_t model, int32_t storage,
     if (block) *block = sh.block;
     if (cells_per_thread) *cells_per_thread = sh.cpt;
     if (size_class_) *size_class_ = size_class(cells);
+    return LBM_OK;
+}
+
+lbm_status lbm_tuning_unset(lbm_lattice lat, int32_t model, int32_t storage, int32_t size_class_) {
+    const lbm_status v = check_key(lat, model, storage, size_class_);
+    if (v != LBM_OK) return v;
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        g_tune.erase(tune_key(lat, model, storage, size_class_));
+    }
+    g_tune_version.fetch_add(1);
+    return LBM_OK;
+}
+
+lbm_status lbm_tuning_is_set(lbm_lattice lat, int32_t model, int32_t storage, int64_t cells,
+                             int32_t* set) {
+    if (cells < 1 || !set) return fail(LBM_EINVAL, "bad cell count, or set is NULL");
+    const lbm_status v = check_key(lat, model, storage, size_class(cells));
+    if (v != LBM_OK) return v;
+    *set = tune_lookup(lat, model, storage, cells).set;
     return LBM_OK;
 }
 

@@ -754,6 +754,24 @@ lbm_status lbm_tuning_get_batch_tile(lbm_lattice lat, int32_t model, int32_t sto
     return LBM_OK;
 }
 
+lbm_status lbm_tuning_unset_batch(lbm_lattice lat, int32_t model, int32_t storage) {
+    if (lattice_q(lat) == 0) return fail(LBM_EINVAL, "unknown lattice %d", lat);
+    if (model != LBM_MODEL_PR && model != LBM_MODEL_IR) return fail(LBM_EINVAL, "unknown model %d", model);
+    if (storage_bytes(storage) == 0) return fail(LBM_EINVAL, "unknown storage %d", storage);
+    {
+        std::lock_guard<std::mutex> lk(g_sched_mu);
+        g_sched_ctas.erase(sched_key(lat, model, storage));
+    }
+    g_sched_version.fetch_add(1);
+    return LBM_OK;
+}
+
+lbm_status lbm_tuning_batch_is_set(lbm_lattice lat, int32_t model, int32_t storage, int32_t* set) {
+    if (!set) return fail(LBM_EINVAL, "set is NULL");
+    *set = sched_ctas(lat, model, storage, -1) >= 0;
+    return LBM_OK;
+}
+
 lbm_status lbm_tuning_set_batch_concurrency(int32_t concurrent) {
     if (concurrent != 0 && concurrent != 1) return fail(LBM_EINVAL, "concurrent must be 0 or 1");
     g_sched_concurrent.store(concurrent);

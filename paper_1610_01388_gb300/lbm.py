@@ -49,7 +49,8 @@ EXPORTED = ["lbm_params_default", "lbm_lattice_info", "lbm_workspace_bytes", "lb
             "lbm_tuning_set_batch_tile", "lbm_tuning_get_batch_tile",
             "lbm_halo_bytes", "lbm_halo_pack", "lbm_halo_unpack", "lbm_set_hash_offset",
             "lbm_check_sums", "lbm_step_cells", "lbm_step_commit",
-            "lbm_workspace_bytes_for_mask"]
+            "lbm_workspace_bytes_for_mask", "lbm_tuning_unset", "lbm_tuning_is_set",
+            "lbm_tuning_unset_batch", "lbm_tuning_batch_is_set"]
 LBM_REQ_QUEUED, LBM_REQ_RUNNING, LBM_REQ_CONVERGED, LBM_REQ_CAPPED, LBM_REQ_FAILED = range(5)
 LBM_STEADY_FLOW, LBM_STEADY_RESIDUAL = 0, 1
 
@@ -153,6 +154,10 @@ def library():
             "lbm_tuning_set": [i32, i32, i32, i32, i32],
             "lbm_tuning_get": [i32, i32, i32, i64, P(i32), P(i32)],
             "lbm_tuning_clear": [],
+            "lbm_tuning_unset": [i32, i32, i32, i32],
+            "lbm_tuning_is_set": [i32, i32, i32, i64, P(i32)],
+            "lbm_tuning_unset_batch": [i32, i32, i32],
+            "lbm_tuning_batch_is_set": [i32, i32, i32, P(i32)],
             "lbm_tuning_set_shape": [i32, i32, i32, i32, i32, i32],
             "lbm_tuning_get_shape": [i32, i32, i32, i64, P(i32), P(i32), P(i32)],
             "lbm_set_wait_limit": [ctypes.c_double],
@@ -369,11 +374,24 @@ def lbm_tuning_set(lat, model, storage, size_class, block):
 
 
 def lbm_tuning_get(lat, model, storage, cells):
-    """(block, size class) the library uses for a problem of `cells` cells."""
+    """(block, size class) set for a problem of `cells` cells; without an entry
+    (lbm_tuning_is_set) 256, while the library chooses for itself."""
     b, c = ctypes.c_int32(), ctypes.c_int32()
     _check(library().lbm_tuning_get(_lat(lat), _mdl(model), _sto(storage), int(cells),
                                     ctypes.byref(b), ctypes.byref(c)))
     return b.value, c.value
+
+
+def lbm_tuning_unset(lat, model, storage, size_class):
+    """Takes an entry back: the library chooses for itself again."""
+    _check(library().lbm_tuning_unset(_lat(lat), _mdl(model), _sto(storage), int(size_class)))
+
+
+def lbm_tuning_is_set(lat, model, storage, cells) -> bool:
+    v = ctypes.c_int32()
+    _check(library().lbm_tuning_is_set(_lat(lat), _mdl(model), _sto(storage), int(cells),
+                                       ctypes.byref(v)))
+    return bool(v.value)
 
 
 def lbm_tuning_clear():
@@ -386,7 +404,8 @@ def lbm_tuning_set_shape(lat, model, storage, size_class, block, cells_per_threa
 
 
 def lbm_tuning_get_shape(lat, model, storage, cells):
-    """(block, cells per thread, size class) the library uses for `cells` cells."""
+    """(block, cells per thread, size class) set for `cells` cells; without an
+    entry (lbm_tuning_is_set) 256 x 1, while the library chooses for itself."""
     b, c, k = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
     _check(library().lbm_tuning_get_shape(_lat(lat), _mdl(model), _sto(storage), int(cells),
                                           ctypes.byref(b), ctypes.byref(c), ctypes.byref(k)))
@@ -398,7 +417,20 @@ def lbm_tuning_set_batch(lat, model, storage, ctas_per_sm):
                                           int(ctas_per_sm)))
 
 
+def lbm_tuning_unset_batch(lat, model, storage):
+    _check(library().lbm_tuning_unset_batch(_lat(lat), _mdl(model), _sto(storage)))
+
+
+def lbm_tuning_batch_is_set(lat, model, storage) -> bool:
+    v = ctypes.c_int32()
+    _check(library().lbm_tuning_batch_is_set(_lat(lat), _mdl(model), _sto(storage),
+                                             ctypes.byref(v)))
+    return bool(v.value)
+
+
 def lbm_tuning_get_batch(lat, model, storage) -> int:
+    """CTAs per SM set for a group; 0 also where none is set
+    (lbm_tuning_batch_is_set) and concurrent groups share the SMs."""
     v = ctypes.c_int32()
     _check(library().lbm_tuning_get_batch(_lat(lat), _mdl(model), _sto(storage),
                                           ctypes.byref(v)))
@@ -425,6 +457,7 @@ def lbm_tuning_set_batch_concurrency(on):
 
 
 def lbm_tuning_get_batch_concurrency() -> bool:
+    """Whether concurrent groups are set (unset, they run concurrently too)."""
     v = ctypes.c_int32()
     _check(library().lbm_tuning_get_batch_concurrency(ctypes.byref(v)))
     return bool(v.value)
