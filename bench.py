@@ -105,26 +105,26 @@ def workload_mask(nx=None):
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
-# step kernels, from ncu captures of this script (the commands are in the
-# profiles/ summaries).  NCU_TRAFFIC: the 256x128x128 D3Q27 duct, keyed by
-# storage, model, block size and cells per thread.  NCU_TRAFFIC_POROUS: the
-# porous box of the porous record (256^3, D3Q19, 256 threads), keyed by
-# layout, storage and model.  Both are valid only
+# step kernels, from ncu captures (the commands are in the profiles/ summaries).
+# NCU_TRAFFIC: the 256x128x128 D3Q27 duct, keyed by
+# storage, model, block size and cells per thread (0, 0: the library's own
+# choice).  NCU_TRAFFIC_POROUS: the porous box of the porous record (256^3,
+# D3Q19, untuned), keyed by layout, storage and model.  Both are valid only
 # for the device-code sources they were captured with (KERNEL_FINGERPRINT)
 # and are reported as null once any of those sources changes.
 NCU_TRAFFIC_POROUS = {
-    ('compact', 'F16', 'IR'): 1017978014, ('compact', 'F16', 'PR'): 1113269616,
-    ('compact', 'F32', 'IR'): 1903769109, ('compact', 'F32', 'PR'): 1998954998,
-    ('dense', 'F16', 'IR'): 1249633474, ('dense', 'F16', 'PR'): 1377774772,
-    ('dense', 'F32', 'IR'): 2433578501, ('dense', 'F32', 'PR'): 2559411298,
+    ('compact', 'F16', 'IR'): 1017785754, ('compact', 'F16', 'PR'): 1114134118,
+    ('compact', 'F32', 'IR'): 1903204915, ('compact', 'F32', 'PR'): 1997050573,
+    ('dense', 'F16', 'IR'): 1249303245, ('dense', 'F16', 'PR'): 1377811968,
+    ('dense', 'F32', 'IR'): 2432536986, ('dense', 'F32', 'PR'): 2561536717,
 }
 NCU_TRAFFIC = {
-    ('F16', 'IR', 128, 1): 420014114, ('F16', 'IR', 128, 2): 419242511, ('F16', 'IR', 256, 1): 419807719, ('F16', 'IR', 256, 2): 420148489, ('F16', 'IR', 512, 1): 420246713,
-    ('F16', 'PR', 128, 1): 451687740, ('F16', 'PR', 128, 2): 450993049, ('F16', 'PR', 256, 1): 451128599, ('F16', 'PR', 256, 2): 451178877, ('F16', 'PR', 512, 1): 451255470,
-    ('F32', 'IR', 128, 1): 855939396, ('F32', 'IR', 128, 2): 855419924, ('F32', 'IR', 256, 1): 855652990, ('F32', 'IR', 256, 2): 857036609, ('F32', 'IR', 512, 1): 857513376,
-    ('F32', 'PR', 128, 1): 889867913, ('F32', 'PR', 128, 2): 889934811, ('F32', 'PR', 256, 1): 889658765, ('F32', 'PR', 256, 2): 890827582, ('F32', 'PR', 512, 1): 890181304,
+    ('F16', 'IR', 0, 0): 420181760, ('F16', 'IR', 128, 1): 420210893, ('F16', 'IR', 256, 1): 419813120, ('F16', 'IR', 512, 1): 420370381, ('F16', 'IR', 128, 2): 419888538, ('F16', 'IR', 256, 2): 420638054,
+    ('F16', 'PR', 0, 0): 451218381, ('F16', 'PR', 128, 1): 451184435, ('F16', 'PR', 256, 1): 450876262, ('F16', 'PR', 512, 1): 450988032, ('F16', 'PR', 128, 2): 450668339, ('F16', 'PR', 256, 2): 450829773,
+    ('F32', 'IR', 0, 0): 855479962, ('F32', 'IR', 128, 1): 855868365, ('F32', 'IR', 256, 1): 855582054, ('F32', 'IR', 512, 1): 857283738, ('F32', 'IR', 128, 2): 855312691, ('F32', 'IR', 256, 2): 856884429,
+    ('F32', 'PR', 0, 0): 889337958, ('F32', 'PR', 128, 1): 891625165, ('F32', 'PR', 256, 1): 889154765, ('F32', 'PR', 512, 1): 889708390, ('F32', 'PR', 128, 2): 889457766, ('F32', 'PR', 256, 2): 890243686,
 }
-KERNEL_FINGERPRINT = "49211dcd9ff1d162"
+KERNEL_FINGERPRINT = "86adaf42fbd961e7"
 KERNEL_SOURCES = ("kernels.cuh", "lattice.cuh", "lbm_internal.h", "fastdiv.h", "kern_d3q27.cu",
                   "kern_d3q19.cu")
 
@@ -354,8 +354,8 @@ def run_ours(args):
             "frac": round(per[dom]["frac"], 4),
             "bytes_per_fluid_update": per[dom]["bytes_per_update"],
             "fluid_cells_per_launch": nfluid,
-            "traffic": ncu_traffic(STORAGE, dom, tuned.get(dom, {}).get("block", 256),
-                                   tuned.get(dom, {}).get("cells_per_thread", 1), args.traffic),
+            "traffic": ncu_traffic(STORAGE, dom, tuned.get(dom, {}).get("block", 0),
+                                   tuned.get(dom, {}).get("cells_per_thread", 0), args.traffic),
             "per_model": {k: {kk: round(vv, 4) if isinstance(vv, float) else vv
                               for kk, vv in v.items()} for k, v in per.items()}}
     for s in solvers.values():

@@ -1326,20 +1326,21 @@ __device__ __forceinline__ void block_sum_store(V (&v)[kNumStats], double* __res
 }
 
 // ---------------------------------------------------------------------------
-// Overlapped launches.  The step kernels are launched with programmatic stream
-// serialisation: a kernel's blocks may start while the previous step drains,
-// read what no step writes (link words, maps, coefficients), and wait for the
+// Overlapped launches.  Step kernels are launched, where it pays (launch_step),
+// with programmatic stream serialisation: a kernel's blocks may start while the
+// previous step drains, read what no step writes (link words, maps,
+// coefficients), and wait for the
 // previous step's stores before they touch anything else.  step_begin() is
 // that wait; `n`, which every later address is formed from, passes through it
 // so that no load can move up past it.  Only then the next launch is let in,
 // so a kernel never overlaps more than the one before it, and the lines it
 // reads (the ones that kernel writes) cannot sit stale in L1: the last kernel
 // that read them has ended before this kernel's blocks are launched.  Every
-// block calls it, also one with nothing to do.  A small step is mostly launch
-// and ramp (D2Q9 FP32 PR, 128 x 66: 2.27 -> 1.90 us a step; D3Q15 FP32 PR, 45 x
-// 47 x 43: 4.16 -> 3.75), a large one gains its last, partly filled wave (D3Q27
-// FP32 duct 256 x 128 x 128: IR 138 -> 136, PR 149 -> 147; FP16 PR 512 x 192 x
-// 192: 540 -> 493 us).
+// block calls it, also one with nothing to do (but for the compact 16-bit steps,
+// which are never overlapped).  A small step is mostly launch and ramp (us a step,
+// plain -> overlapped: D2Q9 FP32 IR, 128 x 128: 2.1 -> 1.6; D3Q15 FP32 PR, 45 x 47 x 43:
+// 3.6 -> 3.1), a large one gains its last, partly filled wave (D3Q27 duct 256 x 128 x
+// 128: FP32 PR 138.8 -> 138.5, FP16 PR 111.6 -> 111.2).
 __device__ __forceinline__ void step_begin(int& n) {
     asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" : "+r"(n) : : "memory");
 }

@@ -145,8 +145,8 @@ int sched_ctas(int lat, int model, int storage, int unset = 0) {
 // Resident CTAs per SM that concurrent groups without a schedule entry share
 // out by the bytes of their steps, at least one each.  With one CTA per tile a
 // large group's blocks, and those of its next step that already wait for it,
-// keep the other groups off the SMs (48 domains of the serving mix, us per step:
-// 52 with a CTA per tile, 42 shared out, with pair-form 16-bit groups).
+// keep the other groups off the SMs (48 domains of the serving mix, us per step
+// at 4 / 6 / 8 / 12 / 16 and with a CTA per tile: 52 / 52 / 44 / 46 / 46 / 55).
 constexpr int kSharedCtas = 8;
 
 // bytes a group's plain step moves at least
@@ -272,7 +272,7 @@ lbm_status rebuild(lbm_batch* b) {
     b->sched_version = g_sched_version.load();
     // Concurrent unless it was switched off: most groups of a mix are too small
     // to fill the GPU (48 domains of the serving mix in 10 groups, us per step:
-    // 90 one after another, 61 as branches).
+    // 83 one after another, 55 as branches).
     b->concurrent = g_sched_concurrent.load() != 0;
     b->rows = 0;
     for (const auto& kv : b->doms) b->rows = std::max(b->rows, kv.second.slot + 1);
